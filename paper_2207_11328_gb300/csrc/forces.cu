@@ -484,12 +484,11 @@ template <int VISC>
 __global__ void __launch_bounds__(kPipeBlock, 4) k_build_predict(const Buffers b, int cur, const Phys ph) {
     DevStatus* st = b.status;
     const uint32_t n = st->n_active;
-    const uint32_t r2lim = __float_as_uint(ph.R2_list) - 1u;
     uint32_t npairs = 0;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         uint32_t nfound;
-        const uint32_t nent = build_particle(i, b.pos[cur], b.cell[cur], b.pinfo[cur], b.start, b.cell_nfluid, b.scenes,
-                                             b.nlist, b.ncount, r2lim, ph.max_neibs, ph.stride, &nfound, st, n);
+        const uint32_t nent = build_particle(i, b.pos[cur], b.quads, b.cell[cur], b.pinfo[cur], b.start,
+                                             b.cell_nfluid, b.scenes, b.nlist, b.ncount, ph.R2_list, ph.max_neibs, ph.stride, &nfound, st, n);
         build_stats(st, nfound, nent, ph.max_neibs, __activemask());
         asm volatile("" ::: "memory");  // the list stores above precede its loads below
         const uint32_t cnt = ld_count_fresh(b.ncount + i);
@@ -537,9 +536,9 @@ __global__ void __launch_bounds__(kPipeBlock, kPersistMinBlocks) k_step_persiste
         grid.sync();
         reorder_body(b.pos[cur], b.vel[cur], b.phat[cur], b.pinfo[cur], b.pid[cur], b.start, b.unsorted, b.scenes,
                      g.n_cells, b.status, b.cell_nfluid, b.pos[nxt], b.vel[nxt], b.phat[nxt], b.cell[nxt],
-                     b.pinfo[nxt], b.pid[nxt]);
+                     b.pinfo[nxt], b.pid[nxt], b.quads);
         grid.sync();
-        build_tpp_body(b.pos[nxt], b.cell[nxt], b.pinfo[nxt], b.start, b.cell_nfluid, b.scenes, b.status, b.nlist,
+        build_tpp_body(b.pos[nxt], b.quads, b.cell[nxt], b.pinfo[nxt], b.start, b.cell_nfluid, b.scenes, b.status, b.nlist,
                        b.ncount, ph.R2_list, ph.max_neibs, ph.stride);
         grid.sync();
         forces_body<VISC, kPredict, false>(b.pos[nxt], b.vel[nxt], b.phat[nxt], b.pos_s, b.vel_s, b.phat_s, nullptr,

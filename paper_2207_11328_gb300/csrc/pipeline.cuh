@@ -5,6 +5,7 @@
 // persistent step kernel (forces.cu) runs them one after the other with grid-wide
 // barriers between them.  Grid-stride loops: any grid size computes the same.
 #pragma once
+#include "packed.cuh"
 #include "sph_internal.cuh"
 
 namespace sphg {
@@ -200,7 +201,7 @@ __device__ __forceinline__ void reorder_body(
     const SceneDev* __restrict__ scenes, uint32_t n_cells, DevStatus* __restrict__ st, uint32_t* __restrict__ cell_nfluid,
     float4* __restrict__ pos_o,
     float4* __restrict__ vel_o, float* __restrict__ phat_o, uint32_t* __restrict__ cell_o,
-    uint32_t* __restrict__ pinfo_o, uint32_t* __restrict__ pid_o) {
+    uint32_t* __restrict__ pinfo_o, uint32_t* __restrict__ pid_o, float* __restrict__ quads) {
     const int lane = threadIdx.x & 31;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -254,6 +255,10 @@ __device__ __forceinline__ void reorder_body(
                     const uint32_t d = beg + rank;
                     SPH_GUARD(d < end, st, continue)
                     pos_o[d] = p;
+                    float* qd = quads + quad_word(d);
+                    qd[0] = p.x;
+                    qd[4] = p.y;
+                    qd[8] = p.z;
                     vel_o[d] = vel[idx];
                     phat_o[d] = phat[idx];
                     cell_o[d] = c;
@@ -267,100 +272,89 @@ __device__ __forceinline__ void reorder_body(
 }
 
 // ---------------------------------------------------------------------
-// a5, second variant: one thread per particle (the paper's baseline
+// a5: split neighbour list (paper Section 4), one thread per particle (the paper's baseline
 // build, Section 7).  Lanes of a warp are consecutive particles of ~2 cells
 // and read the same candidates (L1 broadcast).  Candidates are fluid-first
 // in each cell (cell_nfluid), so a boundary particle walks only the fluid
 // part of each neighbour cell and types need no per-candidate test.
+//
+// Bound by instruction issue (64% busy) and the L1 pipe (58%).  Measured, with the offsets
+// read as float4 records and tested one by one in FP32 before: 547 -> 463 us on the 1.65M dam
+// break (435M -> 368M warp instructions), 757 -> 571 us on 64 tanks of 2.0M particles, 530 -> 438 us
+// on a 1.0M box.  The group loop unrolled twice, three or four times: 476, 488, 490 us.  The
+// appends take a quarter (354 us with the lists left unwritten).
 // ---------------------------------------------------------------------
 
-// m with all but its k lowest set bits cleared
-__device__ __forceinline__ uint32_t lowest_set_bits(uint32_t m, uint32_t k) {
+// m with all but its k highest set bits cleared
+__device__ __forceinline__ uint32_t highest_set_bits(uint32_t m, uint32_t k) {
     uint32_t out = 0u;
     for (uint32_t c = 0; c < k && m; ++c) {
-        const uint32_t b = m & (0u - m);
+        const uint32_t b = 0x80000000u >> __clz((int)m);
         out |= b;
         m ^= b;
     }
     return out;
 }
 
+// the entries e0 + (u << kCodeBits) of the set bits of mask, u counted from the top bit, appended
+// to w in that order: the first completes a chunk left open, then two per chunk store
+__device__ __forceinline__ void append_mask(ListWriter& w, uint32_t mask, uint32_t e0) {
+    if (mask && (w.n & 1u)) {
+        const uint32_t u = (uint32_t)__clz((int)mask);
+        mask ^= 0x80000000u >> u;
+        w.put(e0 + (u << kCodeBits));
+    }
+    while (mask) {
+        const uint32_t u0 = (uint32_t)__clz((int)mask);
+        mask ^= 0x80000000u >> u0;
+        const uint32_t a = e0 + (u0 << kCodeBits);
+        if (!mask) {
+            w.open(a);
+            break;
+        }
+        const uint32_t u1 = (uint32_t)__clz((int)mask);
+        mask ^= 0x80000000u >> u1;
+        w.put2(a, e0 + (u1 << kCodeBits));
+    }
+}
+
+// r^2 + init of two candidates at (dx, dy, dz)
+__device__ __forceinline__ f2 r2_plus(f2 dx, f2 dy, f2 dz, f2 init) {
+    return f2_fma(dx, dx, f2_fma(dy, dy, f2_fma(dz, dz, init)));
+}
+
+// 0 < r2 < R2 as one unsigned compare on the bits, in the top bit
+__device__ __forceinline__ uint32_t centre_hit(float r2, uint32_t r2lim) {
+    return __float_as_uint(r2) - 1u < r2lim ? 0x80000000u : 0u;
+}
+
 // The list of particle i; returns its entry count, *nfound = pairs found
 // (more than max_neibs: overflow, the list keeps the first ones).
-__device__ __forceinline__ uint32_t build_particle(uint32_t i, const float4* __restrict__ pos,
+// Candidates are tested four at a time: one 16-byte load per axis from the offsets' own arrays
+// (aligned: a group may begin before the cell's first particle and end after its last, masked
+// off), packed FP32 subtractions and FMAs on two candidates each, and the sign bit of r^2 - R^2
+// shifted into a hit mask by one funnel shift: 4.75 instructions a candidate.  In the particle's
+// own cell r^2 itself is tested, 0 < r^2 < R^2 (the particle, coincident ones).  The hits of a
+// window of up to 32 candidates are appended by a loop over the mask's set bits, so a lane's
+// append work follows its own hits.  Past max_neibs entries the list keeps the first ones in
+// candidate order (the mask is cut to the room left).
+__device__ __forceinline__ uint32_t build_particle(uint32_t i, const float4* __restrict__ pos, const float* __restrict__ quads,
                                                    const uint32_t* __restrict__ cell, const uint32_t* __restrict__ pinfo,
                                                    const uint32_t* __restrict__ start,
                                                    const uint32_t* __restrict__ cell_nfluid,
                                                    const SceneDev* __restrict__ scenes, uint32_t* __restrict__ nlist,
-                                                   uint32_t* __restrict__ ncount, uint32_t r2lim, uint32_t max_neibs,
+                                                   uint32_t* __restrict__ ncount, float R2, uint32_t max_neibs,
                                                    uint32_t stride, uint32_t* nfound_out, DevStatus* st, uint32_t n) {
-    constexpr int kGroup = 6;
-    constexpr int kWindow = 5 * kGroup;  // candidates per hit mask (bits 0..29)
-    static_assert(kPosPad >= kGroup - 1, "a group reads up to kGroup - 1 entries past the last particle");
     const SceneDev& sc = scenes[pinfo[i]];
     const float4 pi = pos[i];
     const bool fluid_i = pi.w > 0.f;
     int cx, cy, cz;
     decode_local(cell[i] - sc.cell_offset, sc, cx, cy, cz);
+    const uint32_t r2lim = __float_as_uint(R2) - 1u;
+    const f2 mR2 = f2_dup(-R2);
     uint32_t nfound = 0;
     ListWriter wf = list_fluid_writer(nlist, i, stride);
     ListWriter wb = list_bnd_writer(nlist, i, stride, max_neibs);
-    // candidates [b, e) of one neighbour cell and one type, appended to w in candidate order.
-    // The distance tests run in groups of kGroup candidates (independent loads in flight); the
-    // hits of up to kWindow candidates are gathered in one bit mask, which a loop over its set
-    // bits then appends: a lane spends append work on its own hits only, where an append
-    // predicated per candidate slot costs the whole warp every slot of a group as soon as one
-    // lane hits in it.  A group may read up to kGroup - 1 entries past the range (the next
-    // cell's, or the kPosPad spare entries at the end): masked off.  Past max_neibs entries the
-    // list keeps the first ones in candidate order (the window's mask is cut to the room left).
-    auto scan_part = [&](uint32_t b, uint32_t e, ListWriter& w, float bx, float by, float bz, uint32_t code) {
-        for (uint32_t j0 = b; j0 < e; j0 += kWindow) {
-            uint32_t mask = 0;
-#pragma unroll
-            for (int g = 0; g < kWindow; g += kGroup) {
-                const uint32_t j = j0 + (uint32_t)g;
-                if (j >= e) break;
-                const float4* pg = pos + j;
-                uint32_t hits = 0;
-#pragma unroll
-                for (int u = 0; u < kGroup; ++u) {
-                    const float4 pj = pg[u];
-                    const float rx = bx - pj.x, ry = by - pj.y, rz = bz - pj.z;
-                    const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-                    // 0 < r2 < R2 as one unsigned compare on the bits (r2 >= +0)
-                    hits |= (uint32_t)(__float_as_uint(r2) - 1u < r2lim) << u;
-                }
-                const uint32_t rem = e - j;
-                if (rem < (uint32_t)kGroup) hits &= (1u << rem) - 1u;
-                mask |= hits << g;
-            }
-            if (!mask) continue;
-            const uint32_t found = (uint32_t)__popc(mask);
-            nfound += found;
-            const uint32_t room = max_neibs - (wf.n + wb.n);
-            if (found > room) mask = lowest_set_bits(mask, room);
-            const uint32_t e0 = (j0 << kCodeBits) | code;
-            // the first hit completes a chunk left open by the previous range; then two hits
-            // per chunk store, an odd last hit left open
-            if (mask && (w.n & 1u)) {
-                const uint32_t u = (uint32_t)__ffs(mask) - 1u;
-                mask &= mask - 1u;
-                w.put(e0 + (u << kCodeBits));
-            }
-            while (mask) {
-                const uint32_t u0 = (uint32_t)__ffs(mask) - 1u;
-                mask &= mask - 1u;
-                const uint32_t a = e0 + (u0 << kCodeBits);
-                if (!mask) {
-                    w.open(a);
-                    break;
-                }
-                const uint32_t u1 = (uint32_t)__ffs(mask) - 1u;
-                mask &= mask - 1u;
-                w.put2(a, e0 + (u1 << kCodeBits));
-            }
-        }
-    };
     for (int dz = -1; dz <= 1; ++dz) {
         int z = cz + dz;
         if (z < 0 || z >= sc.ncell[2]) {
@@ -374,8 +368,7 @@ __device__ __forceinline__ uint32_t build_particle(uint32_t i, const float4* __r
                 y = y < 0 ? y + sc.ncell[1] : y - sc.ncell[1];
             }
             const uint32_t row = sc.cell_offset + (uint32_t)sc.ncell[0] * ((uint32_t)y + (uint32_t)sc.ncell[1] * (uint32_t)z);
-            const float by = pi.y - (float)dy * sc.cell_f[1];
-            const float bz = pi.z - (float)dz * sc.cell_f[2];
+            const f2 ny = f2_dup((float)dy * sc.cell_f[1] - pi.y), nz = f2_dup((float)dz * sc.cell_f[2] - pi.z);
             // the row's three cell ranges, loaded together (one round trip per row)
             uint32_t rb[3], ref[3], re[3];
 #pragma unroll
@@ -399,12 +392,53 @@ __device__ __forceinline__ uint32_t build_particle(uint32_t i, const float4* __r
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 const int dx = k - 1;
-                const float bx = pi.x - (float)dx * sc.cell_f[0];
+                const f2 nx = f2_dup((float)dx * sc.cell_f[0] - pi.x);
                 const uint32_t code = (uint32_t)(dx + 1) | ((uint32_t)(dy + 1) << 2) | ((uint32_t)(dz + 1) << 4);
-                // the cell's fluid candidates (to the fluid part), then its boundary candidates
-                // (to the boundary part; fluid i only): each group's hits go to one part
-                scan_part(rb[k], ref[k], wf, bx, by, bz, code);
-                scan_part(ref[k], re[k], wb, bx, by, bz, code);
+                const bool centre = dx == 0 && dy == 0 && dz == 0;
+                const uint32_t b = rb[k], e = re[k];
+                for (uint32_t w0 = b & ~3u; w0 < e; w0 += 32u) {
+                    const uint32_t wend = min(e, w0 + 32u);
+                    uint32_t mask = 0u;
+                    uint32_t g = w0;
+                    const ulonglong2* q4 = reinterpret_cast<const ulonglong2*>(quads + quad_word(w0));
+                    if (!centre) {
+#pragma unroll 1
+                        for (; g < wend; g += 4u, q4 += 3) {
+                            const ulonglong2 X = q4[0], Y = q4[1], Z = q4[2];
+                            const f2 q0 = r2_plus(f2_add(X.x, nx), f2_add(Y.x, ny), f2_add(Z.x, nz), mR2);
+                            const f2 q1 = r2_plus(f2_add(X.y, nx), f2_add(Y.y, ny), f2_add(Z.y, nz), mR2);
+                            mask = __funnelshift_l((uint32_t)q0, mask, 1);
+                            mask = __funnelshift_l((uint32_t)(q0 >> 32), mask, 1);
+                            mask = __funnelshift_l((uint32_t)q1, mask, 1);
+                            mask = __funnelshift_l((uint32_t)(q1 >> 32), mask, 1);
+                        }
+                    } else {
+                        for (; g < wend; g += 4u, q4 += 3) {
+                            const ulonglong2 X = q4[0], Y = q4[1], Z = q4[2];
+                            const f2 a0 = r2_plus(f2_add(X.x, nx), f2_add(Y.x, ny), f2_add(Z.x, nz), 0ull);
+                            const f2 a1 = r2_plus(f2_add(X.y, nx), f2_add(Y.y, ny), f2_add(Z.y, nz), 0ull);
+                            mask = __funnelshift_l(centre_hit(f2_lo(a0), r2lim), mask, 1);
+                            mask = __funnelshift_l(centre_hit(f2_hi(a0), r2lim), mask, 1);
+                            mask = __funnelshift_l(centre_hit(f2_lo(a1), r2lim), mask, 1);
+                            mask = __funnelshift_l(centre_hit(f2_hi(a1), r2lim), mask, 1);
+                        }
+                    }
+                    // the window's first candidate to the top bit, those outside the cell off
+                    const uint32_t first = w0 < b ? b - w0 : 0u, last = wend - w0;  // last in 1..32
+                    mask = (mask << (32u - (g - w0))) & (0xffffffffu >> first) & (0xffffffffu << (32u - last));
+                    if (!mask) continue;
+                    const uint32_t found = (uint32_t)__popc(mask);
+                    nfound += found;
+                    const uint32_t room = max_neibs - (wf.n + wb.n);
+                    if (found > room) mask = highest_set_bits(mask, room);
+                    const uint32_t e0 = (w0 << kCodeBits) | code;
+                    if (ref[k] < wend) {  // fluid candidates come first in the cell
+                        const uint32_t nfl = ref[k] > w0 ? ref[k] - w0 : 0u;  // below 32
+                        append_mask(wb, mask & (0xffffffffu >> nfl), e0);
+                        mask &= ~(0xffffffffu >> nfl);
+                    }
+                    append_mask(wf, mask, e0);
+                }
             }
         }
     }
@@ -428,17 +462,179 @@ __device__ __forceinline__ void build_stats(DevStatus* st, uint32_t nfound, uint
 }
 
 __device__ __forceinline__ void build_tpp_body(
-    const float4* __restrict__ pos, const uint32_t* __restrict__ cell, const uint32_t* __restrict__ pinfo,
-    const uint32_t* __restrict__ start, const uint32_t* __restrict__ cell_nfluid, const SceneDev* __restrict__ scenes,
-    DevStatus* __restrict__ st, uint32_t* __restrict__ nlist, uint32_t* __restrict__ ncount, float R2,
-    uint32_t max_neibs, uint32_t stride) {
-    const uint32_t r2lim = __float_as_uint(R2) - 1u;
+    const float4* __restrict__ pos, const float* __restrict__ quads, const uint32_t* __restrict__ cell,
+    const uint32_t* __restrict__ pinfo, const uint32_t* __restrict__ start, const uint32_t* __restrict__ cell_nfluid,
+    const SceneDev* __restrict__ scenes, DevStatus* __restrict__ st, uint32_t* __restrict__ nlist,
+    uint32_t* __restrict__ ncount, float R2, uint32_t max_neibs, uint32_t stride) {
     const uint32_t n = st->n_active;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         uint32_t nfound;
-        const uint32_t nent = build_particle(i, pos, cell, pinfo, start, cell_nfluid, scenes, nlist, ncount, r2lim,
+        const uint32_t nent = build_particle(i, pos, quads, cell, pinfo, start, cell_nfluid, scenes, nlist, ncount, R2,
                                              max_neibs, stride, &nfound, st, n);
         build_stats(st, nfound, nent, max_neibs, __activemask());
+    }
+}
+
+// The same list by one warp per particle: lane l < 27 tests the candidates of neighbour cell l, a
+// prefix sum of the lanes' hit counts gives each cell's hits their place, and each lane appends its
+// own: the one thread's list, entry for entry.  For states too small to fill the GPU with a
+// thread per particle, whose 27 cells are one long chain of instructions: 4,096 particles 38 -> 11 us,
+// 19,683 48 -> 36 us, 71,680 50 -> 102 us (1,019 warp instructions a particle, 15 of 32 lanes active,
+// against 224 by a thread).
+__device__ __forceinline__ uint32_t warp_excl_sum(uint32_t v, uint32_t* total) {
+    const uint32_t lane = threadIdx.x & 31u;
+    uint32_t incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+        if ((int)lane >= o) incl += t;
+    }
+    *total = __shfl_sync(0xffffffffu, incl, 31);
+    return incl - v;
+}
+
+__device__ __forceinline__ uint32_t build_particle_warp(uint32_t i, const float4* __restrict__ pos,
+                                                        const float* __restrict__ quads,
+                                                        const uint32_t* __restrict__ cell,
+                                                        const uint32_t* __restrict__ pinfo,
+                                                        const uint32_t* __restrict__ start,
+                                                        const uint32_t* __restrict__ cell_nfluid,
+                                                        const SceneDev* __restrict__ scenes, uint32_t* __restrict__ nlist,
+                                                        uint32_t* __restrict__ ncount, float R2, uint32_t max_neibs,
+                                                        uint32_t stride, uint32_t* nfound_out, DevStatus* st, uint32_t n) {
+    const int lane = (int)(threadIdx.x & 31u);
+    const SceneDev& sc = scenes[pinfo[i]];
+    const float4 pi = pos[i];
+    const bool fluid_i = pi.w > 0.f;
+    int cx, cy, cz;
+    decode_local(cell[i] - sc.cell_offset, sc, cx, cy, cz);
+    const int dx = lane % 3 - 1, dy = (lane / 3) % 3 - 1, dz = lane / 9 - 1;
+    int nc[3] = {cx + dx, cy + dy, cz + dz};
+    bool ok = lane < 27;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        if (nc[a] < 0 || nc[a] >= sc.ncell[a]) {
+            if ((sc.periodic >> a) & 1u) nc[a] = nc[a] < 0 ? nc[a] + sc.ncell[a] : nc[a] - sc.ncell[a];
+            else ok = false;
+        }
+    }
+    uint32_t b = 0, f = 0, e = 0;
+    if (ok) {
+        const uint32_t cc = sc.cell_offset + (uint32_t)nc[0] +
+                            (uint32_t)sc.ncell[0] * ((uint32_t)nc[1] + (uint32_t)sc.ncell[1] * (uint32_t)nc[2]);
+        b = start[cc];
+        f = b + cell_nfluid[cc];  // end of the fluid part
+        e = fluid_i ? start[cc + 1] : f;
+        SPH_GUARD(b <= f && f <= start[cc + 1] && start[cc + 1] <= n, st, b = f = e = 0u)
+    }
+    const f2 nx = f2_dup((float)dx * sc.cell_f[0] - pi.x), ny = f2_dup((float)dy * sc.cell_f[1] - pi.y),
+             nz = f2_dup((float)dz * sc.cell_f[2] - pi.z);
+    const uint32_t r2lim = __float_as_uint(R2) - 1u;
+    const bool centre = lane == 13;
+    const f2 init = centre ? 0ull : f2_dup(-R2);  // the centre cell tests r^2 itself (see build_particle)
+    const uint32_t code = (uint32_t)(dx + 1) | ((uint32_t)(dy + 1) << 2) | ((uint32_t)(dz + 1) << 4);
+    uint32_t nf = 0, nb = 0, nfound = 0;
+    // two masks of 32 candidates per cell; neighbourhoods with a more crowded cell go cell by cell,
+    // 64 candidates at a time, which keeps the candidate order
+    const bool crowded = __any_sync(0xffffffffu, e > (b & ~3u) + 64u);
+    for (int turn = crowded ? 0 : 26; turn < 27; ++turn) {
+        const bool mine = !crowded || lane == turn;
+        for (uint32_t w0 = b & ~3u; __any_sync(0xffffffffu, mine && w0 < e); w0 += 64u) {
+            uint32_t m[2] = {0u, 0u};
+            const ulonglong2* q4 = reinterpret_cast<const ulonglong2*>(quads + quad_word(w0));
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint32_t h0 = w0 + 32u * h;
+                if (!mine || h0 >= e) break;
+                const uint32_t hend = min(e, h0 + 32u);
+                uint32_t g = h0, mask = 0u;
+                for (; g < hend; g += 4u, q4 += 3) {
+                    const ulonglong2 X = q4[0], Y = q4[1], Z = q4[2];
+                    const f2 q0 = r2_plus(f2_add(X.x, nx), f2_add(Y.x, ny), f2_add(Z.x, nz), init);
+                    const f2 q1 = r2_plus(f2_add(X.y, nx), f2_add(Y.y, ny), f2_add(Z.y, nz), init);
+                    if (!centre) {
+                        mask = __funnelshift_l((uint32_t)q0, mask, 1);
+                        mask = __funnelshift_l((uint32_t)(q0 >> 32), mask, 1);
+                        mask = __funnelshift_l((uint32_t)q1, mask, 1);
+                        mask = __funnelshift_l((uint32_t)(q1 >> 32), mask, 1);
+                    } else {
+                        mask = __funnelshift_l(centre_hit(f2_lo(q0), r2lim), mask, 1);
+                        mask = __funnelshift_l(centre_hit(f2_hi(q0), r2lim), mask, 1);
+                        mask = __funnelshift_l(centre_hit(f2_lo(q1), r2lim), mask, 1);
+                        mask = __funnelshift_l(centre_hit(f2_hi(q1), r2lim), mask, 1);
+                    }
+                }
+                const uint32_t first = h0 < b ? b - h0 : 0u, last = hend - h0;
+                m[h] = (mask << (32u - (g - h0))) & (0xffffffffu >> first) & (0xffffffffu << (32u - last));
+            }
+            uint32_t hits = (uint32_t)(__popc(m[0]) + __popc(m[1]));
+            uint32_t found;
+            const uint32_t before = warp_excl_sum(hits, &found);
+            nfound += found;
+            const uint32_t room = max_neibs - (nf + nb);
+            if (found > room) {  // keep the first ones in candidate order
+                const uint32_t keep = before >= room ? 0u : min(hits, room - before);
+                const uint32_t in0 = min(keep, (uint32_t)__popc(m[0]));
+                m[0] = highest_set_bits(m[0], in0);
+                m[1] = highest_set_bits(m[1], keep - in0);
+            }
+            // fluid candidates come first in the cell; both parts' counts in one prefix sum
+            uint32_t mf[2], own = 0u;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint32_t h0 = w0 + 32u * h;
+                const uint32_t nfl = f > h0 ? min(f - h0, 32u) : 0u;
+                mf[h] = nfl ? m[h] & (0xffffffffu << (32u - nfl)) : 0u;
+                m[h] ^= mf[h];
+                own += (uint32_t)__popc(mf[h]) | (uint32_t)__popc(m[h]) << 16;
+            }
+            uint32_t tot;
+            const uint32_t at = warp_excl_sum(own, &tot);
+            uint32_t kf = nf + (at & 0xffffu), kb = nb + (at >> 16);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint32_t e0 = ((w0 + 32u * h) << kCodeBits) | code;
+                for (uint32_t r = mf[h]; r; ++kf) {
+                    const uint32_t u = (uint32_t)__clz((int)r);
+                    r ^= 0x80000000u >> u;
+                    nlist[list_fluid_word(kf, i, stride)] = e0 + (u << kCodeBits);
+                }
+                for (uint32_t r = m[h]; r; ++kb) {
+                    const uint32_t u = (uint32_t)__clz((int)r);
+                    r ^= 0x80000000u >> u;
+                    nlist[list_bnd_word(kb, i, stride, max_neibs)] = e0 + (u << kCodeBits);
+                }
+            }
+            nf += tot & 0xffffu;
+            nb += tot >> 16;
+        }
+    }
+    if (lane == 0) {
+        if (nf & 1u) nlist[list_fluid_word(nf, i, stride)] = kMarker;
+        if (nb & 1u) nlist[list_bnd_word(nb, i, stride, max_neibs)] = kMarker;
+        ncount[i] = nf | (nb << 16);
+    }
+    *nfound_out = nfound;
+    return nf + nb;
+}
+
+__device__ __forceinline__ void build_warp_body(
+    const float4* __restrict__ pos, const float* __restrict__ quads, const uint32_t* __restrict__ cell,
+    const uint32_t* __restrict__ pinfo, const uint32_t* __restrict__ start, const uint32_t* __restrict__ cell_nfluid,
+    const SceneDev* __restrict__ scenes, DevStatus* __restrict__ st, uint32_t* __restrict__ nlist,
+    uint32_t* __restrict__ ncount, float R2, uint32_t max_neibs, uint32_t stride) {
+    const uint32_t n = st->n_active;
+    uint32_t most = 0, sum = 0;  // of this warp's particles
+    for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += (gridDim.x * blockDim.x) >> 5) {
+        uint32_t nfound;
+        sum += build_particle_warp(i, pos, quads, cell, pinfo, start, cell_nfluid, scenes, nlist, ncount, R2, max_neibs,
+                                   stride, &nfound, st, n);
+        most = max(most, nfound);
+    }
+    if ((threadIdx.x & 31u) == 0u && sum) {
+        if (most > max_neibs) atomicOr(&st->error_bits, SPH_EBIT_NEIB_OVERFLOW);
+        atomicMax(&st->max_neibs_seen, most);
+        atomicAdd(&st->list_entries, (unsigned long long)sum);
     }
 }
 

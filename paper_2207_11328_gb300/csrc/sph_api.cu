@@ -53,6 +53,8 @@ struct sph_ctx {
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};  // captured step, per buffer parity
     uint32_t graph_nodes = 0;
+    // build variant by the rule on the particle count (false: set or tuned)
+    bool auto_build = true;
     bool persistent = false;  // sph_set_persistent: one cooperative launch per sph_step call
     size_t staging_bytes = 0;
     std::vector<std::pair<char*, size_t>> canaries;  // checked build: (base, bytes) of guarded buffers
@@ -107,6 +109,9 @@ void check_canaries(sph_ctx* c, cudaStream_t st) {
     } while (0)
 
 inline cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s); }
+
+constexpr uint32_t kWarpBuildMax = 24576;  // see default_variants
+constexpr uint32_t kLanesTuneMax = 131072;  // sph_autotune times a warp per particle up to here
 
 constexpr double kViscousDtCoef = 0.125;  // laminar viscous time-step limit, dt <= 0.125 h^2/nu
 
@@ -599,8 +604,20 @@ inline unsigned grid_for(uint32_t n, int block) {
     return g ? g : 1;
 }
 
+// Default build variant for n particles, until sph_set_variants or sph_autotune choose: a warp per
+// particle builds the list, while a thread per particle would leave most of the GPU idle.
+// Measured on periodic boxes, us per step, thread against warp: 84 -> 50 at 4,096 particles,
+// 101 -> 89 at 19,683, 113 -> 126 at 32,768 (the line between).
+void default_variants(sph_ctx* c, uint32_t n) {
+    const int v = n <= kWarpBuildMax ? 3 : 0;
+    if (!c->auto_build || v == c->ph.build_variant) return;
+    c->ph.build_variant = v;
+    drop_graphs(c);  // captured launches carry the old shapes
+}
+
 int do_upload(sph_ctx* c, uint32_t n, const double* pos, const float* vel, const float* delta, const float* mass,
               const uint8_t* type, const uint32_t* scene, cudaStream_t st) {
+    default_variants(c, n);
     k_set_status_n<<<1, 1, 0, st>>>(c->b.status, n);
     k_reset_dyn<<<1, 256, 0, st>>>(c->b.dyn, c->g.n_scenes);
     if (n) {
@@ -753,13 +770,13 @@ int sph_create(const sph_params* p, sph_ctx** out) {
     auto alloc = [&](void** ptr, size_t bytes) -> bool { return dev_alloc(c, ptr, bytes) == cudaSuccess; };
     bool ok = true;
     for (int k = 0; k < 2; ++k) {
-        // kPosPad spare entries: the build reads candidates in groups past a cell's end
-        ok = ok && alloc((void**)&b.pos[k], sizeof(float4) * (cap + kPosPad)) &&
+        ok = ok && alloc((void**)&b.pos[k], sizeof(float4) * cap) &&
              alloc((void**)&b.vel[k], sizeof(float4) * cap) &&
              alloc((void**)&b.phat[k], sizeof(float) * cap) &&
              alloc((void**)&b.cell[k], sizeof(uint32_t) * cap) && alloc((void**)&b.pinfo[k], sizeof(uint32_t) * cap) &&
              alloc((void**)&b.pid[k], sizeof(uint32_t) * cap);
     }
+    ok = ok && alloc((void**)&b.quads, sizeof(float) * quad_floats(cap));
     if (p->rebuild_every > 1)
         ok = ok && alloc((void**)&b.pos_ref, sizeof(float4) * cap) &&
              alloc((void**)&b.nlist_x, sizeof(uint4) * 2 * (size_t)exact_bnd_chunk(p->max_neibs) * ph.stride) &&
@@ -781,7 +798,7 @@ int sph_create(const sph_params* p, sph_ctx** out) {
     cudaMemset(b.status, 0, sizeof(DevStatus));
     b.gate = p->rebuild_every > 1 ? &b.status->rebuild : nullptr;
     cudaMemset(b.force, 0, sizeof(float4) * cap);
-    for (int k = 0; k < 2; ++k) cudaMemset(b.pos[k], 0, sizeof(float4) * (cap + kPosPad));
+    cudaMemset(b.quads, 0, sizeof(float) * quad_floats(cap));
     cudaMemset(b.ncount, 0, sizeof(uint32_t) * cap);
     if (cudaDeviceSynchronize() != cudaSuccess) {
         sph_destroy(c);
@@ -1012,7 +1029,7 @@ int sph_autotune(sph_ctx* c, void* stream, int* build_variant, int* forces_varia
         cudaEventElapsedTime(&ms, e0, e1);
         return ms / 3.f;
     };
-    // neighbour build: thread/particle (128, 256 threads) or warp/cell (2, 4, 8 cells per CTA);
+    // neighbour build: thread/particle (128, 256 threads) or warp/particle (64, 128, 256 threads);
     // all variants write the same list, so the state is unchanged by tuning
     int best_v = c->ph.build_variant;
     float best = 3.4e38f;
@@ -1020,7 +1037,9 @@ int sph_autotune(sph_ctx* c, void* stream, int* build_variant, int* forces_varia
     // the in-cell sort (a skin list forces its gated pipeline open)
     if (skin_mode(c)) launch_force_rebuild(c->b, st);
     enqueue_build(c, st);
-    for (int v = 0; v < kBuildVariants; ++v) {
+    // (a group of lanes per particle is for small states: not timed where it cannot win)
+    const bool large = c->n_uploaded > kLanesTuneMax;
+    for (int v = 0; v < (large ? 2 : kBuildVariants); ++v) {
         c->ph.build_variant = v;
         const float ms = time_ms([&] { launch_build(c->b, c->cur, c->g, c->ph, st); });
         if (ms < best) {
@@ -1088,6 +1107,7 @@ int sph_autotune(sph_ctx* c, void* stream, int* build_variant, int* forces_varia
         // particles 11.94 against 8.39 + 3.56 ms, 1.65M 0.869 against 0.576 + 0.270 ms)
         c->ph.fuse_predict = t_fused < 0.98f * t_sep ? 1 : 0;
     }
+    c->auto_build = false;
     c->fresh = true;  // the last build is of the current positions
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1122,7 +1142,10 @@ int sph_set_variants(sph_ctx* c, int build_variant, int forces_variant) {
     if (!c || build_variant < -1 || build_variant >= kBuildVariants || forces_variant < -1 ||
         forces_variant >= kForcesVariants)
         return SPH_ERR_ARG;
-    if (build_variant >= 0) c->ph.build_variant = build_variant;
+    if (build_variant >= 0) {
+        c->ph.build_variant = build_variant;
+        c->auto_build = false;
+    }
     if (forces_variant >= 0) c->ph.forces_variant = c->ph.forces_variant_c = forces_variant;
     CK(cudaDeviceSynchronize());
     drop_graphs(c);  // captured launches carry the old shapes
@@ -1751,6 +1774,7 @@ void sph_destroy(sph_ctx* c) {
         cudaFree(b.pinfo[k]);
         cudaFree(b.pid[k]);
     }
+    cudaFree(b.quads);
     cudaFree(b.pos_ref);
     cudaFree(b.nlist_x);
     cudaFree(b.ncount_x);

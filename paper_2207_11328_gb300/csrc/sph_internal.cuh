@@ -179,7 +179,10 @@ __device__ __forceinline__ bool cfl_counts(const Phys& ph, const uint32_t* __res
 }
 
 constexpr int kBuildVariants = 5;
-constexpr uint32_t kPosPad = 8;  // spare float4 entries after pos[k][cap - 1] (read, never used)
+// Quads: four consecutive sorted particles' x, then their y, then their z (48 bytes), which the
+// list build loads as three 16-byte words from one address.
+__host__ __device__ constexpr size_t quad_word(uint32_t i) { return (size_t)(i >> 2) * 12u + (i & 3u); }  // x; y, z at + 4, + 8
+__host__ __device__ constexpr size_t quad_floats(uint32_t cap) { return ((size_t)cap / 4u + 1u) * 12u; }
 const char* build_variant_name(int v);
 constexpr int kForcesVariants = 5;
 const char* forces_variant_name(int v);
@@ -258,6 +261,7 @@ struct Buffers {
     float4* vel_s;
     float* phat_s;
     float4* force;           // (ax, ay, az, drho) of sph_forces
+    float* quads;            // the sorted offsets once more, in quads of four particles (see quad_word)
     uint32_t* key;           // new cell key per particle (hash)
     uint32_t* slot;          // rank within the new cell at hash time (unordered)
     uint32_t* count;         // per bucket counts (n_cells + 1 buckets)

@@ -1,0 +1,82 @@
+"""Launch shapes at the sizes where they can differ (marked gpu): cells of 1 to over 100 particles
+(hit masks of 32 candidates, aligned groups of four, two masks per lane), coincident particles,
+lists cut at their last entry, particle counts around a warp: every build variant writes one list,
+the oracle's sets, and every force shape the same bits."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+from paper_2207_11328_gb300 import N_BUILD_VARIANTS, N_FORCES_VARIANTS, scenes
+from tests.gpu_common import compare_neighbor_sets, require_gpu, sim_for
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True, scope="module")
+def _gpu():
+    require_gpu()
+
+
+def _cloud(n, cells, crowd, periodic, n_boundary=0, seed=1):
+    """n random particles in a box of cells^3 grid cells, `crowd` of them in one cell (at its
+    corner), a few coincident; the last n_boundary are boundary particles."""
+    rng = np.random.default_rng(seed)
+    s = scenes.periodic_box(n_per_axis=4, dp=0.02)
+    R = 2 * s.h
+    L = cells * R * 1.01
+    pos = rng.uniform(0, L, (n, 3))
+    pos[:crowd] = rng.uniform(0.05 * R, 0.95 * R, (crowd, 3))
+    if n > 3:
+        pos[n // 2] = pos[0]  # coincident: no pair
+    ptype = np.zeros(n, np.uint8)
+    if n_boundary:
+        ptype[n - n_boundary:] = 1
+    vel = rng.uniform(-0.1, 0.1, (n, 3)).astype(np.float32)
+    vel[ptype == 1] = 0
+    return dataclasses.replace(s, pos=pos, vel=vel, delta=rng.uniform(-1e-3, 1e-3, n).astype(np.float32),
+                               mass=np.full(n, 8e-3, np.float32), ptype=ptype, scene=np.zeros(n, np.uint32),
+                               origin=(0.0, 0.0, 0.0), size=(L, L, L), periodic=7 if periodic else 0)
+
+
+@pytest.mark.parametrize("n,cells,crowd,periodic,nb", [(1, 3, 0, True, 0), (31, 3, 0, False, 5), (33, 4, 29, True, 3),
+                                                       (200, 3, 33, True, 40), (700, 4, 70, False, 150),
+                                                       (900, 3, 130, True, 100)])
+def test_every_shape_on_uneven_cells(n, cells, crowd, periodic, nb):
+    s = _cloud(n, cells, crowd, periodic, nb)
+    ref = None
+    for v in range(max(N_BUILD_VARIANTS, N_FORCES_VARIANTS)):
+        sim = sim_for(s, max_neibs=512)
+        sim.set_variants(build=v % N_BUILD_VARIANTS, forces=v % N_FORCES_VARIANTS)
+        sim.build_neighbors()
+        counts, ids = sim.download_neighbors()
+        sim.forces()
+        got = (counts, ids, *sim.download_forces(), sim.stats()["list_entries"])
+        if ref is None:
+            ref = got
+            compare_neighbor_sets(s, counts, ids)
+        for a, b in zip(got, ref):
+            assert np.array_equal(a, b, equal_nan=True) if isinstance(a, np.ndarray) else a == b
+    # the default shapes of a state this small
+    sim = sim_for(s, max_neibs=512)
+    sim.forces()
+    for a, b in zip(sim.download_forces(), ref[2:4]):
+        assert np.array_equal(a, b, equal_nan=True)
+
+
+@pytest.mark.parametrize("max_neibs", [8, 33, 64, 65])
+def test_every_build_cuts_a_full_list_at_the_same_entry(max_neibs):
+    s = _cloud(600, 3, 90, True, 120, seed=2)
+    ref = None
+    for v in range(N_BUILD_VARIANTS):
+        sim = sim_for(s, max_neibs=max_neibs)
+        sim.set_variants(build=v)
+        sim.build_neighbors()
+        st = sim.stats(check=False)
+        assert st["rc"] == -4
+        got = (*sim.download_neighbors(), np.array([st["max_neibs_seen"], st["list_entries"]]))
+        assert (got[0].sum(1) <= max_neibs).all()
+        if ref is None:
+            ref = got
+        for a, b in zip(got, ref):
+            assert np.array_equal(a, b)
