@@ -331,8 +331,9 @@ int sph_tape_generation(sph_ctx* ctx, uint64_t* gen);
  * neighbour-build variant (one thread per particle with 128 or 256 threads
  * per block, or one warp per particle with 64, 128 or 256 threads) and each
  * force-kernel shape (64, 128 or 256 threads per block with at most 64
- * registers; 128 threads with at most 85 or 128) on the uploaded state (warps
- * per particle up to 131,072 particles), the
+ * registers; 4 or 8 lanes per particle, on a skin list 128 threads with at
+ * most 85 or 128 registers) on the uploaded state (warps and lanes per
+ * particle up to 131,072 particles), the
  * predictor and the corrector pass apart (3 timed launches each, CUDA events
  * on `stream`; the corrector runs on a scratch copy of the state), then the
  * list build and the predictor pass fused against apart (every-step list,
@@ -347,7 +348,7 @@ int sph_autotune(sph_ctx* ctx, void* stream, int* build_variant, int* forces_var
 
 /* Select the neighbour-build variant (0..4) and the force-kernel launch shape
  * (0..4, for every pass) directly, as sph_autotune would (-1 keeps the
- * current one); until then each upload picks the build by the particle count.
+ * current one); until then each upload picks them by the particle count.
  * Every variant computes the same bits.  Synchronises the
  * device; SPH_ERR_ARG for an index out of range. */
 int sph_set_variants(sph_ctx* ctx, int build_variant, int forces_variant);

@@ -38,11 +38,45 @@ namespace {
 // pass over the pairs within the cutoff; slower in the passes that filter a
 // skin list (more registers live beside the exact-list writers), which keep
 // the gather.
-template <int VISC, bool BND, bool FILTER, bool RECOMP>
+// The pair's terms go to `out` as they are formed: the running sums (Acc), or their values
+// (Terms), for a group of lanes that adds its lanes' terms in list order.
+__device__ __forceinline__ void add_rate(Acc& a, float mF, float udx) { a.drho = fmaf(mF, udx, a.drho); }
+__device__ __forceinline__ void add_force(Acc& a, float coef, float rx, float ry, float rz) {
+    a.ax = fmaf(-coef, rx, a.ax);
+    a.ay = fmaf(-coef, ry, a.ay);
+    a.az = fmaf(-coef, rz, a.az);
+}
+__device__ __forceinline__ void add_laminar(Acc& a, float lam, float ux, float uy, float uz) {
+    a.ax = fmaf(lam, ux, a.ax);
+    a.ay = fmaf(lam, uy, a.ay);
+    a.az = fmaf(lam, uz, a.az);
+}
+struct Terms {
+    float mF, udx, coef, rx, ry, rz;
+    float lam, ux, uy, uz;  // laminar only
+};
+__device__ __forceinline__ void add_rate(Terms& t, float mF, float udx) {
+    t.mF = mF;
+    t.udx = udx;
+}
+__device__ __forceinline__ void add_force(Terms& t, float coef, float rx, float ry, float rz) {
+    t.coef = coef;
+    t.rx = rx;
+    t.ry = ry;
+    t.rz = rz;
+}
+__device__ __forceinline__ void add_laminar(Terms& t, float lam, float ux, float uy, float uz) {
+    t.lam = lam;
+    t.ux = ux;
+    t.uy = uy;
+    t.uz = uz;
+}
+
+template <int VISC, bool BND, bool FILTER, bool RECOMP, class Out>
 __device__ __forceinline__ bool fluid_pair(uint32_t e, const Central& ci, const float4& vi, float phat_i,
                                            const float4* __restrict__ pos, const float4* __restrict__ vel,
                                            const float* __restrict__ phat, float phat_coef, float pi_coef,
-                                           const Phys& ph, Acc& acc, uint32_t& npairs) {
+                                           const Phys& ph, Out& out, uint32_t& npairs) {
     const uint32_t j = e >> kCodeBits;
     const float4 pj = pos[j];
     const float4 vj = vel[j];  // all gathers issued together
@@ -64,24 +98,79 @@ __device__ __forceinline__ bool fluid_pair(uint32_t e, const Central& ci, const 
     const float uy = BND ? vi.y : vi.y - vj.y;
     const float uz = BND ? vi.z : vi.z - vj.z;
     const float udx = fmaf(ux, rx, fmaf(uy, ry, uz * rz));
-    acc.drho = fmaf(mF, udx, acc.drho);
+    add_rate(out, mF, udx);
     float bracket = phat_i + phat_j;
     if (VISC == SPH_VISC_ARTIFICIAL) {
         // approaching pairs only (u.x < 0), without a branch: receding pairs add -pi*0
         const float den = (r2 + ph.eps_h2) * fmaf(0.5f, vi.w + vj.w, 1.0f);
         bracket = fmaf(-pi_coef, __fdividef(fminf(udx, 0.f), den), bracket);
     }
-    const float coef = mF * bracket;
-    acc.ax = fmaf(-coef, rx, acc.ax);
-    acc.ay = fmaf(-coef, ry, acc.ay);
-    acc.az = fmaf(-coef, rz, acc.az);
-    if (VISC == SPH_VISC_LAMINAR) {
-        const float lam = ph.nu4 * ph.inv_rho0 * __fdividef(mF, 2.0f + vi.w + vj.w);
-        acc.ax = fmaf(lam, ux, acc.ax);
-        acc.ay = fmaf(lam, uy, acc.ay);
-        acc.az = fmaf(lam, uz, acc.az);
-    }
+    add_force(out, mF * bracket, rx, ry, rz);
+    if (VISC == SPH_VISC_LAMINAR)
+        add_laminar(out, ph.nu4 * ph.inv_rho0 * __fdividef(mF, 2.0f + vi.w + vj.w), ux, uy, uz);
     return true;
+}
+
+// one fluid neighbour of a boundary particle: continuity, u_i = 0
+template <bool FILTER, class Out>
+__device__ __forceinline__ bool boundary_pair(uint32_t e, const Central& ci, const float4* __restrict__ pos,
+                                              const float4* __restrict__ vel, const Phys& ph, Out& out) {
+    const uint32_t j = e >> kCodeBits;
+    const float4 pj = pos[j];
+    const float4 vj = vel[j];
+    const float rx = pick(e, ci.xm, ci.x0, ci.xp) - pj.x;
+    const float ry = pick(e >> 2, ci.ym, ci.y0, ci.yp) - pj.y;
+    const float rz = pick(e >> 4, ci.zm, ci.z0, ci.zp) - pj.z;
+    const float r2 = fmaxf(fmaf(rx, rx, fmaf(ry, ry, rz * rz)), 1e-30f);
+    if (FILTER && !(r2 < ph.R2)) return false;
+    const float r = r2 * rsqrtf(r2);
+    const float t = fminf(fmaf(r, ph.inv_h, -2.0f), 0.0f);
+    add_rate(out, pj.w * (t * t * t), -fmaf(vj.x, rx, fmaf(vj.y, ry, vj.z * rz)));
+    return true;
+}
+
+// A part of a particle's every-step list by LANES consecutive lanes of a warp: each lane evaluates
+// every LANES-th entry's terms, then all lanes add the group's terms in list order, so the sums are
+// those of one thread, to the bit (the terms travel by shuffles: 6 a pair and lane).  For states too
+// small to fill the GPU with a thread per particle, where one thread's list is a long chain of
+// instructions: a pass over 4,096 particles 17 -> 7 us (8 lanes), 19,683 24 -> 13 us (4 lanes),
+// 71,680 32 -> 49 us (4 lanes).  terms(entry, tm) gives an entry's terms.
+template <int VISC, int LANES, class F>
+__device__ __forceinline__ void lanes_sum(const uint2* __restrict__ lp, ptrdiff_t step, uint32_t cnt, uint32_t n,
+                                          DevStatus* st, Acc& acc, F&& terms) {
+    const uint32_t sub = threadIdx.x % LANES;
+    const unsigned gmask = ((1u << (LANES & 31)) - 1u) << ((threadIdx.x & 31u) & ~(uint32_t)(LANES - 1));
+    auto entry = [&](uint32_t k) -> uint32_t {
+        return __ldg(reinterpret_cast<const uint32_t*>(lp + (ptrdiff_t)(k >> 1) * step) + (k & 1u));
+    };
+    uint32_t next = sub < cnt ? entry(sub) : 0u;
+    for (uint32_t k0 = 0; k0 < cnt; k0 += LANES) {
+        const uint32_t k = k0 + sub, e = next;
+        if (k + LANES < cnt) next = entry(k + LANES);  // one round ahead
+        Terms tm{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // past the end: zeros
+        bool ok = k < cnt;
+        SPH_GUARD(!ok || (e >> kCodeBits) < n, st, ok = false)
+        if (ok) terms(e, tm);
+#pragma unroll
+        for (int l = 0; l < LANES; ++l) {
+            Terms o;
+            o.mF = __shfl_sync(gmask, tm.mF, l, LANES);
+            o.udx = __shfl_sync(gmask, tm.udx, l, LANES);
+            o.coef = __shfl_sync(gmask, tm.coef, l, LANES);
+            o.rx = __shfl_sync(gmask, tm.rx, l, LANES);
+            o.ry = __shfl_sync(gmask, tm.ry, l, LANES);
+            o.rz = __shfl_sync(gmask, tm.rz, l, LANES);
+            if (VISC == SPH_VISC_LAMINAR) {
+                o.lam = __shfl_sync(gmask, tm.lam, l, LANES);
+                o.ux = __shfl_sync(gmask, tm.ux, l, LANES);
+                o.uy = __shfl_sync(gmask, tm.uy, l, LANES);
+                o.uz = __shfl_sync(gmask, tm.uz, l, LANES);
+            }
+            add_rate(acc, o.mF, o.udx);
+            add_force(acc, o.coef, o.rx, o.ry, o.rz);
+            if (VISC == SPH_VISC_LAMINAR) add_laminar(acc, o.lam, o.ux, o.uy, o.uz);
+        }
+    }
 }
 
 // SKIN: the list carries a skin (rebuild every k steps).  The predictor pass
@@ -110,7 +199,7 @@ __device__ __forceinline__ uint2 ld_chunk(const uint2* p) {
     return v;
 }
 
-template <int VISC, int MODE, bool SKIN, bool FRESH = false>
+template <int VISC, int MODE, bool SKIN, bool FRESH = false, int LANES = 1>
 __device__ __forceinline__ void particle_pass(
     uint32_t i, uint32_t n, const float4* __restrict__ pos, const float4* __restrict__ vel,
     const float* __restrict__ phat, float4* io_pos, float4* io_vel, float* io_phat, float4* __restrict__ force_out,
@@ -118,6 +207,7 @@ __device__ __forceinline__ void particle_pass(
     const SceneDev* __restrict__ scenes, SceneDyn* __restrict__ dyn, DevStatus* __restrict__ st, const Phys& ph,
     int acc_dt, const float4* __restrict__ pos_ref, uint32_t* __restrict__ nlist_x,
     uint32_t* __restrict__ ncount_x, const uint32_t* __restrict__ pid, uint32_t& npairs, uint32_t cnt_fresh = 0) {
+    static_assert(LANES == 1 || !(SKIN || FRESH), "a group of lanes takes an every-step list");
     static_assert(!(FRESH && SKIN), "a list written in the same kernel is a list built at this step");
     constexpr bool FILTER = SKIN && MODE != kCorrect;
     constexpr bool COMPACT = SKIN && MODE == kPredict;
@@ -137,7 +227,27 @@ __device__ __forceinline__ void particle_pass(
     const uint32_t kxb = exact_bnd_chunk(ph.max_neibs);
     ChunkWriter xf{make_uint4(0u, 0u, 0u, 0u), 0u, reinterpret_cast<uint4*>(nlist_x), S, i};
     ChunkWriter xb{make_uint4(0u, 0u, 0u, 0u), 0u, reinterpret_cast<uint4*>(nlist_x) + (size_t)kxb * S, S, i};
-    if (fluid_i && CHUNKED) {
+    if (LANES > 1) {
+        const float phat_i = phat[i];
+        const float pic = sc.pi_coef;
+        const Central ci = central_of(pi, cx, cy, cz);
+        const uint2* fl = reinterpret_cast<const uint2*>(nlist) + i;
+        const uint2* bl = fl + (size_t)(list_chunks(ph.max_neibs) - 1u) * S;
+        if (fluid_i) {
+            lanes_sum<VISC, LANES>(fl, (ptrdiff_t)S, nf, n, st, acc, [&](uint32_t e, Terms& tm) {
+                fluid_pair<VISC, false, false, RECOMP>(e, ci, vi, phat_i, pos, vel, phat, sc.phat_coef, pic, ph, tm, npairs); });
+            lanes_sum<VISC, LANES>(bl, -(ptrdiff_t)S, nb, n, st, acc, [&](uint32_t e, Terms& tm) {
+                fluid_pair<VISC, true, false, RECOMP>(e, ci, vi, phat_i, pos, vel, phat, sc.phat_coef, pic, ph, tm, npairs); });
+            acc.ax = fmaf(ph.aF, acc.ax, ph.g[0]);
+            acc.ay = fmaf(ph.aF, acc.ay, ph.g[1]);
+            acc.az = fmaf(ph.aF, acc.az, ph.g[2]);
+        } else {
+            lanes_sum<VISC, LANES>(fl, (ptrdiff_t)S, nf, n, st, acc, [&](uint32_t e, Terms& tm) {
+                boundary_pair<false>(e, ci, pos, vel, ph, tm); });
+        }
+        acc.drho *= ph.aF;
+        if (threadIdx.x % LANES != 0) return;  // the first lane finishes the particle
+    } else if (fluid_i && CHUNKED) {
         const float phat_i = phat[i];
         const float pic = sc.pi_coef;
         const Central ci = central_of(pi, cx, cy, cz);
@@ -259,24 +369,10 @@ __device__ __forceinline__ void particle_pass(
                 }
                 e = (k & 1u) ? q2.y : q2.x;
             }
-            const uint32_t j = e >> kCodeBits;
-            SPH_GUARD(j < n, st, continue)
-            const float4 pj = pos[j];
-            const float4 vj = vel[j];
-            const float rx = pick(e, ci.xm, ci.x0, ci.xp) - pj.x;
-            const float ry = pick(e >> 2, ci.ym, ci.y0, ci.yp) - pj.y;
-            const float rz = pick(e >> 4, ci.zm, ci.z0, ci.zp) - pj.z;
-            const float r2 = fmaxf(fmaf(rx, rx, fmaf(ry, ry, rz * rz)), 1e-30f);
-            if (FILTER) {
-                if (!(r2 < ph.R2)) continue;
-                ++npairs;
-            }
+            SPH_GUARD((e >> kCodeBits) < n, st, continue)
+            if (!boundary_pair<FILTER>(e, ci, pos, vel, ph, acc)) continue;
+            if (FILTER) ++npairs;
             SPH_KEEP_F(e)
-            const float r = r2 * rsqrtf(r2);
-            const float t = fminf(fmaf(r, ph.inv_h, -2.0f), 0.0f);
-            const float mF = pj.w * (t * t * t);
-            const float udx = -fmaf(vj.x, rx, fmaf(vj.y, ry, vj.z * rz));
-            acc.drho = fmaf(mF, udx, acc.drho);
         }
         acc.drho *= ph.aF;
     }
@@ -356,7 +452,7 @@ __device__ __forceinline__ void particle_pass(
     }
 }
 
-template <int VISC, int MODE, bool SKIN>
+template <int VISC, int MODE, bool SKIN, int LANES = 1>
 __device__ __forceinline__ void forces_body(
     const float4* __restrict__ pos, const float4* __restrict__ vel, const float* __restrict__ phat,
     float4* io_pos, float4* io_vel, float* io_phat, float4* __restrict__ force_out,
@@ -366,8 +462,8 @@ __device__ __forceinline__ void forces_body(
     uint32_t* __restrict__ ncount_x, const uint32_t* __restrict__ pid) {
     const uint32_t n = st->n_active;
     uint32_t npairs = 0;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        particle_pass<VISC, MODE, SKIN>(i, n, pos, vel, phat, io_pos, io_vel, io_phat, force_out, pinfo, nlist, ncount,
+    for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) / LANES; i < n; i += gridDim.x * blockDim.x / LANES)
+        particle_pass<VISC, MODE, SKIN, false, LANES>(i, n, pos, vel, phat, io_pos, io_vel, io_phat, force_out, pinfo, nlist, ncount,
                                         scenes, dyn, st, ph, acc_dt, pos_ref, nlist_x, ncount_x, pid, npairs);
     if (SKIN && MODE == kPredict) {
         const uint32_t w = __reduce_add_sync(0xffffffffu, npairs);
@@ -375,7 +471,7 @@ __device__ __forceinline__ void forces_body(
     }
 }
 
-template <int VISC, int MODE, int kBlock, int kMinBlocks, bool SKIN>
+template <int VISC, int MODE, int kBlock, int kMinBlocks, bool SKIN, int LANES>
 __global__ void __launch_bounds__(kBlock, MODE == kForcesOnly ? (kMinBlocks * 2 + 2) / 3 : kMinBlocks) k_forces(
     const float4* __restrict__ pos, const float4* __restrict__ vel, const float* __restrict__ phat,
     float4* io_pos, float4* io_vel, float* io_phat, float4* __restrict__ force_out,
@@ -383,7 +479,7 @@ __global__ void __launch_bounds__(kBlock, MODE == kForcesOnly ? (kMinBlocks * 2 
     const SceneDev* __restrict__ scenes, SceneDyn* __restrict__ dyn, DevStatus* __restrict__ st, const Phys ph,
     int acc_dt, const float4* __restrict__ pos_ref, uint32_t* __restrict__ nlist_x,
     uint32_t* __restrict__ ncount_x, const uint32_t* __restrict__ pid) {
-    forces_body<VISC, MODE, SKIN>(pos, vel, phat, io_pos, io_vel, io_phat, force_out, pinfo, nlist, ncount, scenes, dyn,
+    forces_body<VISC, MODE, SKIN, LANES>(pos, vel, phat, io_pos, io_vel, io_phat, force_out, pinfo, nlist, ncount, scenes, dyn,
                                   st, ph, acc_dt, pos_ref, nlist_x, ncount_x, pid);
 }
 
@@ -552,23 +648,23 @@ __global__ void __launch_bounds__(kPipeBlock, kPersistMinBlocks) k_step_persiste
     }
 }
 
-template <int VISC, int B, int MB, bool SKIN>
+template <int VISC, int B, int MB, bool SKIN, int LANES>
 void launch_forces_s(const Buffers& b, int cur, const Geometry& g, const Phys& ph, ForceMode mode, int acc_dt,
                      cudaStream_t st) {
-    const unsigned grid = g.cap ? (g.cap + B - 1) / B : 1;
+    const unsigned grid = g.cap ? (unsigned)(((uint64_t)g.cap * LANES + B - 1) / B) : 1;
     switch (mode) {
         case kForcesOnly:
-            k_forces<VISC, kForcesOnly, B, MB, SKIN><<<grid, B, 0, st>>>(
+            k_forces<VISC, kForcesOnly, B, MB, SKIN, LANES><<<grid, B, 0, st>>>(
                 b.pos[cur], b.vel[cur], b.phat[cur], nullptr, nullptr, nullptr, b.force, b.pinfo[cur], b.nlist,
                 b.ncount, b.scenes, b.dyn, b.status, ph, acc_dt, nullptr, nullptr, nullptr, b.pid[cur]);
             break;
         case kPredict:
-            k_forces<VISC, kPredict, B, MB, SKIN><<<grid, B, 0, st>>>(
+            k_forces<VISC, kPredict, B, MB, SKIN, LANES><<<grid, B, 0, st>>>(
                 b.pos[cur], b.vel[cur], b.phat[cur], b.pos_s, b.vel_s, b.phat_s, nullptr, b.pinfo[cur], b.nlist,
                 b.ncount, b.scenes, b.dyn, b.status, ph, 0, nullptr, b.nlist_x, b.ncount_x, b.pid[cur]);
             break;
         case kCorrect:  // a skin list: the exact list the predictor wrote
-            k_forces<VISC, kCorrect, B, MB, SKIN><<<grid, B, 0, st>>>(
+            k_forces<VISC, kCorrect, B, MB, SKIN, LANES><<<grid, B, 0, st>>>(
                 b.pos_s, b.vel_s, b.phat_s, b.pos[cur], b.vel[cur], b.phat[cur], nullptr, b.pinfo[cur],
                 SKIN ? b.nlist_x : b.nlist, SKIN ? b.ncount_x : b.ncount, b.scenes, b.dyn, b.status, ph, 0,
                 b.pos_ref, nullptr, nullptr, b.pid[cur]);
@@ -576,25 +672,27 @@ void launch_forces_s(const Buffers& b, int cur, const Geometry& g, const Phys& p
     }
 }
 
-template <int VISC, int B, int MB>
+template <int VISC, int B, int MB, int LANES = 1>
 void launch_forces_b(const Buffers& b, int cur, const Geometry& g, const Phys& ph, ForceMode mode, int acc_dt,
                      cudaStream_t st, bool skin) {
     if (skin)
-        launch_forces_s<VISC, B, MB, true>(b, cur, g, ph, mode, acc_dt, st);
+        launch_forces_s<VISC, B, MB, true, 1>(b, cur, g, ph, mode, acc_dt, st);
     else
-        launch_forces_s<VISC, B, MB, false>(b, cur, g, ph, mode, acc_dt, st);
+        launch_forces_s<VISC, B, MB, false, LANES>(b, cur, g, ph, mode, acc_dt, st);
 }
 
 // launch shapes of the force kernels (autotuned, the corrector pass on its own):
-// threads per block and the register cap implied by a minimum of resident blocks per SM
+// threads per block and the register cap implied by a minimum of resident blocks per SM; the
+// last two are groups of lanes per particle (an every-step list) or looser register caps (a
+// skin list)
 template <int VISC>
 void launch_forces_v(const Buffers& b, int cur, const Geometry& g, const Phys& ph, ForceMode mode, int acc_dt,
                      cudaStream_t st, bool skin) {
     switch (mode == kCorrect ? ph.forces_variant_c : ph.forces_variant) {
         case 0: launch_forces_b<VISC, 64, 16>(b, cur, g, ph, mode, acc_dt, st, skin); break;
         case 2: launch_forces_b<VISC, 256, 4>(b, cur, g, ph, mode, acc_dt, st, skin); break;
-        case 3: launch_forces_b<VISC, 128, 6>(b, cur, g, ph, mode, acc_dt, st, skin); break;
-        case 4: launch_forces_b<VISC, 128, 4>(b, cur, g, ph, mode, acc_dt, st, skin); break;
+        case 3: launch_forces_b<VISC, 128, 6, 4>(b, cur, g, ph, mode, acc_dt, st, skin); break;
+        case 4: launch_forces_b<VISC, 128, 4, 8>(b, cur, g, ph, mode, acc_dt, st, skin); break;
         default: launch_forces_b<VISC, 128, 8>(b, cur, g, ph, mode, acc_dt, st, skin); break;
     }
 }
@@ -672,8 +770,8 @@ void launch_forces(const Buffers& b, int cur, const Geometry& g, const Phys& ph,
 
 const char* forces_variant_name(int v) {
     static const char* names[kForcesVariants] = {"64 threads, <=64 regs", "128 threads, <=64 regs",
-                                                 "256 threads, <=64 regs", "128 threads, <=85 regs",
-                                                 "128 threads, <=128 regs"};
+                                                 "256 threads, <=64 regs", "4 lanes/particle (skin list: <=85 regs)",
+                                                 "8 lanes/particle (skin list: <=128 regs)"};
     return v >= 0 && v < kForcesVariants ? names[v] : "?";
 }
 

@@ -53,8 +53,8 @@ struct sph_ctx {
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};  // captured step, per buffer parity
     uint32_t graph_nodes = 0;
-    // build variant by the rule on the particle count (false: set or tuned)
-    bool auto_build = true;
+    // build variant / force shapes by the rule on the particle count (false: set or tuned)
+    bool auto_build = true, auto_forces = true;
     bool persistent = false;  // sph_set_persistent: one cooperative launch per sph_step call
     size_t staging_bytes = 0;
     std::vector<std::pair<char*, size_t>> canaries;  // checked build: (base, bytes) of guarded buffers
@@ -110,8 +110,8 @@ void check_canaries(sph_ctx* c, cudaStream_t st) {
 
 inline cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
-constexpr uint32_t kWarpBuildMax = 24576;  // see default_variants
-constexpr uint32_t kLanesTuneMax = 131072;  // sph_autotune times a warp per particle up to here
+constexpr uint32_t kWarpBuildMax = 24576, kLanes8Max = 8192, kLanes4Max = 24576;  // see default_variants
+constexpr uint32_t kLanesTuneMax = 131072;  // sph_autotune times groups of lanes up to here
 
 constexpr double kViscousDtCoef = 0.125;  // laminar viscous time-step limit, dt <= 0.125 h^2/nu
 
@@ -604,14 +604,22 @@ inline unsigned grid_for(uint32_t n, int block) {
     return g ? g : 1;
 }
 
-// Default build variant for n particles, until sph_set_variants or sph_autotune choose: a warp per
-// particle builds the list, while a thread per particle would leave most of the GPU idle.
-// Measured on periodic boxes, us per step, thread against warp: 84 -> 50 at 4,096 particles,
-// 101 -> 89 at 19,683, 113 -> 126 at 32,768 (the line between).
+// Default launch shapes for n particles, until sph_set_variants, sph_set_forces_variants or
+// sph_autotune choose: a warp per particle builds the list, and 8 or 4 lanes per particle evaluate
+// the every-step passes, while a thread per particle would leave most of the GPU idle.
+// Measured on periodic boxes, us per step, thread against group: list build by a warp per particle
+// 84 -> 50 at 4,096 particles, 101 -> 89 at 19,683, 113 -> 126 at 32,768 (the line between); passes
+// by 8 lanes 70 -> 50 at 4,096, by 4 lanes 105 -> 89 at 19,683, 113 -> 128 at 32,768; 8 lanes
+// against 4: 65 / 70 at 8,000, 84 / 77 at 12,167.
 void default_variants(sph_ctx* c, uint32_t n) {
-    const int v = n <= kWarpBuildMax ? 3 : 0;
-    if (!c->auto_build || v == c->ph.build_variant) return;
-    c->ph.build_variant = v;
+    Phys ph = c->ph;
+    if (c->auto_build) ph.build_variant = n <= kWarpBuildMax ? 3 : 0;
+    if (c->auto_forces)
+        ph.forces_variant = ph.forces_variant_c = skin_mode(c) || c->ph.general ? 1 : (n <= kLanes8Max ? 4 : (n <= kLanes4Max ? 3 : 1));
+    if (ph.build_variant == c->ph.build_variant && ph.forces_variant == c->ph.forces_variant &&
+        ph.forces_variant_c == c->ph.forces_variant_c)
+        return;
+    c->ph = ph;
     drop_graphs(c);  // captured launches carry the old shapes
 }
 
@@ -1052,7 +1060,8 @@ int sph_autotune(sph_ctx* c, void* stream, int* build_variant, int* forces_varia
     // force kernels: threads per block and register cap
     int best_f = c->ph.forces_variant;
     best = 3.4e38f;
-    for (int v = 0; v < kForcesVariants; ++v) {
+    const int n_shapes = large && !skin_mode(c) ? 3 : kForcesVariants;
+    for (int v = 0; v < n_shapes; ++v) {
         c->ph.forces_variant = v;
         // the predictor pass as the step runs it (it writes only the predicted-state scratch)
         const float ms = time_ms([&] { launch_forces(c->b, c->cur, c->g, c->ph, kPredict, 0, st); });
@@ -1084,7 +1093,7 @@ int sph_autotune(sph_ctx* c, void* stream, int* build_variant, int* forces_varia
         tb.vel[c->cur] = c->b.vel[alt];
         tb.phat[c->cur] = c->b.phat[alt];
         best = 3.4e38f;
-        for (int v = 0; v < kForcesVariants; ++v) {
+        for (int v = 0; v < n_shapes; ++v) {
             c->ph.forces_variant_c = v;
             const float ms = time_ms([&] { launch_forces(tb, c->cur, c->g, c->ph, kCorrect, 0, st); });
             if (ms < best) {
@@ -1107,7 +1116,7 @@ int sph_autotune(sph_ctx* c, void* stream, int* build_variant, int* forces_varia
         // particles 11.94 against 8.39 + 3.56 ms, 1.65M 0.869 against 0.576 + 0.270 ms)
         c->ph.fuse_predict = t_fused < 0.98f * t_sep ? 1 : 0;
     }
-    c->auto_build = false;
+    c->auto_build = c->auto_forces = false;
     c->fresh = true;  // the last build is of the current positions
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1131,6 +1140,7 @@ int sph_set_forces_variants(sph_ctx* c, int forces_predict, int forces_correct) 
     if (!c || forces_predict < -1 || forces_predict >= kForcesVariants || forces_correct < -1 ||
         forces_correct >= kForcesVariants)
         return SPH_ERR_ARG;
+    if (forces_predict >= 0 || forces_correct >= 0) c->auto_forces = false;
     if (forces_predict >= 0) c->ph.forces_variant = forces_predict;
     if (forces_correct >= 0) c->ph.forces_variant_c = forces_correct;
     CK(cudaDeviceSynchronize());
@@ -1146,6 +1156,7 @@ int sph_set_variants(sph_ctx* c, int build_variant, int forces_variant) {
         c->ph.build_variant = build_variant;
         c->auto_build = false;
     }
+    if (forces_variant >= 0) c->auto_forces = false;
     if (forces_variant >= 0) c->ph.forces_variant = c->ph.forces_variant_c = forces_variant;
     CK(cudaDeviceSynchronize());
     drop_graphs(c);  // captured launches carry the old shapes
