@@ -82,15 +82,15 @@ __global__ void __launch_bounds__(kBlockT, 1024 / kBlockT) k_build_tpp(
     build_tpp_body(pos, quads, cell, pinfo, start, cell_nfluid, scenes, st, nlist, ncount, R2, max_neibs, stride);
 }
 
-// the same list by one warp per particle (build_particle_warp)
-template <int kBlockT>
-__global__ void __launch_bounds__(kBlockT) k_build_warp(
+// the same list by nine warps per 32 particles (build_rows_body)
+template <int kMinBlocks>
+__global__ void __launch_bounds__(kRowBlock, kMinBlocks) k_build_rows(
     const float4* __restrict__ pos, const float* __restrict__ quads, const uint32_t* __restrict__ cell,
     const uint32_t* __restrict__ pinfo, const uint32_t* __restrict__ start, const uint32_t* __restrict__ cell_nfluid,
     const SceneDev* __restrict__ scenes, DevStatus* __restrict__ st, uint32_t* __restrict__ nlist,
     uint32_t* __restrict__ ncount, float R2, uint32_t max_neibs, uint32_t stride, const uint32_t* __restrict__ gate) {
     if (gate && *gate == 0u) return;
-    build_warp_body(pos, quads, cell, pinfo, start, cell_nfluid, scenes, st, nlist, ncount, R2, max_neibs, stride);
+    build_rows_body(pos, quads, cell, pinfo, start, cell_nfluid, scenes, st, nlist, ncount, R2, max_neibs, stride);
 }
 
 inline unsigned grid_for(uint64_t n, int block) {
@@ -139,17 +139,19 @@ void launch_build_tpp(const Buffers& b, int cur, const Geometry& g, const Phys& 
                                                      ph.stride, b.gate);
 }
 
-template <int B>
-void launch_build_warp(const Buffers& b, int cur, const Geometry& g, const Phys& ph, cudaStream_t st) {
-    // 16 warps per scheduler slot at most: a warp then takes several particles in turn
-    const unsigned grid = std::min(grid_for((uint64_t)g.cap * 32u, B), 152u * (2048u / B));
-    k_build_warp<B><<<grid, B, 0, st>>>(b.pos[cur], b.quads, b.cell[cur], b.pinfo[cur], b.start, b.cell_nfluid, b.scenes,
-                                        b.status, b.nlist, b.ncount, ph.R2_list, ph.max_neibs, ph.stride, b.gate);
+template <int MB>
+void launch_build_rows(const Buffers& b, int cur, const Geometry& g, const Phys& ph, cudaStream_t st) {
+    const size_t smem = ph.max_neibs <= kStageNeibs ? sizeof(uint32_t) * rows_smem_words(ph.max_neibs) : 0;
+    // resident blocks at most: a block then takes several tiles in turn
+    const unsigned grid = std::min(grid_for(g.cap, 32), 152u * MB);
+    k_build_rows<MB><<<grid, kRowBlock, smem, st>>>(b.pos[cur], b.quads, b.cell[cur], b.pinfo[cur], b.start, b.cell_nfluid,
+                                                   b.scenes, b.status, b.nlist, b.ncount, ph.R2_list, ph.max_neibs,
+                                                   ph.stride, b.gate);
 }
 
 const char* build_variant_name(int v) {
-    static const char* names[kBuildVariants] = {"thread/particle x128", "thread/particle x256", "warp/particle x64",
-                                                "warp/particle x128", "warp/particle x256"};
+    static const char* names[kBuildVariants] = {"thread/particle x128", "thread/particle x256", "warp/row x2 blocks/SM",
+                                                "warp/row x3 blocks/SM", "warp/row x4 blocks/SM"};
     return v >= 0 && v < kBuildVariants ? names[v] : "?";
 }
 
@@ -198,9 +200,9 @@ void launch_build(const Buffers& b, int cur, const Geometry& g, const Phys& ph, 
     switch (ph.build_variant) {
         case 0: launch_build_tpp<128>(b, cur, g, ph, st); break;
         case 1: launch_build_tpp<256>(b, cur, g, ph, st); break;
-        case 2: launch_build_warp<64>(b, cur, g, ph, st); break;
-        case 3: launch_build_warp<128>(b, cur, g, ph, st); break;
-        default: launch_build_warp<256>(b, cur, g, ph, st); break;
+        case 2: launch_build_rows<2>(b, cur, g, ph, st); break;
+        case 3: launch_build_rows<3>(b, cur, g, ph, st); break;
+        default: launch_build_rows<4>(b, cur, g, ph, st); break;
     }
 }
 

@@ -475,166 +475,228 @@ __device__ __forceinline__ void build_tpp_body(
     }
 }
 
-// The same list by one warp per particle: lane l < 27 tests the candidates of neighbour cell l, a
-// prefix sum of the lanes' hit counts gives each cell's hits their place, and each lane appends its
-// own: the one thread's list, entry for entry.  For states too small to fill the GPU with a
-// thread per particle, whose 27 cells are one long chain of instructions: 4,096 particles 38 -> 11 us,
-// 19,683 48 -> 36 us, 71,680 50 -> 102 us (1,019 warp instructions a particle, 15 of 32 lanes active,
-// against 224 by a thread).
-__device__ __forceinline__ uint32_t warp_excl_sum(uint32_t v, uint32_t* total) {
-    const uint32_t lane = threadIdx.x & 31u;
-    uint32_t incl = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-        if ((int)lane >= o) incl += t;
-    }
-    *total = __shfl_sync(0xffffffffu, incl, 31);
-    return incl - v;
+// The same list by a block of nine warps for 32 particles: lane l of every warp is particle l of the
+// tile, warp r tests the candidates of neighbour row r (three cells), with the broadcast loads of
+// the one thread's build.  The rows' hit counts give each row's hits their place; the lists are put
+// together in shared memory and written chunk by chunk, the tile's particles side by side.  The one
+// thread's list, entry for entry.  For states too small to fill the GPU with a thread per particle,
+// whose nine rows are one long chain of instructions: one thread against the nine warps, us: 38 / 9
+// at 4,096 particles, 48 / 19 at 19,683, 51 / 42 at 71,680; 466 / 725 at 1.65M (380 warp
+// instructions a particle against 224).  Before, a warp per particle with a lane per cell: 11, 36, 102 us
+// (1,019 instructions, every lane at an address of its own); nine lanes per particle: 11, 33, 91 us.
+// A tile beside a cell of over 64 candidate slots, and lists of over kStageNeibs entries, take the one
+// thread's build.
+constexpr int kRowWarps = 9;
+constexpr int kRowBlock = 32 * kRowWarps;
+constexpr uint32_t kStageNeibs = 256;
+// shared words: the tile's lists (an odd stride apart: lanes of a warp write different banks), the
+// hits of every row and particle
+__host__ __device__ constexpr uint32_t rows_list_words(uint32_t max_neibs) { return max_neibs | 1u; }
+__host__ __device__ constexpr uint32_t rows_smem_words(uint32_t max_neibs) {
+    return 32u * (rows_list_words(max_neibs) + 2u * kRowWarps);
 }
 
-__device__ __forceinline__ uint32_t build_particle_warp(uint32_t i, const float4* __restrict__ pos,
-                                                        const float* __restrict__ quads,
-                                                        const uint32_t* __restrict__ cell,
-                                                        const uint32_t* __restrict__ pinfo,
-                                                        const uint32_t* __restrict__ start,
-                                                        const uint32_t* __restrict__ cell_nfluid,
-                                                        const SceneDev* __restrict__ scenes, uint32_t* __restrict__ nlist,
-                                                        uint32_t* __restrict__ ncount, float R2, uint32_t max_neibs,
-                                                        uint32_t stride, uint32_t* nfound_out, DevStatus* st, uint32_t n) {
-    const int lane = (int)(threadIdx.x & 31u);
-    const SceneDev& sc = scenes[pinfo[i]];
-    const float4 pi = pos[i];
-    const bool fluid_i = pi.w > 0.f;
-    int cx, cy, cz;
-    decode_local(cell[i] - sc.cell_offset, sc, cx, cy, cz);
-    const int dx = lane % 3 - 1, dy = (lane / 3) % 3 - 1, dz = lane / 9 - 1;
-    int nc[3] = {cx + dx, cy + dy, cz + dz};
-    bool ok = lane < 27;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        if (nc[a] < 0 || nc[a] >= sc.ncell[a]) {
-            if ((sc.periodic >> a) & 1u) nc[a] = nc[a] < 0 ? nc[a] + sc.ncell[a] : nc[a] - sc.ncell[a];
-            else ok = false;
+// hit mask (first candidate in the top bit) of the candidates [b, e) at or after h0, 32 at most;
+// h0 a multiple of four
+__device__ __forceinline__ uint32_t cell_mask(const float* __restrict__ quads, uint32_t h0, uint32_t b, uint32_t e, f2 nx,
+                                              f2 ny, f2 nz, f2 mR2, bool centre, uint32_t r2lim) {
+    if (h0 >= e) return 0u;
+    const uint32_t hend = min(e, h0 + 32u);
+    const ulonglong2* q4 = reinterpret_cast<const ulonglong2*>(quads + quad_word(h0));
+    uint32_t g = h0, mask = 0u;
+    if (!centre) {
+#pragma unroll 1
+        for (; g < hend; g += 4u, q4 += 3) {
+            const ulonglong2 X = q4[0], Y = q4[1], Z = q4[2];
+            const f2 q0 = r2_plus(f2_add(X.x, nx), f2_add(Y.x, ny), f2_add(Z.x, nz), mR2);
+            const f2 q1 = r2_plus(f2_add(X.y, nx), f2_add(Y.y, ny), f2_add(Z.y, nz), mR2);
+            mask = __funnelshift_l((uint32_t)q0, mask, 1);
+            mask = __funnelshift_l((uint32_t)(q0 >> 32), mask, 1);
+            mask = __funnelshift_l((uint32_t)q1, mask, 1);
+            mask = __funnelshift_l((uint32_t)(q1 >> 32), mask, 1);
+        }
+    } else {
+#pragma unroll 1
+        for (; g < hend; g += 4u, q4 += 3) {
+            const ulonglong2 X = q4[0], Y = q4[1], Z = q4[2];
+            const f2 a0 = r2_plus(f2_add(X.x, nx), f2_add(Y.x, ny), f2_add(Z.x, nz), 0ull);
+            const f2 a1 = r2_plus(f2_add(X.y, nx), f2_add(Y.y, ny), f2_add(Z.y, nz), 0ull);
+            mask = __funnelshift_l(centre_hit(f2_lo(a0), r2lim), mask, 1);
+            mask = __funnelshift_l(centre_hit(f2_hi(a0), r2lim), mask, 1);
+            mask = __funnelshift_l(centre_hit(f2_lo(a1), r2lim), mask, 1);
+            mask = __funnelshift_l(centre_hit(f2_hi(a1), r2lim), mask, 1);
         }
     }
-    uint32_t b = 0, f = 0, e = 0;
-    if (ok) {
-        const uint32_t cc = sc.cell_offset + (uint32_t)nc[0] +
-                            (uint32_t)sc.ncell[0] * ((uint32_t)nc[1] + (uint32_t)sc.ncell[1] * (uint32_t)nc[2]);
-        b = start[cc];
-        f = b + cell_nfluid[cc];  // end of the fluid part
-        e = fluid_i ? start[cc + 1] : f;
-        SPH_GUARD(b <= f && f <= start[cc + 1] && start[cc + 1] <= n, st, b = f = e = 0u)
-    }
-    const f2 nx = f2_dup((float)dx * sc.cell_f[0] - pi.x), ny = f2_dup((float)dy * sc.cell_f[1] - pi.y),
-             nz = f2_dup((float)dz * sc.cell_f[2] - pi.z);
-    const uint32_t r2lim = __float_as_uint(R2) - 1u;
-    const bool centre = lane == 13;
-    const f2 init = centre ? 0ull : f2_dup(-R2);  // the centre cell tests r^2 itself (see build_particle)
-    const uint32_t code = (uint32_t)(dx + 1) | ((uint32_t)(dy + 1) << 2) | ((uint32_t)(dz + 1) << 4);
-    uint32_t nf = 0, nb = 0, nfound = 0;
-    // two masks of 32 candidates per cell; neighbourhoods with a more crowded cell go cell by cell,
-    // 64 candidates at a time, which keeps the candidate order
-    const bool crowded = __any_sync(0xffffffffu, e > (b & ~3u) + 64u);
-    for (int turn = crowded ? 0 : 26; turn < 27; ++turn) {
-        const bool mine = !crowded || lane == turn;
-        for (uint32_t w0 = b & ~3u; __any_sync(0xffffffffu, mine && w0 < e); w0 += 64u) {
-            uint32_t m[2] = {0u, 0u};
-            const ulonglong2* q4 = reinterpret_cast<const ulonglong2*>(quads + quad_word(w0));
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const uint32_t h0 = w0 + 32u * h;
-                if (!mine || h0 >= e) break;
-                const uint32_t hend = min(e, h0 + 32u);
-                uint32_t g = h0, mask = 0u;
-                for (; g < hend; g += 4u, q4 += 3) {
-                    const ulonglong2 X = q4[0], Y = q4[1], Z = q4[2];
-                    const f2 q0 = r2_plus(f2_add(X.x, nx), f2_add(Y.x, ny), f2_add(Z.x, nz), init);
-                    const f2 q1 = r2_plus(f2_add(X.y, nx), f2_add(Y.y, ny), f2_add(Z.y, nz), init);
-                    if (!centre) {
-                        mask = __funnelshift_l((uint32_t)q0, mask, 1);
-                        mask = __funnelshift_l((uint32_t)(q0 >> 32), mask, 1);
-                        mask = __funnelshift_l((uint32_t)q1, mask, 1);
-                        mask = __funnelshift_l((uint32_t)(q1 >> 32), mask, 1);
-                    } else {
-                        mask = __funnelshift_l(centre_hit(f2_lo(q0), r2lim), mask, 1);
-                        mask = __funnelshift_l(centre_hit(f2_hi(q0), r2lim), mask, 1);
-                        mask = __funnelshift_l(centre_hit(f2_lo(q1), r2lim), mask, 1);
-                        mask = __funnelshift_l(centre_hit(f2_hi(q1), r2lim), mask, 1);
-                    }
-                }
-                const uint32_t first = h0 < b ? b - h0 : 0u, last = hend - h0;
-                m[h] = (mask << (32u - (g - h0))) & (0xffffffffu >> first) & (0xffffffffu << (32u - last));
-            }
-            uint32_t hits = (uint32_t)(__popc(m[0]) + __popc(m[1]));
-            uint32_t found;
-            const uint32_t before = warp_excl_sum(hits, &found);
-            nfound += found;
-            const uint32_t room = max_neibs - (nf + nb);
-            if (found > room) {  // keep the first ones in candidate order
-                const uint32_t keep = before >= room ? 0u : min(hits, room - before);
-                const uint32_t in0 = min(keep, (uint32_t)__popc(m[0]));
-                m[0] = highest_set_bits(m[0], in0);
-                m[1] = highest_set_bits(m[1], keep - in0);
-            }
-            // fluid candidates come first in the cell; both parts' counts in one prefix sum
-            uint32_t mf[2], own = 0u;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const uint32_t h0 = w0 + 32u * h;
-                const uint32_t nfl = f > h0 ? min(f - h0, 32u) : 0u;
-                mf[h] = nfl ? m[h] & (0xffffffffu << (32u - nfl)) : 0u;
-                m[h] ^= mf[h];
-                own += (uint32_t)__popc(mf[h]) | (uint32_t)__popc(m[h]) << 16;
-            }
-            uint32_t tot;
-            const uint32_t at = warp_excl_sum(own, &tot);
-            uint32_t kf = nf + (at & 0xffffu), kb = nb + (at >> 16);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const uint32_t e0 = ((w0 + 32u * h) << kCodeBits) | code;
-                for (uint32_t r = mf[h]; r; ++kf) {
-                    const uint32_t u = (uint32_t)__clz((int)r);
-                    r ^= 0x80000000u >> u;
-                    nlist[list_fluid_word(kf, i, stride)] = e0 + (u << kCodeBits);
-                }
-                for (uint32_t r = m[h]; r; ++kb) {
-                    const uint32_t u = (uint32_t)__clz((int)r);
-                    r ^= 0x80000000u >> u;
-                    nlist[list_bnd_word(kb, i, stride, max_neibs)] = e0 + (u << kCodeBits);
-                }
-            }
-            nf += tot & 0xffffu;
-            nb += tot >> 16;
-        }
-    }
-    if (lane == 0) {
-        if (nf & 1u) nlist[list_fluid_word(nf, i, stride)] = kMarker;
-        if (nb & 1u) nlist[list_bnd_word(nb, i, stride, max_neibs)] = kMarker;
-        ncount[i] = nf | (nb << 16);
-    }
-    *nfound_out = nfound;
-    return nf + nb;
+    const uint32_t first = h0 < b ? b - h0 : 0u, last = hend - h0;
+    return (mask << (32u - (g - h0))) & (0xffffffffu >> first) & (0xffffffffu << (32u - last));
 }
 
-__device__ __forceinline__ void build_warp_body(
+// the fallback, out of line (its registers would spill the common path's)
+__device__ __noinline__ uint32_t build_particle_alone(uint32_t i, const float4* __restrict__ pos,
+                                                      const float* __restrict__ quads, const uint32_t* __restrict__ cell,
+                                                      const uint32_t* __restrict__ pinfo, const uint32_t* __restrict__ start,
+                                                      const uint32_t* __restrict__ cell_nfluid,
+                                                      const SceneDev* __restrict__ scenes, uint32_t* __restrict__ nlist,
+                                                      uint32_t* __restrict__ ncount, float R2, uint32_t max_neibs,
+                                                      uint32_t stride, uint32_t* nfound, DevStatus* st, uint32_t n) {
+    return build_particle(i, pos, quads, cell, pinfo, start, cell_nfluid, scenes, nlist, ncount, R2, max_neibs, stride,
+                          nfound, st, n);
+}
+
+__device__ __forceinline__ void build_rows_body(
     const float4* __restrict__ pos, const float* __restrict__ quads, const uint32_t* __restrict__ cell,
     const uint32_t* __restrict__ pinfo, const uint32_t* __restrict__ start, const uint32_t* __restrict__ cell_nfluid,
     const SceneDev* __restrict__ scenes, DevStatus* __restrict__ st, uint32_t* __restrict__ nlist,
     uint32_t* __restrict__ ncount, float R2, uint32_t max_neibs, uint32_t stride) {
+    extern __shared__ uint32_t rows_smem[];
+    const int lane = (int)(threadIdx.x & 31u), r = (int)(threadIdx.x >> 5);
+    const bool can_stage = max_neibs <= kStageNeibs;
+    uint32_t* const list = rows_smem + lane * rows_list_words(max_neibs);  // fluid entries from the front, boundary from the back
+    uint32_t* const hit_s = rows_smem + 32u * rows_list_words(max_neibs);  // [row][particle]: fluid | boundary << 16
+    uint32_t* const kept_s = hit_s + 32 * kRowWarps;                       // the same after a cut at max_neibs
     const uint32_t n = st->n_active;
-    uint32_t most = 0, sum = 0;  // of this warp's particles
-    for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += (gridDim.x * blockDim.x) >> 5) {
-        uint32_t nfound;
-        sum += build_particle_warp(i, pos, quads, cell, pinfo, start, cell_nfluid, scenes, nlist, ncount, R2, max_neibs,
-                                   stride, &nfound, st, n);
-        most = max(most, nfound);
+    const uint32_t r2lim = __float_as_uint(R2) - 1u;
+    const f2 mR2 = f2_dup(-R2);
+    uint32_t most = 0, sum = 0;  // of this lane's particles
+    for (uint32_t i0 = blockIdx.x * 32u; i0 < n; i0 += gridDim.x * 32u) {
+        const uint32_t i = i0 + (uint32_t)lane;
+        const bool have = i < n;
+        uint32_t b[3] = {0u, 0u, 0u}, f[3] = {0u, 0u, 0u}, e[3] = {0u, 0u, 0u};
+        float4 pi = make_float4(0.f, 0.f, 0.f, 0.f);
+        f2 ny = 0ull, nz = 0ull;
+        float cell_x = 0.f;
+        if (have) {
+            const SceneDev& sc = scenes[pinfo[i]];
+            pi = pos[i];
+            int cx, cy, cz;
+            decode_local(cell[i] - sc.cell_offset, sc, cx, cy, cz);
+            const int dy = r % 3 - 1, dz = r / 3 - 1;
+            int y = cy + dy, z = cz + dz;
+            bool row_ok = true;
+            if (y < 0 || y >= sc.ncell[1]) {
+                if ((sc.periodic >> 1) & 1u) y = y < 0 ? y + sc.ncell[1] : y - sc.ncell[1];
+                else row_ok = false;
+            }
+            if (z < 0 || z >= sc.ncell[2]) {
+                if ((sc.periodic >> 2) & 1u) z = z < 0 ? z + sc.ncell[2] : z - sc.ncell[2];
+                else row_ok = false;
+            }
+            const uint32_t row = sc.cell_offset + (uint32_t)sc.ncell[0] * ((uint32_t)y + (uint32_t)sc.ncell[1] * (uint32_t)z);
+            cell_x = sc.cell_f[0];
+            ny = f2_dup((float)dy * sc.cell_f[1] - pi.y);
+            nz = f2_dup((float)dz * sc.cell_f[2] - pi.z);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                int x = cx + k - 1;
+                bool ok = row_ok;
+                if (x < 0 || x >= sc.ncell[0]) {
+                    if (sc.periodic & 1u) x = x < 0 ? x + sc.ncell[0] : x - sc.ncell[0];
+                    else ok = false;
+                }
+                if (ok) {
+                    const uint32_t cc = row + (uint32_t)x;
+                    b[k] = start[cc];
+                    f[k] = b[k] + cell_nfluid[cc];  // end of the fluid part
+                    e[k] = pi.w > 0.f ? start[cc + 1] : f[k];
+                    SPH_GUARD(b[k] <= f[k] && f[k] <= start[cc + 1] && start[cc + 1] <= n, st, b[k] = f[k] = e[k] = 0u)
+                }
+            }
+        }
+        const bool crowded = e[0] > (b[0] & ~3u) + 64u || e[1] > (b[1] & ~3u) + 64u || e[2] > (b[2] & ~3u) + 64u;
+        if (__syncthreads_or(crowded || !can_stage)) {
+            if (r == 0 && have) {
+                uint32_t nfound;
+                sum += build_particle_alone(i, pos, quads, cell, pinfo, start, cell_nfluid, scenes, nlist, ncount, R2,
+                                            max_neibs, stride, &nfound, st, n);
+                most = max(most, nfound);
+            }
+            continue;
+        }
+        // hits of the row's three cells, up to 64 candidate slots each; fluid candidates first in a cell
+        uint32_t m[6], fluid[6], hits = 0u;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            const int k = q / 2;
+            const uint32_t h0 = (b[k] & ~3u) + 32u * (uint32_t)(q & 1);
+            m[q] = 0u;
+            if ((q & 1) == 0 || h0 < e[k])
+                m[q] = cell_mask(quads, h0, b[k], e[k], f2_dup((float)(k - 1) * cell_x - pi.x), ny, nz, mR2, k == 1 && r == 4,
+                                 r2lim);
+            const uint32_t nfl = f[k] > h0 ? min(f[k] - h0, 32u) : 0u;
+            fluid[q] = nfl ? 0xffffffffu << (32u - nfl) : 0u;
+            hits += (uint32_t)__popc(m[q] & fluid[q]) | (uint32_t)__popc(m[q] & ~fluid[q]) << 16;
+        }
+        hit_s[32 * r + lane] = hits;
+        __syncthreads();
+        uint32_t at = 0u, all = 0u;  // hits of the rows before, of all rows
+#pragma unroll
+        for (int q = 0; q < kRowWarps; ++q) {
+            const uint32_t h = hit_s[32 * q + lane];
+            at += q < r ? h : 0u;
+            all += h;
+        }
+        const uint32_t nfound = (all & 0xffffu) + (all >> 16);
+        if (__syncthreads_or(nfound > max_neibs)) {  // keep the first ones in candidate order
+            const uint32_t before = (at & 0xffffu) + (at >> 16);
+            uint32_t keep = before < max_neibs ? max_neibs - before : 0u;
+            hits = 0u;
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                const uint32_t c = min(keep, (uint32_t)__popc(m[q]));
+                m[q] = highest_set_bits(m[q], c);
+                keep -= c;
+                hits += (uint32_t)__popc(m[q] & fluid[q]) | (uint32_t)__popc(m[q] & ~fluid[q]) << 16;
+            }
+            kept_s[32 * r + lane] = hits;
+            __syncthreads();
+            at = all = 0u;
+            for (int q = 0; q < kRowWarps; ++q) {
+                const uint32_t h = kept_s[32 * q + lane];
+                at += q < r ? h : 0u;
+                all += h;
+            }
+        }
+        uint32_t kf = at & 0xffffu, kb = max_neibs - 1u - (at >> 16);
+        const uint32_t code = ((uint32_t)(r % 3) << 2) | ((uint32_t)(r / 3) << 4);
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            const int k = q / 2;
+            const uint32_t e0 = (((b[k] & ~3u) + 32u * (uint32_t)(q & 1)) << kCodeBits) | code | (uint32_t)k;
+            for (uint32_t s = m[q] & fluid[q]; s; ++kf) {
+                const uint32_t u = (uint32_t)__clz((int)s);
+                s ^= 0x80000000u >> u;
+                list[kf] = e0 + (u << kCodeBits);
+            }
+            for (uint32_t s = m[q] & ~fluid[q]; s; --kb) {
+                const uint32_t u = (uint32_t)__clz((int)s);
+                s ^= 0x80000000u >> u;
+                list[kb] = e0 + (u << kCodeBits);
+            }
+        }
+        __syncthreads();
+        // chunks r, r + 9, ... of both parts, one particle per lane
+        const uint32_t nf = all & 0xffffu, nb = all >> 16;
+        uint2* const rows = reinterpret_cast<uint2*>(nlist) + i;
+        for (uint32_t c = (uint32_t)r; 2u * c < nf; c += kRowWarps)
+            rows[(size_t)c * stride] = make_uint2(list[2u * c], 2u * c + 1u < nf ? list[2u * c + 1u] : kMarker);
+        for (uint32_t c = (uint32_t)r; 2u * c < nb; c += kRowWarps)
+            rows[(size_t)(list_chunks(max_neibs) - 1u - c) * stride] =
+                make_uint2(list[max_neibs - 1u - 2u * c], 2u * c + 1u < nb ? list[max_neibs - 2u - 2u * c] : kMarker);
+        if (r == 0 && have) {
+            ncount[i] = all;
+            most = max(most, nfound);
+            sum += nf + nb;
+        }
+        __syncthreads();  // the shared lists are free again
     }
-    if ((threadIdx.x & 31u) == 0u && sum) {
-        if (most > max_neibs) atomicOr(&st->error_bits, SPH_EBIT_NEIB_OVERFLOW);
-        atomicMax(&st->max_neibs_seen, most);
-        atomicAdd(&st->list_entries, (unsigned long long)sum);
+    if (r == 0) {
+        most = __reduce_max_sync(0xffffffffu, most);
+        sum = __reduce_add_sync(0xffffffffu, sum);
+        if (lane == 0 && most) {
+            if (most > max_neibs) atomicOr(&st->error_bits, SPH_EBIT_NEIB_OVERFLOW);
+            atomicMax(&st->max_neibs_seen, most);
+            atomicAdd(&st->list_entries, (unsigned long long)sum);
+        }
     }
 }
 

@@ -110,7 +110,7 @@ void check_canaries(sph_ctx* c, cudaStream_t st) {
 
 inline cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
-constexpr uint32_t kWarpBuildMax = 24576, kLanes8Max = 8192, kLanes4Max = 24576;  // see default_variants
+constexpr uint32_t kRowBuildMax = 81920, kLanes8Max = 8192, kLanes4Max = 24576;  // see default_variants
 constexpr uint32_t kLanesTuneMax = 131072;  // sph_autotune times groups of lanes up to here
 
 constexpr double kViscousDtCoef = 0.125;  // laminar viscous time-step limit, dt <= 0.125 h^2/nu
@@ -605,15 +605,15 @@ inline unsigned grid_for(uint32_t n, int block) {
 }
 
 // Default launch shapes for n particles, until sph_set_variants, sph_set_forces_variants or
-// sph_autotune choose: a warp per particle builds the list, and 8 or 4 lanes per particle evaluate
-// the every-step passes, while a thread per particle would leave most of the GPU idle.
-// Measured on periodic boxes, us per step, thread against group: list build by a warp per particle
-// 84 -> 50 at 4,096 particles, 101 -> 89 at 19,683, 113 -> 126 at 32,768 (the line between); passes
-// by 8 lanes 70 -> 50 at 4,096, by 4 lanes 105 -> 89 at 19,683, 113 -> 128 at 32,768; 8 lanes
-// against 4: 65 / 70 at 8,000, 84 / 77 at 12,167.
+// sph_autotune choose: nine warps per 32 particles build the list, and 8 or 4 lanes per particle
+// evaluate the every-step passes, while a thread per particle would leave most of the GPU idle.
+// Measured on periodic boxes, us per step, thread against group: list build 98 / 71 at 4,096
+// particles, 114 / 94 at 32,768, 124 / 117 at 64,000, 166 / 174 at 125,000 (the line between); passes
+// by 8 lanes 69 / 48 at 4,096, by 4 lanes 86 / 73 at 19,683, 98 / 107 at 32,768 (the line between);
+// 8 lanes against 4: 65 / 70 at 8,000, 68 / 60 at 12,167.
 void default_variants(sph_ctx* c, uint32_t n) {
     Phys ph = c->ph;
-    if (c->auto_build) ph.build_variant = n <= kWarpBuildMax ? 3 : 0;
+    if (c->auto_build) ph.build_variant = n <= kRowBuildMax ? 4 : 0;
     if (c->auto_forces)
         ph.forces_variant = ph.forces_variant_c = skin_mode(c) || c->ph.general ? 1 : (n <= kLanes8Max ? 4 : (n <= kLanes4Max ? 3 : 1));
     if (ph.build_variant == c->ph.build_variant && ph.forces_variant == c->ph.forces_variant &&
@@ -1037,7 +1037,7 @@ int sph_autotune(sph_ctx* c, void* stream, int* build_variant, int* forces_varia
         cudaEventElapsedTime(&ms, e0, e1);
         return ms / 3.f;
     };
-    // neighbour build: thread/particle (128, 256 threads) or warp/particle (64, 128, 256 threads);
+    // neighbour build: thread/particle (128, 256 threads) or warp/row (2, 3, 4 blocks per SM);
     // all variants write the same list, so the state is unchanged by tuning
     int best_v = c->ph.build_variant;
     float best = 3.4e38f;
