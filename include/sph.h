@@ -370,7 +370,8 @@ const char* sph_forces_variant_name(int variant);
 
 /* Same work as sph_step, launched kernel by kernel (no graph) with CUDA
  * events recorded on `stream` between the launches; adds the elapsed
- * milliseconds of each phase to phase_ms[0..7]: 0 dt, 1 hash, 2 scan,
+ * milliseconds of each phase to phase_ms[0..7]: 0 dt (skin list; else
+ * computed beside the scan, phase 2), 1 hash, 2 scan,
  * 3 scatter, 4 in-cell sort + reorder, 5 neighbour-list build (with the
  * predictor pass when they are fused, see sph_set_fused_predict),
  * 6 forces + predictor (0 when fused), 7 forces + corrector.  Synchronises after each

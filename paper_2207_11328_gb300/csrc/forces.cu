@@ -513,60 +513,13 @@ __global__ void k_predict_from_forces(const float4* __restrict__ pos, const floa
     }
 }
 
-// One thread per scene: dt for the coming step (reading C7), simulated
-// time, reset of the |a|^2 accumulator.
-// The CFL time step of a scene from the largest |a|^2 of the last reduction (reading C7)
-__device__ __forceinline__ double cfl_dt_of(const SceneDev& sc, const SceneDyn& d, double h, double cfl,
-                                            double dt_fixed) {
-    if (dt_fixed > 0.0) return dt_fixed;
-    double dt = sc.dt_cap;
-    const double a2 = (double)__uint_as_float(d.amax2_bits);
-    if (a2 > 0.0) dt = fmin(dt, cfl * sqrt(h / sqrt(a2)));
-    return dt;
-}
-
-__device__ __forceinline__ void dt_body(const SceneDev* __restrict__ scenes, SceneDyn* __restrict__ dyn,
-                                        DevStatus* __restrict__ st, uint32_t n_scenes, double h, double cfl,
-                                        double dt_fixed, int advance, uint32_t rebuild_every, float trig2,
-                                        uint32_t builds_inc) {
-    const double dt_host = st->dt_next;  // the host's time step for this step (sph_set_dt), or <= 0
-    __syncthreads();
-    for (uint32_t s = threadIdx.x; s < n_scenes; s += blockDim.x) {
-        const double dt = dt_host > 0.0 ? dt_host : cfl_dt_of(scenes[s], dyn[s], h, cfl, dt_fixed);
-        dyn[s].dt = (float)dt;
-        dyn[s].dt_d = dt;
-        if (advance) dyn[s].time += dt;
-        dyn[s].amax2_bits = 0u;
-    }
-    if (threadIdx.x == 0 && dt_host > 0.0) st->dt_next = 0.0;
-    if (threadIdx.x == 0 && advance) {
-        st->steps += 1ull;
-        if (rebuild_every > 1) {
-            // skin list: rebuild when a particle has moved skin/4 (the predicted state of
-            // the step then stays within skin/2: a CFL step moves less than 0.3 h) or after
-            // rebuild_every steps
-            const bool rb = st->since >= rebuild_every || __uint_as_float(st->maxdisp2_bits) > trig2;
-            st->rebuild = rb ? 1u : 0u;
-            st->since = rb ? 1u : st->since + 1u;
-            if (rb) st->maxdisp2_bits = 0u;
-            st->builds += rb ? 1u : 0u;
-        } else {
-            st->builds += builds_inc;
-        }
-    }
-}
-
 // the CFL dt the next step of scene 0 would take, without changing any state
 __global__ void k_dt_peek(const SceneDev* __restrict__ scenes, const SceneDyn* __restrict__ dyn,
                           DevStatus* __restrict__ st, double h, double cfl, double dt_fixed) {
     if (threadIdx.x == 0) st->dt_peek = cfl_dt_of(scenes[0], dyn[0], h, cfl, dt_fixed);
 }
 
-__global__ void k_dt(const SceneDev* __restrict__ scenes, SceneDyn* __restrict__ dyn, DevStatus* __restrict__ st,
-                     uint32_t n_scenes, double h, double cfl, double dt_fixed, int advance, uint32_t rebuild_every,
-                     float trig2, uint32_t builds_inc) {
-    dt_body(scenes, dyn, st, n_scenes, h, cfl, dt_fixed, advance, rebuild_every, trig2, builds_inc);
-}
+__global__ void k_dt(const DtArgs a) { dt_body(a); }
 
 // ---------------------------------------------------------------------
 // The neighbour build and the predictor pass in one kernel: each thread writes
@@ -617,8 +570,7 @@ __global__ void __launch_bounds__(kPipeBlock, kPersistMinBlocks) k_step_persiste
     for (uint32_t s = 0; s < nsteps; ++s) {
         const int cur = (cur0 + (int)s) & 1, nxt = cur ^ 1;
         if (blockIdx.x == 0)
-            dt_body(b.scenes, b.dyn, b.status, g.n_scenes, ph.h_d, ph.cfl, ph.dt_fixed, 1, ph.rebuild_every,
-                    ph.skin_trig2, 1u);
+            dt_body(dt_args(b, g, ph, 1, 1));
         hash_body(b.pos[cur], b.cell[cur], b.pinfo[cur], b.scenes, b.status, b.key, b.slot, b.count, g.n_cells);
         grid.sync();
         for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) scan_reduce_tile(b.count, nb, b.bsum, t);
@@ -630,7 +582,7 @@ __global__ void __launch_bounds__(kPipeBlock, kPersistMinBlocks) k_step_persiste
         grid.sync();
         scatter_body(b.key, b.slot, b.start, b.status, b.unsorted, nb);
         grid.sync();
-        reorder_body(b.pos[cur], b.vel[cur], b.phat[cur], b.pinfo[cur], b.pid[cur], b.start, b.unsorted, b.scenes,
+        reorder_body<kReorderCells>(b.pos[cur], b.vel[cur], b.phat[cur], b.pinfo[cur], b.pid[cur], b.start, b.unsorted, b.scenes,
                      g.n_cells, b.status, b.cell_nfluid, b.pos[nxt], b.vel[nxt], b.phat[nxt], b.cell[nxt],
                      b.pinfo[nxt], b.pid[nxt], b.quads);
         grid.sync();
@@ -777,8 +729,7 @@ const char* forces_variant_name(int v) {
 
 void launch_dt(const Buffers& b, const Geometry& g, const Phys& ph, int advance_time, cudaStream_t st,
                int with_build) {
-    k_dt<<<1, 256, 0, st>>>(b.scenes, b.dyn, b.status, g.n_scenes, ph.h_d, ph.cfl, ph.dt_fixed, advance_time,
-                            ph.rebuild_every, ph.skin_trig2, with_build ? 1u : 0u);
+    k_dt<<<1, 256, 0, st>>>(dt_args(b, g, ph, advance_time, with_build));
 }
 
 // blocks of the persistent step kernel: all resident (a cooperative launch refuses more)

@@ -18,6 +18,50 @@ constexpr int kScanItems = 8;                       // per thread
 constexpr int kScanTile = kScanThreads * kScanItems;  // buckets per block
 
 // ---------------------------------------------------------------------
+// dt.  The CFL time step of a scene from the largest |a|^2 of the last reduction (reading C7)
+__device__ __forceinline__ double cfl_dt_of(const SceneDev& sc, const SceneDyn& d, double h, double cfl,
+                                            double dt_fixed) {
+    if (dt_fixed > 0.0) return dt_fixed;
+    double dt = sc.dt_cap;
+    const double a2 = (double)__uint_as_float(d.amax2_bits);
+    if (a2 > 0.0) dt = fmin(dt, cfl * sqrt(h / sqrt(a2)));
+    return dt;
+}
+
+// One block, a thread per scene: dt for the coming step (reading C7), simulated
+// time, reset of the |a|^2 accumulator.
+__device__ __forceinline__ void dt_body(const DtArgs& a) {
+    const SceneDev* __restrict__ scenes = a.scenes;
+    SceneDyn* __restrict__ dyn = a.dyn;
+    DevStatus* __restrict__ st = a.st;
+    const double dt_host = st->dt_next;  // the host's time step for this step (sph_set_dt), or <= 0
+    __syncthreads();
+    for (uint32_t s = threadIdx.x; s < a.n_scenes; s += blockDim.x) {
+        const double dt = dt_host > 0.0 ? dt_host : cfl_dt_of(scenes[s], dyn[s], a.h, a.cfl, a.dt_fixed);
+        dyn[s].dt = (float)dt;
+        dyn[s].dt_d = dt;
+        if (a.advance) dyn[s].time += dt;
+        dyn[s].amax2_bits = 0u;
+    }
+    if (threadIdx.x == 0 && dt_host > 0.0) st->dt_next = 0.0;
+    if (threadIdx.x == 0 && a.advance) {
+        st->steps += 1ull;
+        if (a.rebuild_every > 1) {
+            // skin list: rebuild when a particle has moved skin/4 (the predicted state of
+            // the step then stays within skin/2: a CFL step moves less than 0.3 h) or after
+            // a.rebuild_every steps
+            const bool rb = st->since >= a.rebuild_every || __uint_as_float(st->maxdisp2_bits) > a.trig2;
+            st->rebuild = rb ? 1u : 0u;
+            st->since = rb ? 1u : st->since + 1u;
+            if (rb) st->maxdisp2_bits = 0u;
+            st->builds += rb ? 1u : 0u;
+        } else {
+            st->builds += a.builds_inc;
+        }
+    }
+}
+
+// ---------------------------------------------------------------------
 // a1: cell hash.  New cell = old cell + floor(offset/cell + 1/2) per axis
 // (cell-relative positions never leave FP32 range); periodic axes wrap;
 // on other axes a particle outside the grid goes to the sentinel bucket
@@ -162,6 +206,41 @@ __device__ __forceinline__ void scan_down_tile(uint32_t* __restrict__ count, uin
     }
 }
 
+// the whole scan by one block of 1024 threads, for few buckets
+constexpr uint32_t kScanOneMax = 24576;
+
+__device__ __forceinline__ void scan_one_body(uint32_t* __restrict__ count, uint32_t nb, uint32_t* __restrict__ start,
+                                              DevStatus* __restrict__ st) {
+    uint32_t carry = 0;
+    for (uint32_t base0 = 0; base0 < nb; base0 += blockDim.x * kScanItems) {
+        const uint32_t base = base0 + threadIdx.x * kScanItems;
+        uint32_t v[kScanItems];
+        uint32_t s = 0;
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k) {
+            v[k] = base + k < nb ? count[base + k] : 0u;
+            s += v[k];
+        }
+        uint32_t total;
+        uint32_t run = block_excl_scan(s, &total) + carry;
+        carry += total;
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k) {
+            const uint32_t b = base + k;
+            if (b < nb) {
+                start[b] = run;
+                count[b] = 0u;
+                if (b == nb - 1) {  // the sentinel of removed particles
+                    start[nb] = run + v[k];
+                    st->n_sorted = run;
+                    st->n_removed += v[k];
+                }
+            }
+            run += v[k];
+        }
+    }
+}
+
 // ---------------------------------------------------------------------
 // a2: scatter particle indices to their bucket slots (order within a
 // bucket is the atomics' order; the reorder fixes it).
@@ -189,11 +268,15 @@ __device__ __forceinline__ uint32_t sort_key(const float4* pos, const uint32_t* 
     return (bnd << 31) | pid[idx];
 }
 
-// cells per warp: 4 measured fastest (1.65M dam break, most cells empty: 78 -> 61 us;
-// 2.1M box, no empty cell: unchanged at 56 us; 8 and 16 cells per warp leave too few warps)
+// cells per warp: 4 measured fastest on large grids (1.65M dam break, most cells empty: 78 -> 61 us;
+// 2.1M box, no empty cell: unchanged at 56 us; 8 and 16 cells per warp leave too few warps); 1 on
+// grids of up to kReorderOneMax cells, whose warps are too few to hide a cell's chain of loads (216
+// cells 8.6 -> 2.5 us, 4,116 cells 8.6 -> 4.5 us)
 constexpr int kReorderCells = 4;
 static_assert(kReorderCells >= 1 && kReorderCells <= 32, "one lane per cell");
+constexpr uint32_t kReorderOneMax = 32768;
 
+template <int kCells>
 __device__ __forceinline__ void reorder_body(
     const float4* __restrict__ pos, const float4* __restrict__ vel, const float* __restrict__ phat,
     const uint32_t* __restrict__ pinfo,
@@ -209,11 +292,11 @@ __device__ __forceinline__ void reorder_body(
         st->n_active = st->n_sorted;
         st->max_neibs_seen = 0u;
     }
-    // kReorderCells consecutive cells per warp: their ranges in one load, empty cells
+    // kCells consecutive cells per warp: their ranges in one load, empty cells
     // (most of a tank's cells) skipped without a round trip each
-    for (uint32_t c0 = warp * kReorderCells; c0 < n_cells; c0 += nwarps * kReorderCells) {
+    for (uint32_t c0 = warp * kCells; c0 < n_cells; c0 += nwarps * kCells) {
         const uint32_t cl = c0 + (uint32_t)lane;
-        const bool own = lane < kReorderCells && cl < n_cells;
+        const bool own = lane < kCells && cl < n_cells;
         const uint32_t b_l = own ? start[cl] : 0u, e_l = own ? start[cl + 1] : 0u;
         if (own && e_l == b_l) cell_nfluid[cl] = 0u;
         unsigned todo = __ballot_sync(0xffffffffu, e_l > b_l);

@@ -515,9 +515,9 @@ int set_scene_table(sph_ctx* c, uint32_t n, const sph_scene* sc) {
 }
 
 // neighbour pipeline on buffer `cur` -> buffer cur^1 (sorted), then list
-void enqueue_sort(sph_ctx* c, cudaStream_t st) {
+void enqueue_sort(sph_ctx* c, const DtArgs* dt, cudaStream_t st) {
     launch_hash(c->b, c->cur, c->g, st);
-    launch_scan(c->b, c->g, st);
+    launch_scan(c->b, c->g, dt, st);
     launch_scatter(c->b, c->g, st);
     launch_reorder(c->b, c->cur, c->g, st);
     c->cur ^= 1;
@@ -527,14 +527,14 @@ void enqueue_build(sph_ctx* c, cudaStream_t st) {
     if (skin_mode(c)) {
         // gated by status->rebuild; the sorted arrays come back to the same buffer
         launch_hash(c->b, c->cur, c->g, st);
-        launch_scan(c->b, c->g, st);
+        launch_scan(c->b, c->g, nullptr, st);
         launch_scatter(c->b, c->g, st);
         launch_reorder(c->b, c->cur, c->g, st);
         launch_copyback(c->b, c->cur, c->g, st);
         launch_build(c->b, c->cur, c->g, c->ph, st);
         return;
     }
-    enqueue_sort(c, st);
+    enqueue_sort(c, nullptr, st);
     launch_build(c->b, c->cur, c->g, c->ph, st);
 }
 
@@ -551,12 +551,13 @@ void enqueue_build_predict(sph_ctx* c, const Phys& ph, cudaStream_t st) {
 }
 
 void enqueue_step(sph_ctx* c, cudaStream_t st) {
-    launch_dt(c->b, c->g, c->ph, 1, st);  // (skin list: decides whether the pipeline runs)
     if (skin_mode(c)) {
+        launch_dt(c->b, c->g, c->ph, 1, st);  // decides whether the pipeline runs
         enqueue_build(c, st);
         launch_forces(c->b, c->cur, c->g, c->ph, kPredict, 0, st);
     } else {
-        enqueue_sort(c, st);
+        const DtArgs dt = dt_args(c->b, c->g, c->ph, 1, 1);  // computed beside the scan
+        enqueue_sort(c, &dt, st);
         enqueue_build_predict(c, c->ph, st);
     }
     launch_forces(c->b, c->cur, c->g, c->ph, kCorrect, 0, st);
@@ -1254,8 +1255,8 @@ Buffers with_list_slot(const sph_ctx* c, char* slot) {
 // one forward step with the frozen dt; optionally tape the sorted and predicted states, and
 // build the step's list into a list slot of the tape (else into the context's list)
 void rec_step(sph_ctx* c, const Phys& ph, char* tape_blk, int advance, cudaStream_t st, char* list_slot = nullptr) {
-    launch_dt(c->b, c->g, ph, advance, st);
-    enqueue_sort(c, st);
+    const DtArgs dt = dt_args(c->b, c->g, ph, advance, 1);
+    enqueue_sort(c, &dt, st);
     const Buffers bb = with_list_slot(c, list_slot);
     launch_build(bb, c->cur, c->g, ph, st);
     launch_forces(bb, c->cur, c->g, ph, kPredict, 0, st);
@@ -1478,11 +1479,12 @@ int sph_step_profiled(sph_ctx* c, uint32_t nsteps, void* stream, double* phase_m
     int rc = SPH_OK;
     for (uint32_t s = 0; s < nsteps && rc == SPH_OK; ++s) {
         cudaEventRecord(ev[0], st);
-        launch_dt(c->b, c->g, c->ph, 1, st);
+        const DtArgs dt = dt_args(c->b, c->g, c->ph, 1, 1);
+        if (skin_mode(c)) launch_dt(c->b, c->g, c->ph, 1, st);  // (else beside the scan)
         cudaEventRecord(ev[1], st);
         launch_hash(c->b, c->cur, c->g, st);
         cudaEventRecord(ev[2], st);
-        launch_scan(c->b, c->g, st);
+        launch_scan(c->b, c->g, skin_mode(c) ? nullptr : &dt, st);
         cudaEventRecord(ev[3], st);
         launch_scatter(c->b, c->g, st);
         cudaEventRecord(ev[4], st);

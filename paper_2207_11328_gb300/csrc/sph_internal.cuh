@@ -284,9 +284,28 @@ struct Geometry {
     uint32_t n_scenes;
 };
 
+// arguments of the time-step update (dt_body, pipeline.cuh)
+struct DtArgs {
+    const SceneDev* scenes;
+    SceneDyn* dyn;
+    DevStatus* st;
+    uint32_t n_scenes;
+    double h, cfl, dt_fixed;
+    int advance;             // the step counts and the simulated time moves
+    uint32_t rebuild_every;
+    float trig2;
+    uint32_t builds_inc;
+};
+__host__ __device__ inline DtArgs dt_args(const Buffers& b, const Geometry& g, const Phys& ph, int advance,
+                                          int with_build) {
+    return DtArgs{b.scenes, b.dyn, b.status, g.n_scenes, ph.h_d, ph.cfl, ph.dt_fixed, advance, ph.rebuild_every,
+                  ph.skin_trig2, with_build ? 1u : 0u};
+}
+
 // neighbours.cu
 void launch_hash(const Buffers& b, int cur, const Geometry& g, cudaStream_t st);
-void launch_scan(const Buffers& b, const Geometry& g, cudaStream_t st);
+// dt: the step's time-step update too, by a block of its own (every-step lists), else null
+void launch_scan(const Buffers& b, const Geometry& g, const DtArgs* dt, cudaStream_t st);
 void launch_scatter(const Buffers& b, const Geometry& g, cudaStream_t st);
 void launch_reorder(const Buffers& b, int cur, const Geometry& g, cudaStream_t st);
 void launch_build(const Buffers& b, int cur, const Geometry& g, const Phys& ph, cudaStream_t st);
