@@ -16,6 +16,7 @@
 //
 // Adjoint layout per particle, sorted order of the step:
 //   xb4 = (xbar, deltabar), ub4 = (ubar, alphabar partial), seed4 = (abar, drhobar).
+#include "packed.cuh"
 #include "sph_internal.cuh"
 
 namespace sphg {
@@ -160,10 +161,10 @@ template <int VISC>
 __device__ __forceinline__ PairGrad2 pair_grad2(const PairIn2& p, const Phys& ph, float pic, float pic_unit) {
     PairGrad2 g;
     const float r2 = fmaxf(p.r2, 1e-30f);
-    const float r = r2 * rsqrtf(r2);
-    const float t = fminf(fmaf(r, ph.inv_h, -2.0f), 0.0f);
+    const float rinv = rsqrt_fast(r2);
+    const float t = fminf(fmaf(r2 * rinv, ph.inv_h, -2.0f), 0.0f);
     const float F = ph.aF * t * t * t;
-    const float Fr = 3.0f * ph.aF * t * t * ph.inv_h / r;  // (dF/dr)/r
+    const float Fr = 3.0f * ph.aF * t * t * ph.inv_h * rinv;  // (dF/dr)/r
     const float w = fmaf(p.ux, p.rx, fmaf(p.uy, p.ry, p.uz * p.rz));
     const float sa = fmaf(p.Ak.x, p.rx, fmaf(p.Ak.y, p.ry, p.Ak.z * p.rz));      // abar_k . x_kj
     const float sb = -fmaf(p.Aj.x, p.rx, fmaf(p.Aj.y, p.ry, p.Aj.z * p.rz));     // abar_j . x_jk
@@ -171,17 +172,17 @@ __device__ __forceinline__ PairGrad2 pair_grad2(const PairIn2& p, const Phys& ph
     if (VISC == SPH_VISC_ARTIFICIAL && w < 0.f) {
         const float E = fmaf(0.5f, p.dk + p.dj, 1.0f);
         const float D = r2 + ph.eps_h2;
-        const float inv = 1.0f / (D * E);
+        const float inv = rcp_fast(D * E);  // 1/D = inv E, 1/E = inv D
         Pi = -pic * w * inv;
         const float k = -pic * inv;             // dPi/du_kj = k x ; dPi/dx_kj = k (u - 2 w x / D)
-        const float c2 = 2.0f * w / D;
+        const float c2 = 2.0f * w * (inv * E);
         dPx = k * (p.ux - c2 * p.rx);
         dPy = k * (p.uy - c2 * p.ry);
         dPz = k * (p.uz - c2 * p.rz);
         dPux = k * p.rx;
         dPuy = k * p.ry;
         dPuz = k * p.rz;
-        dPd = -0.5f * Pi / E;                    // dPi/d delta_k = dPi/d delta_j
+        dPd = -0.5f * Pi * (inv * D);                    // dPi/d delta_k = dPi/d delta_j
         dPa = -pic_unit * w * inv;               // dPi/d alpha
     }
     const float S = p.phk + p.phj + Pi;
@@ -201,7 +202,7 @@ __device__ __forceinline__ PairGrad2 pair_grad2(const PairIn2& p, const Phys& ph
     g.ga = sFma * dPa;
     if (VISC == SPH_VISC_LAMINAR) {
         // a_kj += lam m_j F u_kj / (2 + d_k + d_j), lam = 4 nu / rho0 (and a_jk likewise with m_k)
-        const float inv2 = 1.0f / (2.0f + p.dk + p.dj);
+        const float inv2 = rcp_fast(2.0f + p.dk + p.dj);
         const float lam = ph.nu4 * ph.inv_rho0 * inv2;
         const float Aua = fmaf(p.Ak.x, p.ux, fmaf(p.Ak.y, p.uy, p.Ak.z * p.uz));
         const float Aub = -fmaf(p.Aj.x, p.ux, fmaf(p.Aj.y, p.uy, p.Aj.z * p.uz));
@@ -258,9 +259,14 @@ __global__ void __launch_bounds__(kBlock, 7) k_adj_vjp(
         const uint32_t cnt = ncount[k];
         const uint32_t nf = cnt & 0xffffu, nb = cnt >> 16;
         float gx = 0.f, gy = 0.f, gz = 0.f, gux = 0.f, guy = 0.f, guz = 0.f, gd = 0.f, ga = 0.f;
+        auto entry = [&](uint32_t q) -> uint32_t {
+            return nlist[q < nf ? list_fluid_word(q, k, ph.stride)
+                                : list_bnd_word(q - nf, k, ph.stride, ph.max_neibs)];
+        };
+        uint32_t next = sub < nf + nb ? entry(sub) : 0u;
         for (uint32_t q = sub; q < nf + nb; q += LANES) {
-            const uint32_t e = nlist[q < nf ? list_fluid_word(q, k, ph.stride)
-                                            : list_bnd_word(q - nf, k, ph.stride, ph.max_neibs)];
+            const uint32_t e = next;
+            if (q + LANES < nf + nb) next = entry(q + LANES);  // one round ahead of its gathers
             const uint32_t j = e >> kCodeBits;
             SPH_GUARD(j < st->n_active, st, continue)
             const float4 pj = pos[j];
@@ -418,8 +424,12 @@ void launch_adj_vjps(const AdjBuffers& a, const Buffers& b, int cur, const Geome
 template <int VISC>
 void launch_adj_vjps_v(const AdjBuffers& a, const Buffers& b, int cur, const Geometry& g, const Phys& ph, float dt,
                        cudaStream_t st) {
-    // lanes per particle: enough threads to fill the GPU (~150k resident) on small states
-    if (g.cap <= (1u << 16))
+    // lanes per particle: enough threads to fill the GPU (~150k resident) on small states (backward
+    // pass with 8 / 4 / 2 lanes, ms: 26,082 particles and 16 steps 2.13 / 2.24 / 2.46, 32,768 and 64
+    // steps 8.47 / 8.34 / 9.02)
+    if (g.cap <= 28672u)
+        launch_adj_vjps<VISC, 8>(a, b, cur, g, ph, dt, st);
+    else if (g.cap <= (1u << 16))
         launch_adj_vjps<VISC, 4>(a, b, cur, g, ph, dt, st);
     else if (g.cap <= (1u << 18))
         launch_adj_vjps<VISC, 2>(a, b, cur, g, ph, dt, st);
