@@ -538,7 +538,9 @@ void enqueue_build(sph_ctx* c, cudaStream_t st) {
     launch_build(c->b, c->cur, c->g, c->ph, st);
 }
 
-inline bool can_fuse(const sph_ctx* c) { return !skin_mode(c) && !c->ph.general; }
+// the default model: what the fused, persistent and differentiable runs take
+inline bool default_model(const sph_ctx* c) { return !c->ph.general && c->ph.ddiff == SPH_DDIFF_NONE; }
+inline bool can_fuse(const sph_ctx* c) { return !skin_mode(c) && default_model(c); }
 
 // the list build and the predictor pass (one kernel when fused)
 void enqueue_build_predict(sph_ctx* c, const Phys& ph, cudaStream_t st) {
@@ -741,7 +743,6 @@ int sph_create(const sph_params* p, sph_ctx** out) {
     ph.visc_avg = p->visc_avg;
     ph.ddiff = p->ddiff;
     ph.general = !(p->kernel_type == SPH_KERNEL_WENDLAND && p->formulation == SPH_FORM_1 &&
-                   p->ddiff == SPH_DDIFF_NONE &&
                    (p->visc_model == SPH_VISC_ARTIFICIAL ||
                     (p->visc_model == SPH_VISC_MORRIS && p->visc_avg == SPH_AVG_HARMONIC)));
     // laminar models as (lam_u u_ij + lam_x (u.x/r^2) x_ij) m_j f avg(r_i,r_j)/(r_i r_j):
@@ -1014,7 +1015,7 @@ int sph_get_step_options(sph_ctx* c, int* fused_predict, int* persistent) {
 
 int sph_set_persistent(sph_ctx* c, int on) {
     if (!c) return SPH_ERR_ARG;
-    if (on && (skin_mode(c) || c->ph.general)) return SPH_ERR_ARG;
+    if (on && (skin_mode(c) || !default_model(c))) return SPH_ERR_ARG;
     CK(cudaDeviceSynchronize());
     drop_graphs(c);
     c->persistent = on != 0;
@@ -1340,7 +1341,7 @@ int sph_record(sph_ctx* c, uint32_t T, uint32_t K, void* stream, double* dt_out)
     if (!c || T == 0 || K == 0 || T % K != 0) return SPH_ERR_ARG;
     if (!c->uploaded) return SPH_ERR_STATE;
     // one scene, list rebuilt every step, default model options
-    if (c->g.n_scenes != 1 || skin_mode(c) || c->ph.general) return SPH_ERR_ARG;
+    if (c->g.n_scenes != 1 || skin_mode(c) || !default_model(c)) return SPH_ERR_ARG;
     cudaStream_t st = S(stream);
     AdjTape& t = c->tape;
     t.valid = false;

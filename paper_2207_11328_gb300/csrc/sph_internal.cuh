@@ -161,7 +161,8 @@ struct Phys {
                              //   forces_variant_name
     int forces_variant_c;    // launch shape of the corrector pass (autotuned on its own)
     int fuse_predict;        // the list build and the predictor pass as one kernel (autotuned)
-    // model options (Table 1); general != 0 selects the kernels of forces_models.cu
+    // model options (Table 1); general != 0 selects the kernels of forces_models.cu (density
+    // diffusion alone does not)
     int general;
     int kernel_type;         // SPH_KERNEL_*: F = aF f(q)
     int form;                // SPH_FORM_*

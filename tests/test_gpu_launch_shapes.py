@@ -7,8 +7,9 @@ import dataclasses
 import numpy as np
 import pytest
 
+import oracle
 from paper_2207_11328_gb300 import N_BUILD_VARIANTS, N_FORCES_VARIANTS, scenes
-from tests.gpu_common import compare_neighbor_sets, require_gpu, sim_for
+from tests.gpu_common import compare_neighbor_sets, rel_check, require_gpu, sim_for
 
 pytestmark = pytest.mark.gpu
 
@@ -76,6 +77,38 @@ def test_every_build_cuts_a_full_list_at_the_same_entry(max_neibs):
         assert st["rc"] == -4
         got = (*sim.download_neighbors(), np.array([st["max_neibs_seen"], st["list_entries"]]))
         assert (got[0].sum(1) <= max_neibs).all()
+        if ref is None:
+            ref = got
+        for a, b in zip(got, ref):
+            assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("visc", [0, 1])
+@pytest.mark.parametrize("skin", [0.0, 0.3])
+@pytest.mark.parametrize("walls", [False, True])
+def test_density_diffusion_in_every_shape_matches_the_oracle(visc, skin, walls):
+    # the default kernel, formulation and viscosities with density diffusion
+    if walls:
+        s = scenes.dam_break(dp=0.04)
+        f = s.ptype == 0
+        s.vel[f] = scenes.seeded_normal((int(f.sum()), 3), 0.05, 5).astype(np.float32)
+    else:
+        s = scenes.periodic_box(n_per_axis=12, jitter=0.2, seed=6)
+        s.delta = np.random.default_rng(7).uniform(-1e-3, 1e-3, s.n).astype(np.float32)
+    s = dataclasses.replace(s, visc=visc, nu=1e-3 if visc else 0.0, ddiff=1, ddiff_coef=0.1)
+    kw = dict(rebuild_every=10, skin=skin * s.h, max_neibs=224) if skin else {}
+    a_ref, d_ref, mag = oracle.rhs(oracle.params(s), s.pos, s.vel, s.delta, s.mass, s.ptype, with_mag=True)
+    ref = None
+    for v in range(N_FORCES_VARIANTS):
+        sim = sim_for(s, **kw)
+        sim.set_variants(forces=v)
+        sim.forces()
+        acc, drho = sim.download_forces()
+        rel_check(acc, a_ref, 1e-5, "acceleration", mag[:, 0])
+        rel_check(drho, d_ref, 1e-5, "density rate", mag[:, 1])
+        sim.step(3)
+        got = (acc, drho, *sim.download())
+        assert sim.stats()["error_bits"] == 0
         if ref is None:
             ref = got
         for a, b in zip(got, ref):
