@@ -332,9 +332,8 @@ int sph_tape_generation(sph_ctx* ctx, uint64_t* gen);
  * per block, or nine warps per 32 particles, a warp per row of neighbour
  * cells, with 2, 3 or 4 blocks per SM) and each
  * force-kernel shape (64, 128 or 256 threads per block with at most 64
- * registers; 4 or 8 lanes per particle, on a skin list 128 threads with at
- * most 85 or 128 registers) on the uploaded state (warps per row and lanes
- * per particle up to 131,072 particles), the
+ * registers; 4 or 8 lanes per particle) on the uploaded state (warps per row
+ * and lanes per particle up to 131,072 particles), the
  * predictor and the corrector pass apart (3 timed launches each, CUDA events
  * on `stream`; the corrector runs on a scratch copy of the state), then the
  * list build and the predictor pass fused against apart (every-step list,

@@ -33,11 +33,8 @@ namespace {
 // One neighbour of a fluid particle.  BND: the neighbour is a boundary
 // particle (mass stored negated, velocity zero).  The kernel constant aF is
 // factored out of every term (all terms are linear in F) and applied once.
-// RECOMP: P_j/rho_j^2 from delta_j (the function that stores the per-particle
-// value, so bit-identical to it) in place of a third gather.  Faster in every
-// pass over the pairs within the cutoff; slower in the passes that filter a
-// skin list (more registers live beside the exact-list writers), which keep
-// the gather.
+// P_j/rho_j^2 comes from delta_j (the function that stores the per-particle
+// value, so bit-identical to it) in place of a third gather.
 // The pair's terms go to `out` as they are formed: the running sums (Acc), or their values
 // (Terms), for a group of lanes that adds its lanes' terms in list order.
 __device__ __forceinline__ void add_rate(Acc& a, float mF, float udx) { a.drho = fmaf(mF, udx, a.drho); }
@@ -88,24 +85,18 @@ __host__ __device__ constexpr bool is_artificial(int v) { return (v & ~kDiffusio
 __host__ __device__ constexpr bool is_laminar(int v) { return (v & ~kDiffusion) == SPH_VISC_LAMINAR; }
 __host__ __device__ constexpr bool has_diffusion(int v) { return (v & kDiffusion) != 0; }
 
-template <int VISC, bool BND, bool FILTER, bool RECOMP, class Out>
-__device__ __forceinline__ bool fluid_pair(uint32_t e, const Central& ci, const float4& vi, float phat_i,
+template <int VISC, bool BND, class Out>
+__device__ __forceinline__ void fluid_pair(uint32_t e, const Central& ci, const float4& vi, float phat_i,
                                            const float4* __restrict__ pos, const float4* __restrict__ vel,
-                                           const float* __restrict__ phat, float phat_coef, float pi_coef,
-                                           float dd_coef, const Phys& ph, Out& out, uint32_t& npairs) {
+                                           float phat_coef, float pi_coef, float dd_coef, const Phys& ph, Out& out) {
     const uint32_t j = e >> kCodeBits;
     const float4 pj = pos[j];
-    const float4 vj = vel[j];  // all gathers issued together
-    const float phat_j = RECOMP ? eos_phat(vj.w, ph, phat_coef) : phat[j];
+    const float4 vj = vel[j];  // both gathers issued together
+    const float phat_j = eos_phat(vj.w, ph, phat_coef);
     const float rx = pick(e, ci.xm, ci.x0, ci.xp) - pj.x;
     const float ry = pick(e >> 2, ci.ym, ci.y0, ci.yp) - pj.y;
     const float rz = pick(e >> 4, ci.zm, ci.z0, ci.zp) - pj.z;
     const float r2 = fmaxf(fmaf(rx, rx, fmaf(ry, ry, rz * rz)), 1e-30f);
-    if (FILTER) {
-        // list with a skin: pairs beyond the influence radius (F = 0) skip the arithmetic
-        if (!(r2 < ph.R2)) return false;
-        ++npairs;
-    }
     const float r = r2 * rsqrtf(r2);
     const float t = fminf(fmaf(r, ph.inv_h, -2.0f), 0.0f);
     const float mj = BND ? -pj.w : pj.w;
@@ -125,12 +116,11 @@ __device__ __forceinline__ bool fluid_pair(uint32_t e, const Central& ci, const 
     add_force(out, mF * bracket, rx, ry, rz);
     if (is_laminar(VISC))
         add_laminar(out, ph.nu4 * ph.inv_rho0 * __fdividef(mF, 2.0f + vi.w + vj.w), ux, uy, uz);
-    return true;
 }
 
 // one fluid neighbour of a boundary particle: continuity, u_i = 0
-template <bool FILTER, class Out>
-__device__ __forceinline__ bool boundary_pair(uint32_t e, const Central& ci, const float4* __restrict__ pos,
+template <class Out>
+__device__ __forceinline__ void boundary_pair(uint32_t e, const Central& ci, const float4* __restrict__ pos,
                                               const float4* __restrict__ vel, const Phys& ph, Out& out) {
     const uint32_t j = e >> kCodeBits;
     const float4 pj = pos[j];
@@ -139,14 +129,12 @@ __device__ __forceinline__ bool boundary_pair(uint32_t e, const Central& ci, con
     const float ry = pick(e >> 2, ci.ym, ci.y0, ci.yp) - pj.y;
     const float rz = pick(e >> 4, ci.zm, ci.z0, ci.zp) - pj.z;
     const float r2 = fmaxf(fmaf(rx, rx, fmaf(ry, ry, rz * rz)), 1e-30f);
-    if (FILTER && !(r2 < ph.R2)) return false;
     const float r = r2 * rsqrtf(r2);
     const float t = fminf(fmaf(r, ph.inv_h, -2.0f), 0.0f);
     add_rate(out, pj.w * (t * t * t), -fmaf(vj.x, rx, fmaf(vj.y, ry, vj.z * rz)));
-    return true;
 }
 
-// A part of a particle's every-step list by LANES consecutive lanes of a warp: each lane evaluates
+// A part of a particle's list by LANES consecutive lanes of a warp: each lane evaluates
 // every LANES-th entry's terms, then all lanes add the group's terms in list order, so the sums are
 // those of one thread, to the bit (the terms travel by shuffles: 6 a pair and lane).  For states too
 // small to fill the GPU with a thread per particle, where one thread's list is a long chain of
@@ -195,12 +183,6 @@ __device__ __forceinline__ void lanes_sum(const uint2* __restrict__ lp, ptrdiff_
     }
 }
 
-// SKIN: the list carries a skin (rebuild every k steps).  The predictor pass
-// (and sph_forces) skip pairs beyond the cutoff and count the pairs within it;
-// the predictor also writes those pairs, the step's exact list, to
-// nlist_x/ncount_x (same split layout), which the corrector pass reads as its
-// list (so both passes use the pairs within R at x^n, as with a list built
-// every step) before checking the displacement since the build.
 // (the forces-only pass keeps the |a|^2 reduction for dt0 live beside the sums: it gets
 // a looser register cap than the step's passes, so that no shape spills)
 // One particle of a force pass (one iteration of the pass's particle loop): its pair sums
@@ -221,20 +203,16 @@ __device__ __forceinline__ uint2 ld_chunk(const uint2* p) {
     return v;
 }
 
+// SKIN: nlist/ncount are the step's exact list in its four-entry chunks; the corrector also checks
+// and reduces the displacement since the list's build.
 template <int VISC, int MODE, bool SKIN, bool FRESH = false, int LANES = 1>
 __device__ __forceinline__ void particle_pass(
     uint32_t i, uint32_t n, const float4* __restrict__ pos, const float4* __restrict__ vel,
     const float* __restrict__ phat, float4* io_pos, float4* io_vel, float* io_phat, float4* __restrict__ force_out,
     const uint32_t* __restrict__ pinfo, const uint32_t* __restrict__ nlist, const uint32_t* __restrict__ ncount,
     const SceneDev* __restrict__ scenes, SceneDyn* __restrict__ dyn, DevStatus* __restrict__ st, const Phys& ph,
-    int acc_dt, const float4* __restrict__ pos_ref, uint32_t* __restrict__ nlist_x,
-    uint32_t* __restrict__ ncount_x, const uint32_t* __restrict__ pid, uint32_t& npairs, uint32_t cnt_fresh = 0) {
-    static_assert(LANES == 1 || !(SKIN || FRESH), "a group of lanes takes an every-step list");
-    static_assert(!(FRESH && SKIN), "a list written in the same kernel is a list built at this step");
-    constexpr bool FILTER = SKIN && MODE != kCorrect;
-    constexpr bool COMPACT = SKIN && MODE == kPredict;
-    constexpr bool CHUNKED = SKIN && MODE == kCorrect;  // nlist/ncount: the exact list in chunks
-    constexpr bool RECOMP = !FILTER;  // P_j/rho_j^2 recomputed (see fluid_pair)
+    int acc_dt, const float4* __restrict__ pos_ref, const uint32_t* __restrict__ pid, uint32_t cnt_fresh = 0) {
+    static_assert(LANES == 1 || !(FRESH || SKIN), "a group of lanes takes an every-step list");
     const uint32_t s = pinfo[i];
     const SceneDev& sc = scenes[s];
     const float4 pi = pos[i];
@@ -246,9 +224,7 @@ __device__ __forceinline__ void particle_pass(
     const float cx = sc.cell_f[0], cy = sc.cell_f[1], cz = sc.cell_f[2];
     Acc acc{0.f, 0.f, 0.f, 0.f};
     const size_t S = ph.stride;
-    const uint32_t kxb = exact_bnd_chunk(ph.max_neibs);
-    ChunkWriter xf{make_uint4(0u, 0u, 0u, 0u), 0u, reinterpret_cast<uint4*>(nlist_x), S, i};
-    ChunkWriter xb{make_uint4(0u, 0u, 0u, 0u), 0u, reinterpret_cast<uint4*>(nlist_x) + (size_t)kxb * S, S, i};
+#define SPH_PAIR(BND, e, out) fluid_pair<VISC, BND>(e, ci, vi, phat_i, pos, vel, sc.phat_coef, pic, sc.dd_coef, ph, out)
     if (LANES > 1) {
         const float phat_i = phat[i];
         const float pic = sc.pi_coef;
@@ -256,26 +232,23 @@ __device__ __forceinline__ void particle_pass(
         const uint2* fl = reinterpret_cast<const uint2*>(nlist) + i;
         const uint2* bl = fl + (size_t)(list_chunks(ph.max_neibs) - 1u) * S;
         if (fluid_i) {
-            lanes_sum<VISC, LANES>(fl, (ptrdiff_t)S, nf, n, st, acc, [&](uint32_t e, Terms& tm) {
-                fluid_pair<VISC, false, false, RECOMP>(e, ci, vi, phat_i, pos, vel, phat, sc.phat_coef, pic, sc.dd_coef, ph, tm, npairs); });
-            lanes_sum<VISC, LANES>(bl, -(ptrdiff_t)S, nb, n, st, acc, [&](uint32_t e, Terms& tm) {
-                fluid_pair<VISC, true, false, RECOMP>(e, ci, vi, phat_i, pos, vel, phat, sc.phat_coef, pic, sc.dd_coef, ph, tm, npairs); });
+            lanes_sum<VISC, LANES>(fl, (ptrdiff_t)S, nf, n, st, acc, [&](uint32_t e, Terms& tm) { SPH_PAIR(false, e, tm); });
+            lanes_sum<VISC, LANES>(bl, -(ptrdiff_t)S, nb, n, st, acc, [&](uint32_t e, Terms& tm) { SPH_PAIR(true, e, tm); });
             acc.ax = fmaf(ph.aF, acc.ax, ph.g[0]);
             acc.ay = fmaf(ph.aF, acc.ay, ph.g[1]);
             acc.az = fmaf(ph.aF, acc.az, ph.g[2]);
         } else {
             lanes_sum<VISC, LANES>(fl, (ptrdiff_t)S, nf, n, st, acc, [&](uint32_t e, Terms& tm) {
-                boundary_pair<false>(e, ci, pos, vel, ph, tm); });
+                boundary_pair(e, ci, pos, vel, ph, tm); });
         }
         acc.drho *= ph.aF;
         if (threadIdx.x % LANES != 0) return;  // the first lane finishes the particle
-    } else if (fluid_i && CHUNKED) {
+    } else if (fluid_i && SKIN) {
         const float phat_i = phat[i];
         const float pic = sc.pi_coef;
         const Central ci = central_of(pi, cx, cy, cz);
         // full chunks: four pairs with no test between them (their gathers issue together);
         // then the last chunk of each part (1 to 3 entries, the rest kMarker)
-#define SPH_PAIR(BND, e) fluid_pair<VISC, BND, false, RECOMP>(e, ci, vi, phat_i, pos, vel, phat, sc.phat_coef, pic, sc.dd_coef, ph, acc, npairs)
 #define SPH_OK_E(e) (((e) >> kCodeBits) < n)
         const uint4* cp = reinterpret_cast<const uint4*>(nlist) + i;
         uint32_t k = 0;
@@ -285,37 +258,36 @@ __device__ __forceinline__ void particle_pass(
             const uint4 q = qn;
             if (k + 8 <= nf) qn = __ldg(cp + S);  // the next full chunk, one iteration ahead
             SPH_GUARD(SPH_OK_E(q.x) && SPH_OK_E(q.y) && SPH_OK_E(q.z) && SPH_OK_E(q.w), st, break)
-            SPH_PAIR(false, q.x);
-            SPH_PAIR(false, q.y);
-            SPH_PAIR(false, q.z);
-            SPH_PAIR(false, q.w);
+            SPH_PAIR(false, q.x, acc);
+            SPH_PAIR(false, q.y, acc);
+            SPH_PAIR(false, q.z, acc);
+            SPH_PAIR(false, q.w, acc);
         }
         do {
             if (k >= nf) break;
             const uint4 q = __ldg(cp);
             SPH_GUARD(SPH_OK_E(q.x) && (k + 1 >= nf || SPH_OK_E(q.y)) && (k + 2 >= nf || SPH_OK_E(q.z)), st, break)
-            SPH_PAIR(false, q.x);
-            if (k + 1 < nf) SPH_PAIR(false, q.y);
-            if (k + 2 < nf) SPH_PAIR(false, q.z);
+            SPH_PAIR(false, q.x, acc);
+            if (k + 1 < nf) SPH_PAIR(false, q.y, acc);
+            if (k + 2 < nf) SPH_PAIR(false, q.z, acc);
         } while (0);
-        cp = reinterpret_cast<const uint4*>(nlist) + (size_t)kxb * S + i;
+        cp = reinterpret_cast<const uint4*>(nlist) + (size_t)exact_bnd_chunk(ph.max_neibs) * S + i;
         for (k = 0; k + 4 <= nb; k += 4, cp += S) {
             const uint4 q = __ldg(cp);
             SPH_GUARD(SPH_OK_E(q.x) && SPH_OK_E(q.y) && SPH_OK_E(q.z) && SPH_OK_E(q.w), st, break)
-            SPH_PAIR(true, q.x);
-            SPH_PAIR(true, q.y);
-            SPH_PAIR(true, q.z);
-            SPH_PAIR(true, q.w);
+            SPH_PAIR(true, q.x, acc);
+            SPH_PAIR(true, q.y, acc);
+            SPH_PAIR(true, q.z, acc);
+            SPH_PAIR(true, q.w, acc);
         }
         do {
             if (k >= nb) break;
             const uint4 q = __ldg(cp);
             SPH_GUARD(SPH_OK_E(q.x) && (k + 1 >= nb || SPH_OK_E(q.y)) && (k + 2 >= nb || SPH_OK_E(q.z)), st, break)
-            SPH_PAIR(true, q.x);
-            if (k + 1 < nb) SPH_PAIR(true, q.y);
-            if (k + 2 < nb) SPH_PAIR(true, q.z);
+            SPH_PAIR(true, q.x, acc);
+            if (k + 1 < nb) SPH_PAIR(true, q.y, acc);
+            if (k + 2 < nb) SPH_PAIR(true, q.z, acc);
         } while (0);
-#undef SPH_PAIR
 #undef SPH_OK_E
         acc.ax = fmaf(ph.aF, acc.ax, ph.g[0]);
         acc.ay = fmaf(ph.aF, acc.ay, ph.g[1]);
@@ -329,9 +301,6 @@ __device__ __forceinline__ void particle_pass(
         // iteration ahead so that their latency is not on the path to the gathers
         const uint2* lp = reinterpret_cast<const uint2*>(nlist) + i;
         uint32_t k = 0;
-// keep a pair of the exact list (COMPACT only)
-#define SPH_KEEP_F(e) if (COMPACT) xf.put(e);
-#define SPH_KEEP_B(e) if (COMPACT) xb.put(e);
         uint2 an = make_uint2(0u, 0u), bn = make_uint2(0u, 0u);
         if (nf >= 4) {
             an = ld_chunk<FRESH>(lp);
@@ -344,25 +313,25 @@ __device__ __forceinline__ void particle_pass(
                 bn = ld_chunk<FRESH>(lp + 3 * S);
             }
             SPH_GUARD((max(max(a.x, a.y), max(b.x, b.y)) >> kCodeBits) < n, st, break)
-            if (fluid_pair<VISC, false, FILTER, RECOMP>(a.x, ci, vi, phat_i, pos, vel, phat, sc.phat_coef, pic, sc.dd_coef, ph, acc, npairs)) SPH_KEEP_F(a.x)
-            if (fluid_pair<VISC, false, FILTER, RECOMP>(a.y, ci, vi, phat_i, pos, vel, phat, sc.phat_coef, pic, sc.dd_coef, ph, acc, npairs)) SPH_KEEP_F(a.y)
-            if (fluid_pair<VISC, false, FILTER, RECOMP>(b.x, ci, vi, phat_i, pos, vel, phat, sc.phat_coef, pic, sc.dd_coef, ph, acc, npairs)) SPH_KEEP_F(b.x)
-            if (fluid_pair<VISC, false, FILTER, RECOMP>(b.y, ci, vi, phat_i, pos, vel, phat, sc.phat_coef, pic, sc.dd_coef, ph, acc, npairs)) SPH_KEEP_F(b.y)
+            SPH_PAIR(false, a.x, acc);
+            SPH_PAIR(false, a.y, acc);
+            SPH_PAIR(false, b.x, acc);
+            SPH_PAIR(false, b.y, acc);
         }
         for (; k < nf; k += 2, lp += S) {
             const uint2 a = ld_chunk<FRESH>(lp);
             const bool two = k + 1 < nf;
             SPH_GUARD((a.x >> kCodeBits) < n && (!two || (a.y >> kCodeBits) < n), st, break)
-            if (fluid_pair<VISC, false, FILTER, RECOMP>(a.x, ci, vi, phat_i, pos, vel, phat, sc.phat_coef, pic, sc.dd_coef, ph, acc, npairs)) SPH_KEEP_F(a.x)
-            if (two && fluid_pair<VISC, false, FILTER, RECOMP>(a.y, ci, vi, phat_i, pos, vel, phat, sc.phat_coef, pic, sc.dd_coef, ph, acc, npairs)) SPH_KEEP_F(a.y)
+            SPH_PAIR(false, a.x, acc);
+            if (two) SPH_PAIR(false, a.y, acc);
         }
         lp = reinterpret_cast<const uint2*>(nlist) + (size_t)(list_chunks(ph.max_neibs) - 1u) * S + i;
         for (k = 0; k < nb; k += 2, lp -= S) {
             const uint2 a = ld_chunk<FRESH>(lp);
             const bool two = k + 1 < nb;
             SPH_GUARD((a.x >> kCodeBits) < n && (!two || (a.y >> kCodeBits) < n), st, break)
-            if (fluid_pair<VISC, true, FILTER, RECOMP>(a.x, ci, vi, phat_i, pos, vel, phat, sc.phat_coef, pic, sc.dd_coef, ph, acc, npairs)) SPH_KEEP_B(a.x)
-            if (two && fluid_pair<VISC, true, FILTER, RECOMP>(a.y, ci, vi, phat_i, pos, vel, phat, sc.phat_coef, pic, sc.dd_coef, ph, acc, npairs)) SPH_KEEP_B(a.y)
+            SPH_PAIR(true, a.x, acc);
+            if (two) SPH_PAIR(true, a.y, acc);
         }
         acc.ax = fmaf(ph.aF, acc.ax, ph.g[0]);
         acc.ay = fmaf(ph.aF, acc.ay, ph.g[1]);
@@ -371,14 +340,14 @@ __device__ __forceinline__ void particle_pass(
     } else {
         // boundary particle: continuity over its fluid neighbours, u_i = 0
         const Central ci = central_of(pi, cx, cy, cz);
-        const uint2* lp = reinterpret_cast<const uint2*>(nlist) + i;  // list of the build
-        const uint4* cp = reinterpret_cast<const uint4*>(nlist) + i;  // chunked exact list
+        const uint2* lp = reinterpret_cast<const uint2*>(nlist) + i;
+        const uint4* cp = reinterpret_cast<const uint4*>(nlist) + i;  // SKIN
         uint4 q = make_uint4(0u, 0u, 0u, 0u);
         uint2 q2 = make_uint2(0u, 0u);
 #pragma unroll 2
         for (uint32_t k = 0; k < nf; ++k) {
             uint32_t e;
-            if (CHUNKED) {
+            if (SKIN) {
                 if ((k & 3u) == 0u) {
                     q = __ldg(cp);
                     cp += S;
@@ -392,19 +361,11 @@ __device__ __forceinline__ void particle_pass(
                 e = (k & 1u) ? q2.y : q2.x;
             }
             SPH_GUARD((e >> kCodeBits) < n, st, continue)
-            if (!boundary_pair<FILTER>(e, ci, pos, vel, ph, acc)) continue;
-            if (FILTER) ++npairs;
-            SPH_KEEP_F(e)
+            boundary_pair(e, ci, pos, vel, ph, acc);
         }
         acc.drho *= ph.aF;
     }
-#undef SPH_KEEP_F
-#undef SPH_KEEP_B
-    if (COMPACT) {
-        xf.flush();
-        xb.flush();
-        ncount_x[i] = xf.n | (xb.n << 16);
-    }
+#undef SPH_PAIR
 
     // epilogue written out here rather than through finish_particle() of
     // forces_common.cuh (same operations): measured 7 % faster in these kernels
@@ -480,17 +441,11 @@ __device__ __forceinline__ void forces_body(
     float4* io_pos, float4* io_vel, float* io_phat, float4* __restrict__ force_out,
     const uint32_t* __restrict__ pinfo, const uint32_t* __restrict__ nlist, const uint32_t* __restrict__ ncount,
     const SceneDev* __restrict__ scenes, SceneDyn* __restrict__ dyn, DevStatus* __restrict__ st, const Phys& ph,
-    int acc_dt, const float4* __restrict__ pos_ref, uint32_t* __restrict__ nlist_x,
-    uint32_t* __restrict__ ncount_x, const uint32_t* __restrict__ pid) {
+    int acc_dt, const float4* __restrict__ pos_ref, const uint32_t* __restrict__ pid) {
     const uint32_t n = st->n_active;
-    uint32_t npairs = 0;
     for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) / LANES; i < n; i += gridDim.x * blockDim.x / LANES)
-        particle_pass<VISC, MODE, SKIN, false, LANES>(i, n, pos, vel, phat, io_pos, io_vel, io_phat, force_out, pinfo, nlist, ncount,
-                                        scenes, dyn, st, ph, acc_dt, pos_ref, nlist_x, ncount_x, pid, npairs);
-    if (SKIN && MODE == kPredict) {
-        const uint32_t w = __reduce_add_sync(0xffffffffu, npairs);
-        if ((threadIdx.x & 31) == 0 && w) atomicAdd(&st->interactions, (unsigned long long)w);
-    }
+        particle_pass<VISC, MODE, SKIN, false, LANES>(i, n, pos, vel, phat, io_pos, io_vel, io_phat, force_out, pinfo,
+                                                      nlist, ncount, scenes, dyn, st, ph, acc_dt, pos_ref, pid);
 }
 
 template <int VISC, int MODE, int kBlock, int kMinBlocks, bool SKIN, int LANES>
@@ -499,10 +454,85 @@ __global__ void __launch_bounds__(kBlock, MODE == kForcesOnly ? (kMinBlocks * 2 
     float4* io_pos, float4* io_vel, float* io_phat, float4* __restrict__ force_out,
     const uint32_t* __restrict__ pinfo, const uint32_t* __restrict__ nlist, const uint32_t* __restrict__ ncount,
     const SceneDev* __restrict__ scenes, SceneDyn* __restrict__ dyn, DevStatus* __restrict__ st, const Phys ph,
-    int acc_dt, const float4* __restrict__ pos_ref, uint32_t* __restrict__ nlist_x,
-    uint32_t* __restrict__ ncount_x, const uint32_t* __restrict__ pid) {
-    forces_body<VISC, MODE, SKIN, LANES>(pos, vel, phat, io_pos, io_vel, io_phat, force_out, pinfo, nlist, ncount, scenes, dyn,
-                                  st, ph, acc_dt, pos_ref, nlist_x, ncount_x, pid);
+    int acc_dt, const float4* __restrict__ pos_ref, const uint32_t* __restrict__ pid) {
+    forces_body<VISC, MODE, SKIN, LANES>(pos, vel, phat, io_pos, io_vel, io_phat, force_out, pinfo, nlist, ncount, scenes,
+                                         dyn, st, ph, acc_dt, pos_ref, pid);
+}
+
+// ---------------------------------------------------------------------
+// A list with a skin (rebuilt every k steps): the step's exact list, the listed pairs within the
+// influence radius at x^n, in list order, in chunks of four entries.  Both passes of the step (and
+// sph_forces) then run over it.  One gather and one test a listed pair; the
+// predictor over the skin list itself evaluated a warp's pairs beyond the radius along with the others
+// (1.65M dam break, skin 0.3 h: 640 us, now 290 for the list and 283 for the pass; bound by the gathers
+// through L1).
+// count: add the pairs kept to DevStatus.interactions.
+// ---------------------------------------------------------------------
+__global__ void __launch_bounds__(128, 8) k_exact_list(const float4* __restrict__ pos, const uint32_t* __restrict__ pinfo,
+                                                       const uint32_t* __restrict__ nlist,
+                                                       const uint32_t* __restrict__ ncount,
+                                                       const SceneDev* __restrict__ scenes, DevStatus* __restrict__ st,
+                                                       float R2, uint32_t max_neibs, uint32_t stride, int count,
+                                                       uint32_t* __restrict__ nlist_x, uint32_t* __restrict__ ncount_x) {
+    const uint32_t n = st->n_active;
+    uint32_t kept = 0;
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const SceneDev& sc = scenes[pinfo[i]];
+        const Central ci = central_of(pos[i], sc.cell_f[0], sc.cell_f[1], sc.cell_f[2]);
+        const uint32_t cnt = ncount[i];
+        uint32_t nf = cnt & 0xffffu, nb = cnt >> 16;
+        SPH_GUARD(nf + nb <= max_neibs, st, nf = nb = 0)
+        const size_t S = stride;
+        auto within = [&](uint32_t e, const float4& pj) -> bool {
+            const float rx = pick(e, ci.xm, ci.x0, ci.xp) - pj.x;
+            const float ry = pick(e >> 2, ci.ym, ci.y0, ci.yp) - pj.y;
+            const float rz = pick(e >> 4, ci.zm, ci.z0, ci.zp) - pj.z;
+            return fmaf(rx, rx, fmaf(ry, ry, rz * rz)) < R2;
+        };
+        auto part = [&](const uint2* lp, ptrdiff_t step, uint32_t m, ChunkWriter& w) {
+            uint32_t k = 0;
+            uint2 an = make_uint2(0u, 0u), bn = make_uint2(0u, 0u);
+            if (m >= 4) {
+                an = __ldg(lp);
+                bn = __ldg(lp + step);
+            }
+            for (; k + 4 <= m; k += 4, lp += 2 * step) {
+                const uint2 a = an, b = bn;
+                if (k + 8 <= m) {  // the next iteration's chunks
+                    an = __ldg(lp + 2 * step);
+                    bn = __ldg(lp + 3 * step);
+                }
+                SPH_GUARD((max(max(a.x, a.y), max(b.x, b.y)) >> kCodeBits) < n, st, break)
+                const float4 p0 = pos[a.x >> kCodeBits], p1 = pos[a.y >> kCodeBits];
+                const float4 p2 = pos[b.x >> kCodeBits], p3 = pos[b.y >> kCodeBits];
+                const bool h0 = within(a.x, p0), h1 = within(a.y, p1), h2 = within(b.x, p2), h3 = within(b.y, p3);
+                w.put(h0, a.x);
+                w.put(h1, a.y);
+                w.put(h2, b.x);
+                w.put(h3, b.y);
+            }
+            for (; k < m; k += 2, lp += step) {
+                const uint2 a = __ldg(lp);
+                const bool two = k + 1 < m;
+                SPH_GUARD((a.x >> kCodeBits) < n && (!two || (a.y >> kCodeBits) < n), st, break)
+                w.put(within(a.x, pos[a.x >> kCodeBits]), a.x);
+                if (two) w.put(within(a.y, pos[a.y >> kCodeBits]), a.y);
+            }
+            w.flush();
+        };
+        const uint2* const fl = reinterpret_cast<const uint2*>(nlist) + i;
+        ChunkWriter wf{make_uint4(0u, 0u, 0u, 0u), 0u, reinterpret_cast<uint4*>(nlist_x) + i, S};
+        part(fl, (ptrdiff_t)S, nf, wf);
+        ChunkWriter wb{make_uint4(0u, 0u, 0u, 0u), 0u,
+                       reinterpret_cast<uint4*>(nlist_x) + (size_t)exact_bnd_chunk(max_neibs) * S + i, S};
+        part(fl + (size_t)(list_chunks(max_neibs) - 1u) * S, -(ptrdiff_t)S, nb, wb);
+        ncount_x[i] = wf.n | (wb.n << 16);
+        kept += wf.n + wb.n;
+    }
+    if (count) {
+        const uint32_t w = __reduce_add_sync(0xffffffffu, kept);
+        if ((threadIdx.x & 31) == 0 && w) atomicAdd(&st->interactions, (unsigned long long)w);
+    }
 }
 
 // Predictor update (reading C6) from forces already stored by a
@@ -555,7 +585,6 @@ template <int VISC>
 __global__ void __launch_bounds__(kPipeBlock, 4) k_build_predict(const Buffers b, int cur, const Phys ph) {
     DevStatus* st = b.status;
     const uint32_t n = st->n_active;
-    uint32_t npairs = 0;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         uint32_t nfound;
         const uint32_t nent = build_particle(i, b.pos[cur], b.quads, b.cell[cur], b.pinfo[cur], b.start,
@@ -565,8 +594,7 @@ __global__ void __launch_bounds__(kPipeBlock, 4) k_build_predict(const Buffers b
         const uint32_t cnt = ld_count_fresh(b.ncount + i);
         particle_pass<VISC, kPredict, false, true>(i, n, b.pos[cur], b.vel[cur], b.phat[cur], b.pos_s, b.vel_s,
                                                    b.phat_s, nullptr, b.pinfo[cur], b.nlist, b.ncount, b.scenes,
-                                                   b.dyn, st, ph, 0, nullptr, nullptr, nullptr, b.pid[cur], npairs,
-                                                   cnt);
+                                                   b.dyn, st, ph, 0, nullptr, b.pid[cur], cnt);
     }
 }
 
@@ -613,11 +641,11 @@ __global__ void __launch_bounds__(kPipeBlock, kPersistMinBlocks) k_step_persiste
         grid.sync();
         forces_body<VISC, kPredict, false>(b.pos[nxt], b.vel[nxt], b.phat[nxt], b.pos_s, b.vel_s, b.phat_s, nullptr,
                                            b.pinfo[nxt], b.nlist, b.ncount, b.scenes, b.dyn, b.status, ph, 0,
-                                           nullptr, nullptr, nullptr, b.pid[nxt]);
+                                           nullptr, b.pid[nxt]);
         grid.sync();
         forces_body<VISC, kCorrect, false>(b.pos_s, b.vel_s, b.phat_s, b.pos[nxt], b.vel[nxt], b.phat[nxt], nullptr,
                                            b.pinfo[nxt], b.nlist, b.ncount, b.scenes, b.dyn, b.status, ph, 0,
-                                           nullptr, nullptr, nullptr, b.pid[nxt]);
+                                           nullptr, b.pid[nxt]);
         grid.sync();
     }
 }
@@ -626,53 +654,54 @@ template <int VISC, int B, int MB, bool SKIN, int LANES>
 void launch_forces_s(const Buffers& b, int cur, const Geometry& g, const Phys& ph, ForceMode mode, int acc_dt,
                      cudaStream_t st) {
     const unsigned grid = g.cap ? (unsigned)(((uint64_t)g.cap * LANES + B - 1) / B) : 1;
+    const uint32_t* const list = SKIN ? b.nlist_x : b.nlist;
+    const uint32_t* const count = SKIN ? b.ncount_x : b.ncount;
     switch (mode) {
         case kForcesOnly:
             k_forces<VISC, kForcesOnly, B, MB, SKIN, LANES><<<grid, B, 0, st>>>(
-                b.pos[cur], b.vel[cur], b.phat[cur], nullptr, nullptr, nullptr, b.force, b.pinfo[cur], b.nlist,
-                b.ncount, b.scenes, b.dyn, b.status, ph, acc_dt, nullptr, nullptr, nullptr, b.pid[cur]);
+                b.pos[cur], b.vel[cur], b.phat[cur], nullptr, nullptr, nullptr, b.force, b.pinfo[cur], list, count,
+                b.scenes, b.dyn, b.status, ph, acc_dt, nullptr, b.pid[cur]);
             break;
         case kPredict:
             k_forces<VISC, kPredict, B, MB, SKIN, LANES><<<grid, B, 0, st>>>(
-                b.pos[cur], b.vel[cur], b.phat[cur], b.pos_s, b.vel_s, b.phat_s, nullptr, b.pinfo[cur], b.nlist,
-                b.ncount, b.scenes, b.dyn, b.status, ph, 0, nullptr, b.nlist_x, b.ncount_x, b.pid[cur]);
+                b.pos[cur], b.vel[cur], b.phat[cur], b.pos_s, b.vel_s, b.phat_s, nullptr, b.pinfo[cur], list, count,
+                b.scenes, b.dyn, b.status, ph, 0, nullptr, b.pid[cur]);
             break;
-        case kCorrect:  // a skin list: the exact list the predictor wrote
+        case kCorrect:
             k_forces<VISC, kCorrect, B, MB, SKIN, LANES><<<grid, B, 0, st>>>(
-                b.pos_s, b.vel_s, b.phat_s, b.pos[cur], b.vel[cur], b.phat[cur], nullptr, b.pinfo[cur],
-                SKIN ? b.nlist_x : b.nlist, SKIN ? b.ncount_x : b.ncount, b.scenes, b.dyn, b.status, ph, 0,
-                b.pos_ref, nullptr, nullptr, b.pid[cur]);
+                b.pos_s, b.vel_s, b.phat_s, b.pos[cur], b.vel[cur], b.phat[cur], nullptr, b.pinfo[cur], list, count,
+                b.scenes, b.dyn, b.status, ph, 0, b.pos_ref, b.pid[cur]);
             break;
     }
 }
 
+// (a skin list's passes run with one thread per particle)
 template <int VISC, int B, int MB, int LANES = 1>
 void launch_forces_b(const Buffers& b, int cur, const Geometry& g, const Phys& ph, ForceMode mode, int acc_dt,
-                     cudaStream_t st, bool skin) {
-    if (skin)
-        launch_forces_s<VISC, B, MB, true, 1>(b, cur, g, ph, mode, acc_dt, st);
+                     cudaStream_t st) {
+    if (b.pos_ref)
+        launch_forces_s<VISC, (LANES > 1 ? 128 : B), (LANES > 1 ? 8 : MB), true, 1>(b, cur, g, ph, mode, acc_dt, st);
     else
         launch_forces_s<VISC, B, MB, false, LANES>(b, cur, g, ph, mode, acc_dt, st);
 }
 
 // launch shapes of the force kernels (autotuned, the corrector pass on its own):
 // threads per block and the register cap implied by a minimum of resident blocks per SM; the
-// last two are groups of lanes per particle (an every-step list) or looser register caps (a
-// skin list)
+// last two are groups of lanes per particle
 template <int VISC>
 void launch_forces_v(const Buffers& b, int cur, const Geometry& g, const Phys& ph, ForceMode mode, int acc_dt,
-                     cudaStream_t st, bool skin) {
+                     cudaStream_t st) {
     const int v = mode == kCorrect ? ph.forces_variant_c : ph.forces_variant;
     if constexpr (has_diffusion(VISC)) {  // one thread shape beside the groups of lanes
-        if (v == 3) launch_forces_b<VISC, 128, 6, 4>(b, cur, g, ph, mode, acc_dt, st, skin);
-        else if (v == 4) launch_forces_b<VISC, 128, 4, 8>(b, cur, g, ph, mode, acc_dt, st, skin);
-        else launch_forces_b<VISC, 128, 8>(b, cur, g, ph, mode, acc_dt, st, skin);
+        if (v == 3) launch_forces_b<VISC, 128, 6, 4>(b, cur, g, ph, mode, acc_dt, st);
+        else if (v == 4) launch_forces_b<VISC, 128, 4, 8>(b, cur, g, ph, mode, acc_dt, st);
+        else launch_forces_b<VISC, 128, 8>(b, cur, g, ph, mode, acc_dt, st);
     } else switch (v) {
-        case 0: launch_forces_b<VISC, 64, 16>(b, cur, g, ph, mode, acc_dt, st, skin); break;
-        case 2: launch_forces_b<VISC, 256, 4>(b, cur, g, ph, mode, acc_dt, st, skin); break;
-        case 3: launch_forces_b<VISC, 128, 6, 4>(b, cur, g, ph, mode, acc_dt, st, skin); break;
-        case 4: launch_forces_b<VISC, 128, 4, 8>(b, cur, g, ph, mode, acc_dt, st, skin); break;
-        default: launch_forces_b<VISC, 128, 8>(b, cur, g, ph, mode, acc_dt, st, skin); break;
+        case 0: launch_forces_b<VISC, 64, 16>(b, cur, g, ph, mode, acc_dt, st); break;
+        case 2: launch_forces_b<VISC, 256, 4>(b, cur, g, ph, mode, acc_dt, st); break;
+        case 3: launch_forces_b<VISC, 128, 6, 4>(b, cur, g, ph, mode, acc_dt, st); break;
+        case 4: launch_forces_b<VISC, 128, 4, 8>(b, cur, g, ph, mode, acc_dt, st); break;
+        default: launch_forces_b<VISC, 128, 8>(b, cur, g, ph, mode, acc_dt, st); break;
     }
 }
 
@@ -736,26 +765,29 @@ void launch_conservation(const Buffers& b, int cur, double* scratch, cudaStream_
 
 void launch_forces(const Buffers& b, int cur, const Geometry& g, const Phys& ph, ForceMode mode, int acc_dt,
                    cudaStream_t st) {
+    if (b.pos_ref && mode != kCorrect)  // a skin list: first the step's exact list
+        k_exact_list<<<g.cap ? (g.cap + 127) / 128 : 1, 128, 0, st>>>(
+            b.pos[cur], b.pinfo[cur], b.nlist, b.ncount, b.scenes, b.status, ph.R2, ph.max_neibs, ph.stride,
+            mode == kPredict, b.nlist_x, b.ncount_x);
     if (ph.general) {
         launch_forces_models(b, cur, g, ph, mode, acc_dt, st);
         return;
     }
-    const bool skin = b.pos_ref != nullptr;
     if (ph.ddiff) {
         if (ph.visc == SPH_VISC_LAMINAR)
-            launch_forces_v<SPH_VISC_LAMINAR | kDiffusion>(b, cur, g, ph, mode, acc_dt, st, skin);
+            launch_forces_v<SPH_VISC_LAMINAR | kDiffusion>(b, cur, g, ph, mode, acc_dt, st);
         else
-            launch_forces_v<SPH_VISC_ARTIFICIAL | kDiffusion>(b, cur, g, ph, mode, acc_dt, st, skin);
+            launch_forces_v<SPH_VISC_ARTIFICIAL | kDiffusion>(b, cur, g, ph, mode, acc_dt, st);
     } else if (ph.visc == SPH_VISC_LAMINAR)
-        launch_forces_v<SPH_VISC_LAMINAR>(b, cur, g, ph, mode, acc_dt, st, skin);
+        launch_forces_v<SPH_VISC_LAMINAR>(b, cur, g, ph, mode, acc_dt, st);
     else
-        launch_forces_v<SPH_VISC_ARTIFICIAL>(b, cur, g, ph, mode, acc_dt, st, skin);
+        launch_forces_v<SPH_VISC_ARTIFICIAL>(b, cur, g, ph, mode, acc_dt, st);
 }
 
 const char* forces_variant_name(int v) {
     static const char* names[kForcesVariants] = {"64 threads, <=64 regs", "128 threads, <=64 regs",
-                                                 "256 threads, <=64 regs", "4 lanes/particle (skin list: <=85 regs)",
-                                                 "8 lanes/particle (skin list: <=128 regs)"};
+                                                 "256 threads, <=64 regs", "4 lanes/particle (skin list: 1)",
+                                                 "8 lanes/particle (skin list: 1)"};
     return v >= 0 && v < kForcesVariants ? names[v] : "?";
 }
 

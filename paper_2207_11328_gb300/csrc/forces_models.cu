@@ -56,13 +56,11 @@ __device__ __forceinline__ float visc_weight(int op, float ri, float rj) {
 }
 
 // one neighbour of a fluid particle (BND: boundary neighbour, negated mass, u_j = 0)
-// (filter: skin list, skip pairs beyond the cutoff and count the rest; returns
-// whether the pair is within it)
 template <int KT, int VISC, bool BND>
-__device__ __forceinline__ bool model_pair(uint32_t e, const Central& ci, const float4& vi, float phat_i, float ri,
+__device__ __forceinline__ void model_pair(uint32_t e, const Central& ci, const float4& vi, float phat_i, float ri,
                                            const float4* __restrict__ pos, const float4* __restrict__ vel,
                                            const float* __restrict__ phat, float pi_coef, float dd_coef,
-                                           const Phys& ph, bool filter, Acc& acc, uint32_t& npairs) {
+                                           const Phys& ph, Acc& acc) {
     const uint32_t j = e >> kCodeBits;
     const float4 pj = pos[j];
     const float4 vj = vel[j];
@@ -71,10 +69,6 @@ __device__ __forceinline__ bool model_pair(uint32_t e, const Central& ci, const 
     const float ry = pick(e >> 2, ci.ym, ci.y0, ci.yp) - pj.y;
     const float rz = pick(e >> 4, ci.zm, ci.z0, ci.zp) - pj.z;
     const float r2 = fmaxf(fmaf(rx, rx, fmaf(ry, ry, rz * rz)), 1e-30f);
-    if (filter) {
-        if (!(r2 < ph.R2)) return false;
-        ++npairs;
-    }
     const float rinv = rsqrtf(r2);
     const float mF = (BND ? -pj.w : pj.w) * kernel_shape<KT>(r2, rinv, ph);  // m_j F / aF
     const float rj = 1.0f + vj.w;
@@ -112,7 +106,6 @@ __device__ __forceinline__ bool model_pair(uint32_t e, const Central& ci, const 
             acc.az = fmaf(lx, rz, acc.az);
         }
     }
-    return true;
 }
 
 template <int KT, int VISC, int MODE>
@@ -121,15 +114,9 @@ __global__ void __launch_bounds__(kModelBlock, 4) k_forces_m(
     float4* io_pos, float4* io_vel, float* io_phat, float4* __restrict__ force_out,
     const uint32_t* __restrict__ pinfo, const uint32_t* __restrict__ nlist, const uint32_t* __restrict__ ncount,
     const SceneDev* __restrict__ scenes, SceneDyn* __restrict__ dyn, DevStatus* __restrict__ st, const Phys ph,
-    int acc_dt, int skin, const float4* __restrict__ pos_ref, uint32_t* __restrict__ nlist_x,
-    uint32_t* __restrict__ ncount_x, const uint32_t* __restrict__ pid) {
-    // skin list: the predictor (and sph_forces) filter by the cutoff; the predictor keeps the
-    // pairs within it (the step's exact list) for the corrector, which reads that list as is
-    const bool filter = skin && MODE != kCorrect;
-    const bool compact = skin && MODE == kPredict;
-    const bool chunked = skin && MODE == kCorrect;  // nlist/ncount: that exact list, in chunks of four
+    int acc_dt, int skin, const float4* __restrict__ pos_ref, const uint32_t* __restrict__ pid) {
+    // skin: nlist/ncount are the step's exact list, in chunks of four entries
     const uint32_t n = st->n_active;
-    uint32_t npairs = 0;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const uint32_t s = pinfo[i];
         const SceneDev& sc = scenes[s];
@@ -144,57 +131,46 @@ __global__ void __launch_bounds__(kModelBlock, 4) k_forces_m(
         const size_t S = ph.stride;
         Acc acc{0.f, 0.f, 0.f, 0.f};
         const uint32_t kxb = exact_bnd_chunk(ph.max_neibs);
-        ChunkWriter xf{make_uint4(0u, 0u, 0u, 0u), 0u, reinterpret_cast<uint4*>(nlist_x), S, i};
-        ChunkWriter xb{make_uint4(0u, 0u, 0u, 0u), 0u, reinterpret_cast<uint4*>(nlist_x) + (size_t)kxb * S, S, i};
-        // entry k of the fluid / boundary part: the list of the build (two-entry
-        // chunks, boundary part from the back) or, in the skin-list corrector, the
-        // step's exact list (four-entry chunks, boundary part from chunk kxb)
         auto fluid_entry = [&](uint32_t k) -> uint32_t {
-            return chunked ? __ldg(nlist + ((size_t)(k >> 2) * S + i) * 4 + (k & 3u))
-                           : __ldg(nlist + list_fluid_word(k, i, S));
+            return skin ? __ldg(nlist + ((size_t)(k >> 2) * S + i) * 4 + (k & 3u)) : __ldg(nlist + list_fluid_word(k, i, S));
         };
         auto bnd_entry = [&](uint32_t k) -> uint32_t {
-            return chunked ? __ldg(nlist + ((size_t)(kxb + (k >> 2)) * S + i) * 4 + (k & 3u))
-                           : __ldg(nlist + list_bnd_word(k, i, S, ph.max_neibs));
+            return skin ? __ldg(nlist + ((size_t)(kxb + (k >> 2)) * S + i) * 4 + (k & 3u))
+                        : __ldg(nlist + list_bnd_word(k, i, S, ph.max_neibs));
         };
         if (fluid_i) {
             const float phat_i = phat[i];
             const float pic = sc.pi_coef, ddc = sc.dd_coef;
             uint32_t k = 0;
-#define SPH_KEEP_F(e) if (compact) xf.put(e);
-#define SPH_KEEP_B(e) if (compact) xb.put(e);
+#define SPH_PAIR(BND, e) model_pair<KT, VISC, BND>(e, ci, vi, phat_i, ri, pos, vel, phat, pic, ddc, ph, acc)
             for (; k + 4 <= nf; k += 4) {
-                uint32_t e0, e1, e2, e3;
-                if (chunked) {
+                uint2 a, b;
+                if (skin) {
                     const uint4 q = __ldg(reinterpret_cast<const uint4*>(nlist) + (size_t)(k >> 2) * S + i);
-                    e0 = q.x;
-                    e1 = q.y;
-                    e2 = q.z;
-                    e3 = q.w;
+                    a = make_uint2(q.x, q.y);
+                    b = make_uint2(q.z, q.w);
                 } else {
                     const uint2* lp = reinterpret_cast<const uint2*>(nlist) + (size_t)(k >> 1) * S + i;
-                    const uint2 a = __ldg(lp), b = __ldg(lp + S);
-                    e0 = a.x;
-                    e1 = a.y;
-                    e2 = b.x;
-                    e3 = b.y;
+                    a = __ldg(lp);
+                    b = __ldg(lp + S);
                 }
-                SPH_GUARD((max(max(e0, e1), max(e2, e3)) >> kCodeBits) < n, st, break)
-                if (model_pair<KT, VISC, false>(e0, ci, vi, phat_i, ri, pos, vel, phat, pic, ddc, ph, filter, acc, npairs)) SPH_KEEP_F(e0)
-                if (model_pair<KT, VISC, false>(e1, ci, vi, phat_i, ri, pos, vel, phat, pic, ddc, ph, filter, acc, npairs)) SPH_KEEP_F(e1)
-                if (model_pair<KT, VISC, false>(e2, ci, vi, phat_i, ri, pos, vel, phat, pic, ddc, ph, filter, acc, npairs)) SPH_KEEP_F(e2)
-                if (model_pair<KT, VISC, false>(e3, ci, vi, phat_i, ri, pos, vel, phat, pic, ddc, ph, filter, acc, npairs)) SPH_KEEP_F(e3)
+                SPH_GUARD((max(max(a.x, a.y), max(b.x, b.y)) >> kCodeBits) < n, st, break)
+                SPH_PAIR(false, a.x);
+                SPH_PAIR(false, a.y);
+                SPH_PAIR(false, b.x);
+                SPH_PAIR(false, b.y);
             }
             for (; k < nf; ++k) {
                 const uint32_t e = fluid_entry(k);
                 SPH_GUARD((e >> kCodeBits) < n, st, continue)
-                if (model_pair<KT, VISC, false>(e, ci, vi, phat_i, ri, pos, vel, phat, pic, ddc, ph, filter, acc, npairs)) SPH_KEEP_F(e)
+                SPH_PAIR(false, e);
             }
             for (k = 0; k < nb; ++k) {
                 const uint32_t e = bnd_entry(k);
                 SPH_GUARD((e >> kCodeBits) < n, st, continue)
-                if (model_pair<KT, VISC, true>(e, ci, vi, phat_i, ri, pos, vel, phat, pic, ddc, ph, filter, acc, npairs)) SPH_KEEP_B(e)
+                SPH_PAIR(true, e);
             }
+#undef SPH_PAIR
             acc.ax = fmaf(ph.aF, acc.ax, ph.g[0]);
             acc.ay = fmaf(ph.aF, acc.ay, ph.g[1]);
             acc.az = fmaf(ph.aF, acc.az, ph.g[2]);
@@ -213,11 +189,6 @@ __global__ void __launch_bounds__(kModelBlock, 4) k_forces_m(
                 const float ry = pick(e >> 2, ci.ym, ci.y0, ci.yp) - pj.y;
                 const float rz = pick(e >> 4, ci.zm, ci.z0, ci.zp) - pj.z;
                 const float r2 = fmaxf(fmaf(rx, rx, fmaf(ry, ry, rz * rz)), 1e-30f);
-                if (filter) {
-                    if (!(r2 < ph.R2)) continue;
-                    ++npairs;
-                }
-                SPH_KEEP_F(e)
                 float mF = pj.w * kernel_shape<KT>(r2, rsqrtf(r2), ph);
                 if (form2) mF *= __fdividef(ri, 1.0f + vj.w);
                 const float udx = -fmaf(vj.x, rx, fmaf(vj.y, ry, vj.z * rz));
@@ -225,19 +196,8 @@ __global__ void __launch_bounds__(kModelBlock, 4) k_forces_m(
             }
             acc.drho *= ph.aF;
         }
-#undef SPH_KEEP_F
-#undef SPH_KEEP_B
-        if (compact) {
-            xf.flush();
-            xb.flush();
-            ncount_x[i] = xf.n | (xb.n << 16);
-        }
         finish_particle<MODE>(i, s, sc, pi, vi, fluid_i, acc, io_pos, io_vel, io_phat, force_out, dyn, st, ph,
                               acc_dt, pos_ref, pid);
-    }
-    if (compact) {
-        const uint32_t w = __reduce_add_sync(0xffffffffu, npairs);
-        if ((threadIdx.x & 31) == 0 && w) atomicAdd(&st->interactions, (unsigned long long)w);
     }
 }
 
@@ -245,23 +205,24 @@ template <int KT, int VISC>
 void launch_m(const Buffers& b, int cur, const Geometry& g, const Phys& ph, ForceMode mode, int acc_dt,
               cudaStream_t st) {
     const unsigned grid = g.cap ? (g.cap + kModelBlock - 1) / kModelBlock : 1;
-    const int skin = b.pos_ref != nullptr;
+    const bool skin = b.pos_ref != nullptr;  // then the step's exact list
+    const uint32_t* const list = skin ? b.nlist_x : b.nlist;
+    const uint32_t* const count = skin ? b.ncount_x : b.ncount;
     switch (mode) {
         case kForcesOnly:
             k_forces_m<KT, VISC, kForcesOnly><<<grid, kModelBlock, 0, st>>>(
-                b.pos[cur], b.vel[cur], b.phat[cur], nullptr, nullptr, nullptr, b.force, b.pinfo[cur], b.nlist,
-                b.ncount, b.scenes, b.dyn, b.status, ph, acc_dt, skin, nullptr, nullptr, nullptr, b.pid[cur]);
+                b.pos[cur], b.vel[cur], b.phat[cur], nullptr, nullptr, nullptr, b.force, b.pinfo[cur], list, count,
+                b.scenes, b.dyn, b.status, ph, acc_dt, skin, nullptr, b.pid[cur]);
             break;
         case kPredict:
             k_forces_m<KT, VISC, kPredict><<<grid, kModelBlock, 0, st>>>(
-                b.pos[cur], b.vel[cur], b.phat[cur], b.pos_s, b.vel_s, b.phat_s, nullptr, b.pinfo[cur], b.nlist,
-                b.ncount, b.scenes, b.dyn, b.status, ph, 0, skin, nullptr, b.nlist_x, b.ncount_x, b.pid[cur]);
+                b.pos[cur], b.vel[cur], b.phat[cur], b.pos_s, b.vel_s, b.phat_s, nullptr, b.pinfo[cur], list, count,
+                b.scenes, b.dyn, b.status, ph, 0, skin, nullptr, b.pid[cur]);
             break;
         case kCorrect:
-            k_forces_m<KT, VISC, kCorrect><<<grid, kModelBlock, 0, st>>>(  // a skin list: the predictor's exact list
-                b.pos_s, b.vel_s, b.phat_s, b.pos[cur], b.vel[cur], b.phat[cur], nullptr, b.pinfo[cur],
-                skin ? b.nlist_x : b.nlist, skin ? b.ncount_x : b.ncount, b.scenes, b.dyn, b.status, ph, 0, skin,
-                b.pos_ref, nullptr, nullptr, b.pid[cur]);
+            k_forces_m<KT, VISC, kCorrect><<<grid, kModelBlock, 0, st>>>(
+                b.pos_s, b.vel_s, b.phat_s, b.pos[cur], b.vel[cur], b.phat[cur], nullptr, b.pinfo[cur], list, count,
+                b.scenes, b.dyn, b.status, ph, 0, skin, b.pos_ref, b.pid[cur]);
             break;
     }
 }

@@ -1062,7 +1062,7 @@ int sph_autotune(sph_ctx* c, void* stream, int* build_variant, int* forces_varia
     // force kernels: threads per block and register cap
     int best_f = c->ph.forces_variant;
     best = 3.4e38f;
-    const int n_shapes = large && !skin_mode(c) ? 3 : kForcesVariants;
+    const int n_shapes = large || skin_mode(c) ? 3 : kForcesVariants;
     for (int v = 0; v < n_shapes; ++v) {
         c->ph.forces_variant = v;
         // the predictor pass as the step runs it (it writes only the predicted-state scratch)

@@ -255,8 +255,8 @@ struct Buffers {
     uint32_t* pid[2];
     float* phat[2];          // P/rho^2 per particle, same order as pos/vel
     float4* pos_ref;         // offsets at the last list build (rebuild_every > 1), else null
-    uint32_t* nlist_x;       // skin list: the step's exact list (pairs within R at x^n), written by
-    uint32_t* ncount_x;      //   the predictor pass, read by the corrector pass; else null
+    uint32_t* nlist_x;       // skin list: the step's exact list (pairs within R at x^n, chunks of
+    uint32_t* ncount_x;      //   four entries), which its passes read; else null
     const uint32_t* gate;    // &status->rebuild for a skin list (pipeline kernels skip when 0), else null
     float4* pos_s;           // predicted state
     float4* vel_s;
@@ -338,11 +338,10 @@ void launch_tape_copy(const void* const* src, void* const* dst, const bool* wide
 
 // forces.cu
 enum ForceMode { kForcesOnly = 0, kPredict = 1, kCorrect = 2 };
-// With a skin list (pos_ref allocated) the predictor pass also writes the
-// pairs within R at x^n to nlist_x/ncount_x, and the corrector reads those.
-// With a skin list (pos_ref allocated) the kernels skip pairs beyond the
-// cutoff, the first pass counts the pairs within it (DevStatus.interactions)
-// and the corrector checks the displacement since the build.
+// With a skin list (pos_ref allocated) the forces-only and predictor passes first write the
+// step's exact list to nlist_x/ncount_x (the predictor counts its pairs,
+// DevStatus.interactions), and every pass reads that; the corrector checks the
+// displacement since the build.
 void launch_forces(const Buffers& b, int cur, const Geometry& g, const Phys& ph, ForceMode mode,
                    int acc_dt, cudaStream_t st);
 // forces_models.cu: the same passes for the other model options of Table 1
