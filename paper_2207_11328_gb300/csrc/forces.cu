@@ -22,6 +22,7 @@
 #include <cooperative_groups.h>
 
 #include "forces_common.cuh"
+#include "packed.cuh"
 #include "pipeline.cuh"
 
 namespace cg = cooperative_groups;
@@ -97,7 +98,7 @@ __device__ __forceinline__ void fluid_pair(uint32_t e, const Central& ci, const 
     const float ry = pick(e >> 2, ci.ym, ci.y0, ci.yp) - pj.y;
     const float rz = pick(e >> 4, ci.zm, ci.z0, ci.zp) - pj.z;
     const float r2 = fmaxf(fmaf(rx, rx, fmaf(ry, ry, rz * rz)), 1e-30f);
-    const float r = r2 * rsqrtf(r2);
+    const float r = r2 * rsqrt_fast(r2);
     const float t = fminf(fmaf(r, ph.inv_h, -2.0f), 0.0f);
     const float mj = BND ? -pj.w : pj.w;
     const float mF = mj * (t * t * t);  // m_j F / aF
@@ -106,16 +107,16 @@ __device__ __forceinline__ void fluid_pair(uint32_t e, const Central& ci, const 
     const float uz = BND ? vi.z : vi.z - vj.z;
     const float udx = fmaf(ux, rx, fmaf(uy, ry, uz * rz));
     add_rate(out, mF, udx);
-    if (has_diffusion(VISC) && !BND) add_diffusion(out, dd_coef * (vi.w - vj.w), __fdividef(mF, 1.0f + vj.w));
+    if (has_diffusion(VISC) && !BND) add_diffusion(out, dd_coef * (vi.w - vj.w), mF * rcp_fast(1.0f + vj.w));
     float bracket = phat_i + phat_j;
     if (is_artificial(VISC)) {
         // approaching pairs only (u.x < 0), without a branch: receding pairs add -pi*0
         const float den = (r2 + ph.eps_h2) * fmaf(0.5f, vi.w + vj.w, 1.0f);
-        bracket = fmaf(-pi_coef, __fdividef(fminf(udx, 0.f), den), bracket);
+        bracket = fmaf(-pi_coef, fminf(udx, 0.f) * rcp_fast(den), bracket);
     }
     add_force(out, mF * bracket, rx, ry, rz);
     if (is_laminar(VISC))
-        add_laminar(out, ph.nu4 * ph.inv_rho0 * __fdividef(mF, 2.0f + vi.w + vj.w), ux, uy, uz);
+        add_laminar(out, ph.nu4 * ph.inv_rho0 * (mF * rcp_fast(2.0f + vi.w + vj.w)), ux, uy, uz);
 }
 
 // one fluid neighbour of a boundary particle: continuity, u_i = 0
@@ -129,7 +130,7 @@ __device__ __forceinline__ void boundary_pair(uint32_t e, const Central& ci, con
     const float ry = pick(e >> 2, ci.ym, ci.y0, ci.yp) - pj.y;
     const float rz = pick(e >> 4, ci.zm, ci.z0, ci.zp) - pj.z;
     const float r2 = fmaxf(fmaf(rx, rx, fmaf(ry, ry, rz * rz)), 1e-30f);
-    const float r = r2 * rsqrtf(r2);
+    const float r = r2 * rsqrt_fast(r2);
     const float t = fminf(fmaf(r, ph.inv_h, -2.0f), 0.0f);
     add_rate(out, pj.w * (t * t * t), -fmaf(vj.x, rx, fmaf(vj.y, ry, vj.z * rz)));
 }

@@ -24,6 +24,7 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include "packed.cuh"
 #include "sph.h"
 
 namespace sphg {
@@ -199,7 +200,7 @@ __device__ __forceinline__ float eos_phat(float d, const Phys& ph, float phat_co
 #pragma unroll
     for (int k = 6; k >= 0; --k) poly = fmaf(poly, d, ph.coef[k]);
     const float opd = 1.0f + d;
-    return __fdividef(phat_coef * d * poly, opd * opd);
+    return phat_coef * d * poly * rcp_fast(opd * opd);
 }
 
 // ---- checked build ----------------------------------------------------
