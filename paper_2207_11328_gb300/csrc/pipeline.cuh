@@ -263,13 +263,13 @@ __device__ __forceinline__ void scatter_body(const uint32_t* __restrict__ key, c
 // ---------------------------------------------------------------------
 // (type, id) in 32 bits (ids < kMaxParticles = 2^26): one shuffle per comparison of the rank
 static_assert(kMaxParticles <= (1u << 31), "the id fits below the type bit");
-__device__ __forceinline__ uint32_t sort_key(const float4* pos, const uint32_t* pid, uint32_t idx) {
-    const uint32_t bnd = __float_as_uint(pos[idx].w) >> 31;  // sign bit = boundary
-    return (bnd << 31) | pid[idx];
+__device__ __forceinline__ uint32_t sort_key(float mass, uint32_t id) {
+    return (__float_as_uint(mass) & 0x80000000u) | id;  // sign bit = boundary
 }
 
 // cells per warp: 4 measured fastest on large grids (1.65M dam break, most cells empty: 78 -> 61 us;
-// 2.1M box, no empty cell: unchanged at 56 us; 8 and 16 cells per warp leave too few warps); 1 on
+// 2.1M box, no empty cell: unchanged at 56 us; 8 and 16 cells per warp leave too few warps; a cell's
+// gathers issued together, before its rank is counted: 66 -> 57 us); 1 on
 // grids of up to kReorderOneMax cells, whose warps are too few to hide a cell's chain of loads (216
 // cells 8.6 -> 2.5 us, 4,116 cells 8.6 -> 4.5 us)
 constexpr int kReorderCells = 4;
@@ -309,11 +309,19 @@ __device__ __forceinline__ void reorder_body(
             uint32_t nfluid = 0;
             for (uint32_t base = 0; base < n; base += 32) {
                 const uint32_t l = base + lane;
-                uint32_t idx = 0;
                 uint32_t mine = ~0u;  // above every key
+                // everything gathered at once: the loads return while the rank is counted
+                float4 p = make_float4(0.f, 0.f, 0.f, 0.f), v = p;
+                float h = 0.f;
+                uint32_t s = 0, id = 0;
                 if (l < n) {
-                    idx = unsorted[beg + l];
-                    mine = sort_key(pos, pid, idx);
+                    const uint32_t idx = unsorted[beg + l];
+                    p = pos[idx];
+                    id = pid[idx];
+                    s = pinfo[idx];
+                    v = vel[idx];
+                    h = phat[idx];
+                    mine = sort_key(p.w, id);
                 }
                 nfluid += __popc(__ballot_sync(0xffffffffu, l < n && (mine >> 31) == 0u));
                 uint32_t rank = 0;
@@ -324,14 +332,13 @@ __device__ __forceinline__ void reorder_body(
                     }
                 } else {
                     for (uint32_t k = 0; k < n; ++k) {
-                        const uint32_t o = sort_key(pos, pid, unsorted[beg + k]);
+                        const uint32_t j = unsorted[beg + k];
+                        const uint32_t o = sort_key(pos[j].w, pid[j]);
                         rank += o < mine;
                     }
                 }
                 if (l < n) {
-                    const uint32_t s = pinfo[idx];
                     const SceneDev& sc = scenes[s];
-                    float4 p = pos[idx];
                     cell_shift(p.x, sc.cell_f[0], sc.inv_cell_f[0], &p.x);
                     cell_shift(p.y, sc.cell_f[1], sc.inv_cell_f[1], &p.y);
                     cell_shift(p.z, sc.cell_f[2], sc.inv_cell_f[2], &p.z);
@@ -342,11 +349,11 @@ __device__ __forceinline__ void reorder_body(
                     qd[0] = p.x;
                     qd[4] = p.y;
                     qd[8] = p.z;
-                    vel_o[d] = vel[idx];
-                    phat_o[d] = phat[idx];
+                    vel_o[d] = v;
+                    phat_o[d] = h;
                     cell_o[d] = c;
                     pinfo_o[d] = s;
-                    pid_o[d] = pid[idx];
+                    pid_o[d] = id;
                 }
             }
             if (lane == 0) cell_nfluid[c] = nfluid;
