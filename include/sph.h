@@ -216,9 +216,10 @@ int sph_forces(sph_ctx* ctx, void* stream);
  * first stage over dt/2, the second over dt) and Section 3 "The GPU in
  * GPUSPH" (the time step is a minimum over particles by parallel reduction);
  * the update formulas are reading C6, the dt formula reading C7 (not
- * printed in the paper).  Replays a captured CUDA graph per step: no host
- * round trip, the counters GPUSPH downloads every step stay on the device
- * until sph_get_stats.  Errors: SPH_ERR_STATE before an upload,
+ * printed in the paper).  Replays captured CUDA graphs of one step and, in
+ * longer runs, of several: no host round trip, the counters GPUSPH downloads
+ * every step stay on the device until sph_get_stats.  Errors:
+ * SPH_ERR_STATE before an upload,
  * SPH_ERR_CUDA on a launch failure; device-found errors are sticky (see
  * Conventions). */
 int sph_step(sph_ctx* ctx, uint32_t nsteps, void* stream);

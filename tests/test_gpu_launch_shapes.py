@@ -113,3 +113,20 @@ def test_density_diffusion_in_every_shape_matches_the_oracle(visc, skin, walls):
             ref = got
         for a, b in zip(got, ref):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("skin", [False, True])
+def test_runs_of_steps_equal_single_steps(skin):
+    """Calls of several steps replay graphs of several, from either buffer: the same bits as one step a call."""
+    s = _cloud(700, 4, 20, True, 60)
+    kw = dict(rebuild_every=4, skin=0.3 * s.h, max_neibs=512) if skin else dict(max_neibs=512)
+    a, b = sim_for(s, **kw), sim_for(s, **kw)
+    for run in (3, 5, 4, 9, 1, 22, 4):  # below, at and above a graph's steps, odd and even; the graph is made in between
+        a.step(run)
+        for _ in range(run):
+            b.step(1)
+        for x, y in zip(a.download(), b.download()):
+            assert np.array_equal(x, y)
+    sa, sb = a.stats(), b.stats()
+    assert sa["steps"] == sb["steps"] == 48 and sa["time"] == sb["time"] and sa["builds"] == sb["builds"]
+    assert sa["kernels_per_step"] == sb["kernels_per_step"]
