@@ -74,17 +74,18 @@ __global__ void __launch_bounds__(kPipeBlock) k_scatter(const uint32_t* __restri
     scatter_body(key, slot, start, st, unsorted, nkeys);
 }
 
-template <int kCells>
+template <int kCells, bool kCopy>
 __global__ void __launch_bounds__(kPipeBlock) k_reorder(
     const float4* __restrict__ pos, const float4* __restrict__ vel, const float* __restrict__ phat,
     const uint32_t* __restrict__ pinfo, const uint32_t* __restrict__ pid, const uint32_t* __restrict__ start,
     const uint32_t* __restrict__ unsorted, const SceneDev* __restrict__ scenes, uint32_t n_cells,
     DevStatus* __restrict__ st, uint32_t* __restrict__ cell_nfluid, float4* __restrict__ pos_o,
     float4* __restrict__ vel_o, float* __restrict__ phat_o, uint32_t* __restrict__ cell_o,
-    uint32_t* __restrict__ pinfo_o, uint32_t* __restrict__ pid_o, float* __restrict__ quads, const uint32_t* __restrict__ gate) {
+    uint32_t* __restrict__ pinfo_o, uint32_t* __restrict__ pid_o, float* __restrict__ quads, const SortedCopy copy,
+    const uint32_t* __restrict__ gate) {
     if (gate && *gate == 0u) return;
-    reorder_body<kCells>(pos, vel, phat, pinfo, pid, start, unsorted, scenes, n_cells, st, cell_nfluid, pos_o, vel_o, phat_o,
-                 cell_o, pinfo_o, pid_o, quads);
+    reorder_body<kCells, kCopy>(pos, vel, phat, pinfo, pid, start, unsorted, scenes, n_cells, st, cell_nfluid, pos_o, vel_o,
+                                phat_o, cell_o, pinfo_o, pid_o, quads, copy);
 }
 
 // 1024 resident threads per SM (64 registers, a 24-byte spill); 1280 threads at 48 registers were
@@ -144,18 +145,25 @@ void launch_scatter(const Buffers& b, const Geometry& g, cudaStream_t st) {
                                                            g.n_cells + 1, b.gate);
 }
 
-template <int kCells>
-void launch_reorder_c(const Buffers& b, int cur, const Geometry& g, cudaStream_t st) {
+template <int kCells, bool kCopy>
+void launch_reorder_c(const Buffers& b, int cur, const Geometry& g, const SortedCopy& copy, cudaStream_t st) {
     const int nxt = cur ^ 1;
     const uint32_t warps = (g.n_cells + kCells - 1) / kCells;
-    k_reorder<kCells><<<grid_for(warps, kPipeBlock / 32), kPipeBlock, 0, st>>>(
+    k_reorder<kCells, kCopy><<<grid_for(warps, kPipeBlock / 32), kPipeBlock, 0, st>>>(
         b.pos[cur], b.vel[cur], b.phat[cur], b.pinfo[cur], b.pid[cur], b.start, b.unsorted, b.scenes, g.n_cells, b.status,
-        b.cell_nfluid, b.pos[nxt], b.vel[nxt], b.phat[nxt], b.cell[nxt], b.pinfo[nxt], b.pid[nxt], b.quads, b.gate);
+        b.cell_nfluid, b.pos[nxt], b.vel[nxt], b.phat[nxt], b.cell[nxt], b.pinfo[nxt], b.pid[nxt], b.quads, copy, b.gate);
 }
 
-void launch_reorder(const Buffers& b, int cur, const Geometry& g, cudaStream_t st) {
-    if (g.n_cells <= kReorderOneMax) launch_reorder_c<1>(b, cur, g, st);
-    else launch_reorder_c<kReorderCells>(b, cur, g, st);
+void launch_reorder(const Buffers& b, int cur, const Geometry& g, cudaStream_t st, const SortedCopy* copy) {
+    const bool one = g.n_cells <= kReorderOneMax;
+    if (copy) {
+        if (one) launch_reorder_c<1, true>(b, cur, g, *copy, st);
+        else launch_reorder_c<kReorderCells, true>(b, cur, g, *copy, st);
+    } else if (one) {
+        launch_reorder_c<1, false>(b, cur, g, SortedCopy(), st);
+    } else {
+        launch_reorder_c<kReorderCells, false>(b, cur, g, SortedCopy(), st);
+    }
 }
 
 template <int B>

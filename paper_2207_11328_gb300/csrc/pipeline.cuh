@@ -276,7 +276,8 @@ constexpr int kReorderCells = 4;
 static_assert(kReorderCells >= 1 && kReorderCells <= 32, "one lane per cell");
 constexpr uint32_t kReorderOneMax = 32768;
 
-template <int kCells>
+// kCopy: the sorted state is also written to `copy` (a step of the backward pass' tape)
+template <int kCells, bool kCopy = false>
 __device__ __forceinline__ void reorder_body(
     const float4* __restrict__ pos, const float4* __restrict__ vel, const float* __restrict__ phat,
     const uint32_t* __restrict__ pinfo,
@@ -284,7 +285,8 @@ __device__ __forceinline__ void reorder_body(
     const SceneDev* __restrict__ scenes, uint32_t n_cells, DevStatus* __restrict__ st, uint32_t* __restrict__ cell_nfluid,
     float4* __restrict__ pos_o,
     float4* __restrict__ vel_o, float* __restrict__ phat_o, uint32_t* __restrict__ cell_o,
-    uint32_t* __restrict__ pinfo_o, uint32_t* __restrict__ pid_o, float* __restrict__ quads) {
+    uint32_t* __restrict__ pinfo_o, uint32_t* __restrict__ pid_o, float* __restrict__ quads,
+    const SortedCopy& copy = SortedCopy()) {
     const int lane = threadIdx.x & 31;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -354,6 +356,13 @@ __device__ __forceinline__ void reorder_body(
                     cell_o[d] = c;
                     pinfo_o[d] = s;
                     pid_o[d] = id;
+                    if constexpr (kCopy) {
+                        copy.pos[d] = p;
+                        copy.vel[d] = v;
+                        copy.phat[d] = h;
+                        copy.pinfo[d] = s;
+                        copy.pid[d] = id;
+                    }
                 }
             }
             if (lane == 0) cell_nfluid[c] = nfluid;

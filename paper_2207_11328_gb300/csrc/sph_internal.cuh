@@ -193,8 +193,8 @@ const char* forces_variant_name(int v);
 // cancellation near rest): phat_coef * delta * sum_k C(gamma,k) delta^(k-1) / (1+delta)^2.
 // Stored per particle by every kernel that writes delta, and recomputed from a
 // neighbour's delta by the tuned force kernels (one function, so both agree
-// bit for bit).  The quotient is __fdividef (reciprocal and product, within
-// 2 ulp for (1+delta)^2 in (2^-126, 2^126)): no slow-path call in the pair loop.
+// bit for bit).  The quotient is a product with rcp_fast: no slow-path call in the
+// pair loop.
 __device__ __forceinline__ float eos_phat(float d, const Phys& ph, float phat_coef) {
     float poly = ph.coef[7];
 #pragma unroll
@@ -280,6 +280,15 @@ struct Buffers {
     void* staging;           // upload/download staging (64 B per particle)
 };
 
+// where the reorder writes the sorted state a second time
+struct SortedCopy {
+    float4* pos = nullptr;
+    float4* vel = nullptr;
+    float* phat = nullptr;
+    uint32_t* pinfo = nullptr;
+    uint32_t* pid = nullptr;
+};
+
 struct Geometry {
     uint32_t cap;
     uint32_t n_cells;        // over all scenes (the sentinel bucket is n_cells)
@@ -309,7 +318,8 @@ void launch_hash(const Buffers& b, int cur, const Geometry& g, cudaStream_t st);
 // dt: the step's time-step update too, by a block of its own (every-step lists), else null
 void launch_scan(const Buffers& b, const Geometry& g, const DtArgs* dt, cudaStream_t st);
 void launch_scatter(const Buffers& b, const Geometry& g, cudaStream_t st);
-void launch_reorder(const Buffers& b, int cur, const Geometry& g, cudaStream_t st);
+// copy: the sorted state is written there too, else null
+void launch_reorder(const Buffers& b, int cur, const Geometry& g, cudaStream_t st, const SortedCopy* copy = nullptr);
 void launch_build(const Buffers& b, int cur, const Geometry& g, const Phys& ph, cudaStream_t st);
 uint32_t scan_blocks(uint32_t n_buckets);
 
@@ -333,7 +343,7 @@ void launch_adj_load(const AdjBuffers& a, uint32_t n, const float* xbar, const f
                      cudaStream_t st);
 void launch_adj_store(const AdjBuffers& a, uint32_t n, float* xbar, float* ubar, float* dbar, cudaStream_t st);
 // copies of n elements of `count` arrays (16-byte elements where wide[k], else 4-byte), one launch
-constexpr int kTapeArrays = 8;
+constexpr int kTapeArrays = 6;
 void launch_tape_copy(const void* const* src, void* const* dst, const bool* wide, int count, uint32_t n,
                       cudaStream_t st);
 
