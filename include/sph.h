@@ -332,9 +332,10 @@ int sph_tape_generation(sph_ctx* ctx, uint64_t* gen);
  * neighbour-build variant (one thread per particle with 128 or 256 threads
  * per block, or nine warps per 32 particles, a warp per row of neighbour
  * cells, with 2, 3 or 4 blocks per SM) and each
- * force-kernel shape (64, 128 or 256 threads per block with at most 64
- * registers; 4 or 8 lanes per particle) on the uploaded state (warps per row
- * and lanes per particle up to 131,072 particles), the
+ * force-kernel shape (128 or 256 threads per block with at most 64
+ * registers; and for small states 8 lanes per particle, or a thread per
+ * particle that evaluates 8 or 16 list entries together) on the uploaded
+ * state (the small states' shapes up to 131,072 particles), the
  * predictor and the corrector pass apart (3 timed launches each, CUDA events
  * on `stream`; the corrector runs on a scratch copy of the state), then the
  * list build and the predictor pass fused against apart (every-step list,

@@ -139,8 +139,7 @@ __device__ __forceinline__ void boundary_pair(uint32_t e, const Central& ci, con
 // every LANES-th entry's terms, then all lanes add the group's terms in list order, so the sums are
 // those of one thread, to the bit (the terms travel by shuffles: 6 a pair and lane).  For states too
 // small to fill the GPU with a thread per particle, where one thread's list is a long chain of
-// instructions: a pass over 4,096 particles 17 -> 7 us (8 lanes), 19,683 24 -> 13 us (4 lanes),
-// 71,680 32 -> 49 us (4 lanes).  terms(entry, tm) gives an entry's terms.
+// instructions: a pass over 4,096 particles 17 -> 7 us (8 lanes).  terms(entry, tm) gives an entry's terms.
 template <int VISC, int LANES, class F>
 __device__ __forceinline__ void lanes_sum(const uint2* __restrict__ lp, ptrdiff_t step, uint32_t cnt, uint32_t n,
                                           DevStatus* st, Acc& acc, F&& terms) {
@@ -206,7 +205,10 @@ __device__ __forceinline__ uint2 ld_chunk(const uint2* p) {
 
 // SKIN: nlist/ncount are the step's exact list in its four-entry chunks; the corrector also checks
 // and reduces the displacement since the list's build.
-template <int VISC, int MODE, bool SKIN, bool FRESH = false, int LANES = 1>
+// WIDE: list chunks of two entries evaluated together as long as the fluid part has so many left, their
+// gathers issued before the first is used.  A state that does not fill the GPU is bound by
+// that latency, and has the registers to spare (see launch_forces_v).
+template <int VISC, int MODE, bool SKIN, bool FRESH = false, int LANES = 1, int WIDE = 0>
 __device__ __forceinline__ void particle_pass(
     uint32_t i, uint32_t n, const float4* __restrict__ pos, const float4* __restrict__ vel,
     const float* __restrict__ phat, float4* io_pos, float4* io_vel, float* io_phat, float4* __restrict__ force_out,
@@ -302,8 +304,33 @@ __device__ __forceinline__ void particle_pass(
         // iteration ahead so that their latency is not on the path to the gathers
         const uint2* lp = reinterpret_cast<const uint2*>(nlist) + i;
         uint32_t k = 0;
+        if constexpr (WIDE > 0) {
+            constexpr uint32_t kRound = 2 * WIDE;
+            uint2 next[WIDE];
+            if (nf >= kRound)
+#pragma unroll
+                for (int c = 0; c < WIDE; ++c) next[c] = ld_chunk<FRESH>(lp + c * S);
+            for (; k + kRound <= nf; k += kRound, lp += WIDE * S) {
+                uint2 a[WIDE];
+                uint32_t top = 0u;
+#pragma unroll
+                for (int c = 0; c < WIDE; ++c) {
+                    a[c] = next[c];
+                    top = max(top, max(a[c].x, a[c].y));
+                }
+                if (k + 2 * kRound <= nf)
+#pragma unroll
+                    for (int c = 0; c < WIDE; ++c) next[c] = ld_chunk<FRESH>(lp + (WIDE + c) * S);
+                SPH_GUARD((top >> kCodeBits) < n, st, break)
+#pragma unroll
+                for (int c = 0; c < WIDE; ++c) {
+                    SPH_PAIR(false, a[c].x, acc);
+                    SPH_PAIR(false, a[c].y, acc);
+                }
+            }
+        }
         uint2 an = make_uint2(0u, 0u), bn = make_uint2(0u, 0u);
-        if (nf >= 4) {
+        if (k + 4 <= nf) {
             an = ld_chunk<FRESH>(lp);
             bn = ld_chunk<FRESH>(lp + S);
         }
@@ -436,7 +463,7 @@ __device__ __forceinline__ void particle_pass(
     }
 }
 
-template <int VISC, int MODE, bool SKIN, int LANES = 1>
+template <int VISC, int MODE, bool SKIN, int LANES = 1, int WIDE = 0>
 __device__ __forceinline__ void forces_body(
     const float4* __restrict__ pos, const float4* __restrict__ vel, const float* __restrict__ phat,
     float4* io_pos, float4* io_vel, float* io_phat, float4* __restrict__ force_out,
@@ -445,19 +472,19 @@ __device__ __forceinline__ void forces_body(
     int acc_dt, const float4* __restrict__ pos_ref, const uint32_t* __restrict__ pid) {
     const uint32_t n = st->n_active;
     for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) / LANES; i < n; i += gridDim.x * blockDim.x / LANES)
-        particle_pass<VISC, MODE, SKIN, false, LANES>(i, n, pos, vel, phat, io_pos, io_vel, io_phat, force_out, pinfo,
-                                                      nlist, ncount, scenes, dyn, st, ph, acc_dt, pos_ref, pid);
+        particle_pass<VISC, MODE, SKIN, false, LANES, WIDE>(i, n, pos, vel, phat, io_pos, io_vel, io_phat, force_out, pinfo,
+                                                            nlist, ncount, scenes, dyn, st, ph, acc_dt, pos_ref, pid);
 }
 
-template <int VISC, int MODE, int kBlock, int kMinBlocks, bool SKIN, int LANES>
+template <int VISC, int MODE, int kBlock, int kMinBlocks, bool SKIN, int LANES, int WIDE>
 __global__ void __launch_bounds__(kBlock, MODE == kForcesOnly ? (kMinBlocks * 2 + 2) / 3 : kMinBlocks) k_forces(
     const float4* __restrict__ pos, const float4* __restrict__ vel, const float* __restrict__ phat,
     float4* io_pos, float4* io_vel, float* io_phat, float4* __restrict__ force_out,
     const uint32_t* __restrict__ pinfo, const uint32_t* __restrict__ nlist, const uint32_t* __restrict__ ncount,
     const SceneDev* __restrict__ scenes, SceneDyn* __restrict__ dyn, DevStatus* __restrict__ st, const Phys ph,
     int acc_dt, const float4* __restrict__ pos_ref, const uint32_t* __restrict__ pid) {
-    forces_body<VISC, MODE, SKIN, LANES>(pos, vel, phat, io_pos, io_vel, io_phat, force_out, pinfo, nlist, ncount, scenes,
-                                         dyn, st, ph, acc_dt, pos_ref, pid);
+    forces_body<VISC, MODE, SKIN, LANES, WIDE>(pos, vel, phat, io_pos, io_vel, io_phat, force_out, pinfo, nlist, ncount,
+                                               scenes, dyn, st, ph, acc_dt, pos_ref, pid);
 }
 
 // ---------------------------------------------------------------------
@@ -651,7 +678,7 @@ __global__ void __launch_bounds__(kPipeBlock, kPersistMinBlocks) k_step_persiste
     }
 }
 
-template <int VISC, int B, int MB, bool SKIN, int LANES>
+template <int VISC, int B, int MB, bool SKIN, int LANES, int WIDE>
 void launch_forces_s(const Buffers& b, int cur, const Geometry& g, const Phys& ph, ForceMode mode, int acc_dt,
                      cudaStream_t st) {
     const unsigned grid = g.cap ? (unsigned)(((uint64_t)g.cap * LANES + B - 1) / B) : 1;
@@ -659,48 +686,51 @@ void launch_forces_s(const Buffers& b, int cur, const Geometry& g, const Phys& p
     const uint32_t* const count = SKIN ? b.ncount_x : b.ncount;
     switch (mode) {
         case kForcesOnly:
-            k_forces<VISC, kForcesOnly, B, MB, SKIN, LANES><<<grid, B, 0, st>>>(
+            k_forces<VISC, kForcesOnly, B, MB, SKIN, LANES, WIDE><<<grid, B, 0, st>>>(
                 b.pos[cur], b.vel[cur], b.phat[cur], nullptr, nullptr, nullptr, b.force, b.pinfo[cur], list, count,
                 b.scenes, b.dyn, b.status, ph, acc_dt, nullptr, b.pid[cur]);
             break;
         case kPredict:
-            k_forces<VISC, kPredict, B, MB, SKIN, LANES><<<grid, B, 0, st>>>(
+            k_forces<VISC, kPredict, B, MB, SKIN, LANES, WIDE><<<grid, B, 0, st>>>(
                 b.pos[cur], b.vel[cur], b.phat[cur], b.pos_s, b.vel_s, b.phat_s, nullptr, b.pinfo[cur], list, count,
                 b.scenes, b.dyn, b.status, ph, 0, nullptr, b.pid[cur]);
             break;
         case kCorrect:
-            k_forces<VISC, kCorrect, B, MB, SKIN, LANES><<<grid, B, 0, st>>>(
+            k_forces<VISC, kCorrect, B, MB, SKIN, LANES, WIDE><<<grid, B, 0, st>>>(
                 b.pos_s, b.vel_s, b.phat_s, b.pos[cur], b.vel[cur], b.phat[cur], nullptr, b.pinfo[cur], list, count,
                 b.scenes, b.dyn, b.status, ph, 0, b.pos_ref, b.pid[cur]);
             break;
     }
 }
 
-// (a skin list's passes run with one thread per particle)
-template <int VISC, int B, int MB, int LANES = 1>
+// (a skin list's passes take the plain shapes)
+template <int VISC, int B, int MB, int LANES = 1, int WIDE = 0>
 void launch_forces_b(const Buffers& b, int cur, const Geometry& g, const Phys& ph, ForceMode mode, int acc_dt,
                      cudaStream_t st) {
+    constexpr bool kPlain = LANES == 1 && WIDE == 0;
     if (b.pos_ref)
-        launch_forces_s<VISC, (LANES > 1 ? 128 : B), (LANES > 1 ? 8 : MB), true, 1>(b, cur, g, ph, mode, acc_dt, st);
+        launch_forces_s<VISC, (kPlain ? B : 128), (kPlain ? MB : 8), true, 1, 0>(b, cur, g, ph, mode, acc_dt, st);
     else
-        launch_forces_s<VISC, B, MB, false, LANES>(b, cur, g, ph, mode, acc_dt, st);
+        launch_forces_s<VISC, B, MB, false, LANES, WIDE>(b, cur, g, ph, mode, acc_dt, st);
 }
 
-// launch shapes of the force kernels (autotuned, the corrector pass on its own):
-// threads per block and the register cap implied by a minimum of resident blocks per SM; the
-// last two are groups of lanes per particle
+// Launch shapes of the force kernels (autotuned, the corrector pass on its own): threads per block, the
+// register cap implied by a minimum of resident blocks per SM, lanes per particle, list chunks
+// evaluated together.  States that do not fill the GPU keep more of a particle's pairs in flight, the
+// fewer particles the more.  us per step with 128 threads (1), 8 lanes (4), 16 entries a round (3),
+// 8 entries a round (0):
+//     4,096 particles  55.5  36.5  40.1  46.8      32,768 particles  75.4  96.6  61.9  64.2
+//     8,000            64.4  40.5  42.3  47.1      46,656            89.8   126  80.2  78.1
+//    12,167            65.2  54.4  44.0  50.5      64,000             101   162   111  95.2
+//    19,683            70.7  72.9  51.4  56.3      97,336             134   236   140   136
+// A pass over 1.65M takes 278 us with 1, 287 with 2, 315 with 0; over a 1.0M box 247 with 1, 244 with 2.
 template <int VISC>
 void launch_forces_v(const Buffers& b, int cur, const Geometry& g, const Phys& ph, ForceMode mode, int acc_dt,
                      cudaStream_t st) {
-    const int v = mode == kCorrect ? ph.forces_variant_c : ph.forces_variant;
-    if constexpr (has_diffusion(VISC)) {  // one thread shape beside the groups of lanes
-        if (v == 3) launch_forces_b<VISC, 128, 6, 4>(b, cur, g, ph, mode, acc_dt, st);
-        else if (v == 4) launch_forces_b<VISC, 128, 4, 8>(b, cur, g, ph, mode, acc_dt, st);
-        else launch_forces_b<VISC, 128, 8>(b, cur, g, ph, mode, acc_dt, st);
-    } else switch (v) {
-        case 0: launch_forces_b<VISC, 64, 16>(b, cur, g, ph, mode, acc_dt, st); break;
+    switch (mode == kCorrect ? ph.forces_variant_c : ph.forces_variant) {
+        case 0: launch_forces_b<VISC, 64, 10, 1, 4>(b, cur, g, ph, mode, acc_dt, st); break;
         case 2: launch_forces_b<VISC, 256, 4>(b, cur, g, ph, mode, acc_dt, st); break;
-        case 3: launch_forces_b<VISC, 128, 6, 4>(b, cur, g, ph, mode, acc_dt, st); break;
+        case 3: launch_forces_b<VISC, 32, 9, 1, 8>(b, cur, g, ph, mode, acc_dt, st); break;
         case 4: launch_forces_b<VISC, 128, 4, 8>(b, cur, g, ph, mode, acc_dt, st); break;
         default: launch_forces_b<VISC, 128, 8>(b, cur, g, ph, mode, acc_dt, st); break;
     }
@@ -786,9 +816,10 @@ void launch_forces(const Buffers& b, int cur, const Geometry& g, const Phys& ph,
 }
 
 const char* forces_variant_name(int v) {
-    static const char* names[kForcesVariants] = {"64 threads, <=64 regs", "128 threads, <=64 regs",
-                                                 "256 threads, <=64 regs", "4 lanes/particle (skin list: 1)",
-                                                 "8 lanes/particle (skin list: 1)"};
+    // (of a skin list: 128 threads but for the third)
+    static const char* names[kForcesVariants] = {"64 threads, 8 entries a round", "128 threads, <=64 regs",
+                                                 "256 threads, <=64 regs", "32 threads, 16 entries a round",
+                                                 "8 lanes/particle"};
     return v >= 0 && v < kForcesVariants ? names[v] : "?";
 }
 

@@ -112,8 +112,9 @@ void check_canaries(sph_ctx* c, cudaStream_t st) {
 
 inline cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
-constexpr uint32_t kRowBuildMax = 81920, kLanes8Max = 8192, kLanes4Max = 24576;  // see default_variants
-constexpr uint32_t kLanesTuneMax = 131072;  // sph_autotune times groups of lanes up to here
+// the largest particle counts of the small states' launch shapes (see default_variants)
+constexpr uint32_t kRowBuildMax = 81920, kLanesMax = 8192, kWide16Max = 40960, kWide8Max = 81920;
+constexpr uint32_t kSmallTuneMax = 131072;  // sph_autotune times those shapes up to here
 
 constexpr double kViscousDtCoef = 0.125;  // laminar viscous time-step limit, dt <= 0.125 h^2/nu
 
@@ -620,17 +621,22 @@ inline unsigned grid_for(uint32_t n, int block) {
 }
 
 // Default launch shapes for n particles, until sph_set_variants, sph_set_forces_variants or
-// sph_autotune choose: nine warps per 32 particles build the list, and 8 or 4 lanes per particle
-// evaluate the every-step passes, while a thread per particle would leave most of the GPU idle.
-// Measured on periodic boxes, us per step, thread against group: list build 98 / 71 at 4,096
-// particles, 114 / 94 at 32,768, 124 / 117 at 64,000, 166 / 174 at 125,000 (the line between); passes
-// by 8 lanes 69 / 48 at 4,096, by 4 lanes 86 / 73 at 19,683, 98 / 107 at 32,768 (the line between);
-// 8 lanes against 4: 65 / 70 at 8,000, 68 / 60 at 12,167.
+// sph_autotune choose.  Nine warps per 32 particles build the list while a thread per particle would
+// leave most of the GPU idle: us per step on periodic boxes, thread against warps, 98 / 71 at 4,096
+// particles, 114 / 94 at 32,768, 124 / 117 at 64,000, 166 / 174 at 125,000 (the line between).  The
+// every-step passes of states that do not fill the GPU keep more of a particle's pairs in flight; the
+// figures on both sides of each line stand at launch_forces_v (forces.cu).
+int default_forces(uint32_t n) {
+    if (n <= kLanesMax) return 4;
+    if (n <= kWide16Max) return 3;
+    return n <= kWide8Max ? 0 : 1;
+}
+
 void default_variants(sph_ctx* c, uint32_t n) {
     Phys ph = c->ph;
     if (c->auto_build) ph.build_variant = n <= kRowBuildMax ? 4 : 0;
     if (c->auto_forces)
-        ph.forces_variant = ph.forces_variant_c = skin_mode(c) || c->ph.general ? 1 : (n <= kLanes8Max ? 4 : (n <= kLanes4Max ? 3 : 1));
+        ph.forces_variant = ph.forces_variant_c = skin_mode(c) || c->ph.general ? 1 : default_forces(n);
     if (ph.build_variant == c->ph.build_variant && ph.forces_variant == c->ph.forces_variant &&
         ph.forces_variant_c == c->ph.forces_variant_c)
         return;
@@ -1068,8 +1074,8 @@ int sph_autotune(sph_ctx* c, void* stream, int* build_variant, int* forces_varia
     // the in-cell sort (a skin list forces its gated pipeline open)
     if (skin_mode(c)) launch_force_rebuild(c->b, st);
     enqueue_build(c, st);
-    // (a group of lanes per particle is for small states: not timed where it cannot win)
-    const bool large = c->n_uploaded > kLanesTuneMax;
+    // (the small states' shapes are not timed where they cannot win)
+    const bool large = c->n_uploaded > kSmallTuneMax;
     for (int v = 0; v < (large ? 2 : kBuildVariants); ++v) {
         c->ph.build_variant = v;
         const float ms = time_ms([&] { launch_build(c->b, c->cur, c->g, c->ph, st); });
@@ -1080,11 +1086,12 @@ int sph_autotune(sph_ctx* c, void* stream, int* build_variant, int* forces_varia
     }
     c->ph.build_variant = best_v;
     launch_build(c->b, c->cur, c->g, c->ph, st);
-    // force kernels: threads per block and register cap
+    // force kernels: the plain shapes, and the small states'
     int best_f = c->ph.forces_variant;
     best = 3.4e38f;
-    const int n_shapes = large || skin_mode(c) ? 3 : kForcesVariants;
-    for (int v = 0; v < n_shapes; ++v) {
+    std::vector<int> shapes{1, 2};
+    if (!large && !skin_mode(c) && !c->ph.general) shapes = {0, 1, 2, 3, 4};
+    for (int v : shapes) {
         c->ph.forces_variant = v;
         // the predictor pass as the step runs it (it writes only the predicted-state scratch)
         const float ms = time_ms([&] { launch_forces(c->b, c->cur, c->g, c->ph, kPredict, 0, st); });
@@ -1116,7 +1123,7 @@ int sph_autotune(sph_ctx* c, void* stream, int* build_variant, int* forces_varia
         tb.vel[c->cur] = c->b.vel[alt];
         tb.phat[c->cur] = c->b.phat[alt];
         best = 3.4e38f;
-        for (int v = 0; v < n_shapes; ++v) {
+        for (int v : shapes) {
             c->ph.forces_variant_c = v;
             const float ms = time_ms([&] { launch_forces(tb, c->cur, c->g, c->ph, kCorrect, 0, st); });
             if (ms < best) {
