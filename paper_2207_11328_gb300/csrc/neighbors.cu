@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(1024) k_scan_bsums(uint32_t* __restrict__ bsum
     scan_bsums_body(bsum, nblocks);
 }
 
-__global__ void __launch_bounds__(1024) k_scan_one(uint32_t* __restrict__ count, uint32_t nb,
+__global__ void __launch_bounds__(1024, 1) k_scan_one(uint32_t* __restrict__ count, uint32_t nb,
                                                    uint32_t* __restrict__ start, DevStatus* __restrict__ st,
                                                    const DtArgs dt, const uint32_t* __restrict__ gate) {
     if (blockIdx.x == 1) {

@@ -151,13 +151,63 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* total)
     return res;
 }
 
+// A thread's kScanItems consecutive counts, zero past the last bucket: in 16-byte loads (the tables and
+// the thread's first bucket are aligned), but for the thread that holds the table's end.  A load and two
+// stores of 4 bytes per bucket, 32 bytes apart over a warp, took three kernels 20.3 us on the 1.65M dam
+// break (536,257 buckets; now 16.6) and 85 us on 20.1M (now 36), the one-block scan of 4,117 buckets
+// 10.4 us (now 7.5).
+__device__ __forceinline__ void scan_load(const uint32_t* __restrict__ count, uint32_t nb, uint32_t base, uint32_t* v) {
+    static_assert(kScanItems == 8, "two 16-byte words");
+    if (base < nb && nb - base >= (uint32_t)kScanItems) {
+        const uint4 a = *reinterpret_cast<const uint4*>(count + base), b = *reinterpret_cast<const uint4*>(count + base + 4);
+        v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+        v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
+    } else {
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k) v[k] = base < nb && (uint32_t)k < nb - base ? count[base + k] : 0u;
+    }
+}
+
+// the starts of those buckets, from the first one's; their counts zeroed; the thread that holds the
+// last bucket, the sentinel of removed particles, publishes the particle counts
+__device__ __forceinline__ void scan_store(uint32_t* __restrict__ count, uint32_t nb, uint32_t* __restrict__ start,
+                                           DevStatus* __restrict__ st, uint32_t base, uint32_t run, const uint32_t* v) {
+    if (base >= nb) return;
+    const uint32_t left = nb - base;
+    uint32_t o[kScanItems];
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+        o[k] = run;
+        run += v[k];
+    }
+    if (left >= (uint32_t)kScanItems) {
+        *reinterpret_cast<uint4*>(start + base) = make_uint4(o[0], o[1], o[2], o[3]);
+        *reinterpret_cast<uint4*>(start + base + 4) = make_uint4(o[4], o[5], o[6], o[7]);
+        *reinterpret_cast<uint4*>(count + base) = make_uint4(0u, 0u, 0u, 0u);
+        *reinterpret_cast<uint4*>(count + base + 4) = make_uint4(0u, 0u, 0u, 0u);
+    }
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+        if (left < (uint32_t)kScanItems && (uint32_t)k < left) {
+            start[base + k] = o[k];
+            count[base + k] = 0u;
+        }
+        if ((uint32_t)k + 1u == left) {
+            start[nb] = o[k] + v[k];
+            st->n_sorted = o[k];
+            st->n_removed += v[k];
+        }
+    }
+}
+
 __device__ __forceinline__ void scan_reduce_tile(const uint32_t* __restrict__ count, uint32_t nb,
                                                  uint32_t* __restrict__ bsum, uint32_t tile) {
     const uint32_t base = tile * kScanTile + threadIdx.x * kScanItems;
+    uint32_t v[kScanItems];
+    scan_load(count, nb, base, v);
     uint32_t s = 0;
 #pragma unroll
-    for (int k = 0; k < kScanItems; ++k)
-        if (base + k < nb) s += count[base + k];
+    for (int k = 0; k < kScanItems; ++k) s += v[k];
     uint32_t total;
     block_excl_scan(s, &total);
     if (threadIdx.x == 0) bsum[tile] = total;
@@ -181,29 +231,13 @@ __device__ __forceinline__ void scan_down_tile(uint32_t* __restrict__ count, uin
                                                DevStatus* __restrict__ st, uint32_t tile) {
     const uint32_t base = tile * kScanTile + threadIdx.x * kScanItems;
     uint32_t v[kScanItems];
+    scan_load(count, nb, base, v);
     uint32_t s = 0;
 #pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        v[k] = base + k < nb ? count[base + k] : 0u;
-        s += v[k];
-    }
+    for (int k = 0; k < kScanItems; ++k) s += v[k];
     uint32_t total;
-    uint32_t run = block_excl_scan(s, &total) + bsum[tile];
-#pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        const uint32_t b = base + k;
-        if (b < nb) {
-            start[b] = run;
-            count[b] = 0u;
-            if (b == nb - 1) {
-                // bucket nb-1 is the sentinel of removed particles
-                start[nb] = run + v[k];
-                st->n_sorted = run;
-                st->n_removed += v[k];
-            }
-        }
-        run += v[k];
-    }
+    const uint32_t run = block_excl_scan(s, &total) + bsum[tile];
+    scan_store(count, nb, start, st, base, run, v);
 }
 
 // the whole scan by one block of 1024 threads, for few buckets
@@ -215,29 +249,14 @@ __device__ __forceinline__ void scan_one_body(uint32_t* __restrict__ count, uint
     for (uint32_t base0 = 0; base0 < nb; base0 += blockDim.x * kScanItems) {
         const uint32_t base = base0 + threadIdx.x * kScanItems;
         uint32_t v[kScanItems];
+        scan_load(count, nb, base, v);
         uint32_t s = 0;
 #pragma unroll
-        for (int k = 0; k < kScanItems; ++k) {
-            v[k] = base + k < nb ? count[base + k] : 0u;
-            s += v[k];
-        }
+        for (int k = 0; k < kScanItems; ++k) s += v[k];
         uint32_t total;
-        uint32_t run = block_excl_scan(s, &total) + carry;
+        const uint32_t run = block_excl_scan(s, &total) + carry;
         carry += total;
-#pragma unroll
-        for (int k = 0; k < kScanItems; ++k) {
-            const uint32_t b = base + k;
-            if (b < nb) {
-                start[b] = run;
-                count[b] = 0u;
-                if (b == nb - 1) {  // the sentinel of removed particles
-                    start[nb] = run + v[k];
-                    st->n_sorted = run;
-                    st->n_removed += v[k];
-                }
-            }
-            run += v[k];
-        }
+        scan_store(count, nb, start, st, base, run, v);
     }
 }
 
