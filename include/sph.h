@@ -259,8 +259,9 @@ int sph_next_dt(sph_ctx* ctx, double* dt, void* stream);
  * or as two (0): each thread writes its particle's list (the thread-per-
  * particle build) and evaluates the predictor pass over it at once, while
  * the list and the candidates it has just tested are in cache.  The same list
- * and the same results, to the bit.  sph_autotune fuses them when that is at
- * least 2% faster.  Only with the list rebuilt every step and the default model
+ * and the same results, to the bit.  Until this call, sph_autotune (which
+ * fuses them when that is at least 2% faster) or a build variant set, each
+ * upload of more than 2.5 million particles fuses them.  Only with the list rebuilt every step and the default model
  * (SPH_ERR_ARG otherwise); the paper runs the two as separate commands
  * (Section 3 "Code structure").  Synchronises the device. */
 int sph_set_fused_predict(sph_ctx* ctx, int on);
@@ -338,7 +339,7 @@ int sph_tape_generation(sph_ctx* ctx, uint64_t* gen);
  * state (the small states' shapes up to 131,072 particles), the
  * predictor and the corrector pass apart (3 timed launches each, CUDA events
  * on `stream`; the corrector runs on a scratch copy of the state), then the
- * list build and the predictor pass fused against apart (every-step list,
+ * list build and the predictor pass fused (128 or 256 threads) against apart (every-step list,
  * default model), keeps the fastest and re-captures the step graph on the
  * next sph_step.  The
  * particle state and the next time step are as before the call (the list
@@ -350,7 +351,9 @@ int sph_autotune(sph_ctx* ctx, void* stream, int* build_variant, int* forces_var
 
 /* Select the neighbour-build variant (0..4) and the force-kernel launch shape
  * (0..4, for every pass) directly, as sph_autotune would (-1 keeps the
- * current one); until then each upload picks them by the particle count.
+ * current one; a build variant set ends the fusion that an upload chose, see
+ * sph_set_fused_predict); until then each upload picks them by the particle
+ * count.
  * Every variant computes the same bits.  Synchronises the
  * device; SPH_ERR_ARG for an index out of range. */
 int sph_set_variants(sph_ctx* ctx, int build_variant, int forces_variant);

@@ -609,8 +609,8 @@ __global__ void k_dt(const DtArgs a) { dt_body(a); }
 // list and, pair for pair in the same order, the same sums and update as the
 // two kernels.  List rebuilt every step (no skin), default model.
 // ---------------------------------------------------------------------
-template <int VISC>
-__global__ void __launch_bounds__(kPipeBlock, 4) k_build_predict(const Buffers b, int cur, const Phys ph) {
+template <int VISC, int kBlockT>
+__global__ void __launch_bounds__(kBlockT, 1024 / kBlockT) k_build_predict(const Buffers b, int cur, const Phys ph) {
     DevStatus* st = b.status;
     const uint32_t n = st->n_active;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -856,11 +856,17 @@ cudaError_t launch_step_persistent(const Buffers& b, int cur, const Geometry& g,
 }
 
 void launch_build_predict(const Buffers& b, int cur, const Geometry& g, const Phys& ph, cudaStream_t st) {
-    const unsigned grid = g.cap ? (g.cap + kPipeBlock - 1) / kPipeBlock : 1;
-    if (ph.visc == SPH_VISC_LAMINAR)
-        k_build_predict<SPH_VISC_LAMINAR><<<grid, kPipeBlock, 0, st>>>(b, cur, ph);
-    else
-        k_build_predict<SPH_VISC_ARTIFICIAL><<<grid, kPipeBlock, 0, st>>>(b, cur, ph);
+    const auto go = [&](auto kernel, unsigned block) {
+        kernel<<<g.cap ? (g.cap + block - 1) / block : 1, block, 0, st>>>(b, cur, ph);
+    };
+    const bool laminar = ph.visc == SPH_VISC_LAMINAR;
+    if (ph.fuse_predict == 256) {
+        if (laminar) go(k_build_predict<SPH_VISC_LAMINAR, 256>, 256);
+        else go(k_build_predict<SPH_VISC_ARTIFICIAL, 256>, 256);
+    } else {
+        if (laminar) go(k_build_predict<SPH_VISC_LAMINAR, 128>, 128);
+        else go(k_build_predict<SPH_VISC_ARTIFICIAL, 128>, 128);
+    }
 }
 
 void launch_dt_peek(const Buffers& b, const Phys& ph, cudaStream_t st) {

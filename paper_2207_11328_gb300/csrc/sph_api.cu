@@ -56,7 +56,7 @@ struct sph_ctx {
     uint64_t run_steps = 0;  // steps of the calls that run_graph could serve, since the graphs were dropped
     uint32_t graph_nodes = 0;
     // build variant / force shapes by the rule on the particle count (false: set or tuned)
-    bool auto_build = true, auto_forces = true;
+    bool auto_build = true, auto_forces = true, auto_fuse = true;
     bool persistent = false;  // sph_set_persistent: one cooperative launch per sph_step call
     size_t staging_bytes = 0;
     std::vector<std::pair<char*, size_t>> canaries;  // checked build: (base, bytes) of guarded buffers
@@ -114,6 +114,7 @@ inline cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
 // the largest particle counts of the small states' launch shapes (see default_variants)
 constexpr uint32_t kRowBuildMax = 81920, kLanesMax = 8192, kWide16Max = 40960, kWide8Max = 81920;
+constexpr uint32_t kTpp128Max = 524288, kApartMax = 2500000;  // and of large ones
 constexpr uint32_t kSmallTuneMax = 131072;  // sph_autotune times those shapes up to here
 
 constexpr double kViscousDtCoef = 0.125;  // laminar viscous time-step limit, dt <= 0.125 h^2/nu
@@ -626,6 +627,16 @@ inline unsigned grid_for(uint32_t n, int block) {
 // particles, 114 / 94 at 32,768, 124 / 117 at 64,000, 166 / 174 at 125,000 (the line between).  The
 // every-step passes of states that do not fill the GPU keep more of a particle's pairs in flight; the
 // figures on both sides of each line stand at launch_forces_v (forces.cu).
+// Large states, us per step: the thread build in blocks of 128 / of 256 / fused with the predictor in
+// blocks of 128 (the build waits on issue, the pass on its gathers: mixed on an SM they overlap, where
+// the particles are mostly fluid) / of 256:
+//   dam break 572,120  397 /  395 /  407 /  406    box 1,030,301   954 /  942 /  920 /  907
+//           1,647,828 1082 / 1066 / 1068 / 1068        2,097,152  1963 / 1912 / 1854 / 1808
+//           2,817,201 1950 / 1900 / 1873 / 1856    tanks 2,030,211 1320 / 1301 / 1320 / 1339
+//           4,250,593 3010 / 2920 / 2865 / 2827          6,573,863 4083 / 4098 / 4073 / 4185
+//          20,139,024 15.52 / 15.35 / 14.82 / 14.80 ms
+// so blocks of 256 above half a million, and the fused kernel above 2.5 million, in the shape that lost
+// nowhere.  A build variant or fusion that was set or tuned stays.
 int default_forces(uint32_t n) {
     if (n <= kLanesMax) return 4;
     if (n <= kWide16Max) return 3;
@@ -634,11 +645,12 @@ int default_forces(uint32_t n) {
 
 void default_variants(sph_ctx* c, uint32_t n) {
     Phys ph = c->ph;
-    if (c->auto_build) ph.build_variant = n <= kRowBuildMax ? 4 : 0;
+    if (c->auto_fuse) ph.fuse_predict = c->auto_build && n > kApartMax && can_fuse(c) ? 128 : 0;
+    if (c->auto_build) ph.build_variant = n <= kRowBuildMax ? 4 : (n <= kTpp128Max ? 0 : 1);
     if (c->auto_forces)
         ph.forces_variant = ph.forces_variant_c = skin_mode(c) || c->ph.general ? 1 : default_forces(n);
     if (ph.build_variant == c->ph.build_variant && ph.forces_variant == c->ph.forces_variant &&
-        ph.forces_variant_c == c->ph.forces_variant_c)
+        ph.forces_variant_c == c->ph.forces_variant_c && ph.fuse_predict == c->ph.fuse_predict)
         return;
     c->ph = ph;
     drop_graphs(c);  // captured launches carry the old shapes
@@ -1028,14 +1040,15 @@ int sph_set_fused_predict(sph_ctx* c, int on) {
     if (!c) return SPH_ERR_ARG;
     if (on && !can_fuse(c)) return SPH_ERR_ARG;
     CK(cudaDeviceSynchronize());
-    c->ph.fuse_predict = on ? 1 : 0;
+    c->ph.fuse_predict = on ? 256 : 0;
+    c->auto_fuse = false;
     drop_graphs(c);
     return SPH_OK;
 }
 
 int sph_get_step_options(sph_ctx* c, int* fused_predict, int* persistent) {
     if (!c) return SPH_ERR_ARG;
-    if (fused_predict) *fused_predict = c->ph.fuse_predict;
+    if (fused_predict) *fused_predict = c->ph.fuse_predict ? 1 : 0;
     if (persistent) *persistent = c->persistent ? 1 : 0;
     return SPH_OK;
 }
@@ -1137,16 +1150,21 @@ int sph_autotune(sph_ctx* c, void* stream, int* build_variant, int* forces_varia
     c->ph.forces_variant_c = best_c;
     // the list build and the predictor pass as one kernel, or apart (every-step list, default model)
     if (can_fuse(c)) {
-        Phys pf = c->ph, ps = c->ph;
-        pf.fuse_predict = 1;
-        ps.fuse_predict = 0;
-        const float t_sep = time_ms([&] { enqueue_build_predict(c, ps, st); });
-        const float t_fused = time_ms([&] { enqueue_build_predict(c, pf, st); });
-        // fused only when clearly faster (measured equal within noise on the dam breaks: 20.1M
-        // particles 11.94 against 8.39 + 3.56 ms, 1.65M 0.869 against 0.576 + 0.270 ms)
-        c->ph.fuse_predict = t_fused < 0.98f * t_sep ? 1 : 0;
+        // (fused only when clearly faster; figures at default_variants)
+        Phys ph = c->ph;
+        ph.fuse_predict = 0;
+        float best_ms = 0.98f * time_ms([&] { enqueue_build_predict(c, ph, st); });
+        c->ph.fuse_predict = 0;
+        for (int threads : {128, 256}) {
+            ph.fuse_predict = threads;
+            const float ms = time_ms([&] { enqueue_build_predict(c, ph, st); });
+            if (ms < best_ms) {
+                best_ms = ms;
+                c->ph.fuse_predict = threads;
+            }
+        }
     }
-    c->auto_build = c->auto_forces = false;
+    c->auto_build = c->auto_forces = c->auto_fuse = false;
     c->fresh = true;  // the last build is of the current positions
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1185,6 +1203,7 @@ int sph_set_variants(sph_ctx* c, int build_variant, int forces_variant) {
     if (build_variant >= 0) {
         c->ph.build_variant = build_variant;
         c->auto_build = false;
+        if (c->auto_fuse) c->ph.fuse_predict = 0;  // the variant asked for
     }
     if (forces_variant >= 0) c->auto_forces = false;
     if (forces_variant >= 0) c->ph.forces_variant = c->ph.forces_variant_c = forces_variant;

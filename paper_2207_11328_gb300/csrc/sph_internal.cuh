@@ -161,7 +161,7 @@ struct Phys {
     int forces_variant;      // launch shape of the forces-only and predictor passes (autotuned), see
                              //   forces_variant_name
     int forces_variant_c;    // launch shape of the corrector pass (autotuned on its own)
-    int fuse_predict;        // the list build and the predictor pass as one kernel (autotuned)
+    int fuse_predict;        // the list build and the predictor pass as one kernel: its threads per block, or 0
     // model options (Table 1); general != 0 selects the kernels of forces_models.cu (density
     // diffusion alone does not)
     int general;

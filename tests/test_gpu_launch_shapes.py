@@ -130,3 +130,23 @@ def test_runs_of_steps_equal_single_steps(skin):
     sa, sb = a.stats(), b.stats()
     assert sa["steps"] == sb["steps"] == 48 and sa["time"] == sb["time"] and sa["builds"] == sb["builds"]
     assert sa["kernels_per_step"] == sb["kernels_per_step"]
+
+
+@pytest.mark.parametrize("n_axis", [9, 137])
+def test_fused_build_and_predictor_by_size(n_axis):
+    """The fused kernel that large uploads choose (2.57 million particles), and the one asked for: the bits
+    of the two kernels; a build variant set ends the choice."""
+    s = scenes.periodic_box(n_per_axis=n_axis, dp=0.02)
+    large = s.n > 2_500_000
+    a, f = sim_for(s), sim_for(s)
+    assert f.step_options()["fused_predict"] == large
+    a.set_variants(build=1)
+    assert not a.step_options()["fused_predict"]
+    if not large:
+        f.set_fused_predict(True)
+    for sim in (a, f):
+        sim.step(3)
+    for x, y in zip(a.download(), f.download()):
+        assert np.array_equal(x, y)
+    sa, sf = a.stats(), f.stats()
+    assert sa["list_entries"] == sf["list_entries"] and sa["dt"] == sf["dt"]
