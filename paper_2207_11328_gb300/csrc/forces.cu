@@ -608,6 +608,9 @@ __global__ void k_dt(const DtArgs a) { dt_body(a); }
 // just loaded are in cache; no separate pass re-reads the list.  The same
 // list and, pair for pair in the same order, the same sums and update as the
 // two kernels.  List rebuilt every step (no skin), default model.
+// The build waits on instruction issue and the pass on its gathers; mixed on an SM they overlap: 1.0M box
+// 942 -> 907 us a step, 20.1M dam break 15.35 -> 14.80 ms; not where many warps hold wall particles
+// (figures by size and block at default_variants, sph_api.cu).
 // ---------------------------------------------------------------------
 template <int VISC, int kBlockT>
 __global__ void __launch_bounds__(kBlockT, 1024 / kBlockT) k_build_predict(const Buffers b, int cur, const Phys ph) {
