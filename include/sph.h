@@ -314,8 +314,10 @@ int sph_record(sph_ctx* ctx, uint32_t T, uint32_t K, void* stream, double* dt_ou
  * dL/dalpha.  Boundary particles' x and u are constants (zero adjoint).
  * Each segment of K steps is recomputed from its checkpoint and reversed
  * step by step; the vector-Jacobian products are gathers over the
- * symmetric neighbour lists (deterministic, no atomics).  Leaves the
- * context at the recorded initial state.  Synchronises `stream`. */
+ * symmetric neighbour lists (deterministic, no atomics).  n is the recorded
+ * upload's, and so is the gradient, whatever was uploaded, stepped or removed
+ * since.  Leaves the context at the recorded initial state (its n again for
+ * the downloads).  Synchronises `stream`. */
 int sph_backward(sph_ctx* ctx, const float* xbar_T, const float* ubar_T, const float* dbar_T, float* xbar_0,
                  float* ubar_0, float* dbar_0, double* alphabar, void* stream);
 

@@ -209,6 +209,7 @@ class Simulation:
         self._h = h
         self.params = params
         self.n = 0
+        self._n_recorded = 0
         if scenes_desc:
             arr = (SceneDesc * len(scenes_desc))()
             for k, d in enumerate(scenes_desc):
@@ -409,6 +410,7 @@ class Simulation:
         """T steps with frozen dt and a checkpoint every K steps; returns dt."""
         dt = ctypes.c_double()
         _check(_lib().sph_record(self._h, int(T), int(K), _stream_handle(stream), ctypes.byref(dt)), "sph_record")
+        self._n_recorded = self.n
         return dt.value
 
     def tape_generation(self):
@@ -418,20 +420,22 @@ class Simulation:
         return g.value
 
     def backward(self, xbar_T=None, ubar_T=None, dbar_T=None, want_x=False, want_delta=False, stream=None):
-        """Adjoint of the last record: torch CUDA float32 inputs (n,3)/(n,) or None;
-        returns (dL/dx0 or None, dL/du0, dL/ddelta0 or None, dL/dalpha)."""
+        """Adjoint of the last record: torch CUDA float32 inputs (n,3)/(n,) or None, n particles as
+        recorded; returns (dL/dx0 or None, dL/du0, dL/ddelta0 or None, dL/dalpha)."""
         import torch
-        n = self.n
+        n = self._n_recorded
         dev = torch.device("cuda", torch.cuda.current_device())
         p = lambda t: None if t is None else ctypes.c_void_p(t.data_ptr())  # noqa: E731
         for t in (xbar_T, ubar_T, dbar_T):
             assert t is None or (t.is_cuda and t.dtype == torch.float32 and t.is_contiguous())
+            assert t is None or t.numel() >= (n if t is dbar_T else 3 * n)  # (fewer would be read past their end)
         ubar0 = torch.empty((n, 3), dtype=torch.float32, device=dev)
         xbar0 = torch.empty((n, 3), dtype=torch.float32, device=dev) if want_x else None
         dbar0 = torch.empty((n,), dtype=torch.float32, device=dev) if want_delta else None
         ab = ctypes.c_double()
         _check(_lib().sph_backward(self._h, p(xbar_T), p(ubar_T), p(dbar_T), p(xbar0), p(ubar0), p(dbar0),
                                    ctypes.byref(ab), _stream_handle(stream)), "sph_backward")
+        self.n = n  # the context holds the recorded initial state again
         return xbar0, ubar0, dbar0, ab.value
 
     PHASES = ("dt", "hash", "scan", "scatter", "reorder", "build", "forces_predict", "forces_correct")

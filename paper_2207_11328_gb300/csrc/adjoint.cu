@@ -113,7 +113,8 @@ __global__ void k_adj_pre(const float4* __restrict__ pos, const float4* __restri
 }
 
 // Tape copies: n elements of each of `count` arrays (16- or 4-byte elements)
-// between the particle buffers and a flat tape block, one launch per copy.
+// between the particle buffers and a flat tape block, one launch per copy.  st (a restored state,
+// else null): the particle counts are the tape's again too, whatever was uploaded or removed since.
 struct TapeCopy {
     const void* src[kTapeArrays];
     void* dst[kTapeArrays];
@@ -121,7 +122,11 @@ struct TapeCopy {
     int count;
 };
 
-__global__ void k_tape_copy(const TapeCopy tc, uint32_t n) {
+__global__ void k_tape_copy(const TapeCopy tc, uint32_t n, DevStatus* st, uint32_t n_removed) {
+    if (st && blockIdx.x == 0 && threadIdx.x == 0) {
+        st->n_active = n;
+        st->n_removed = n_removed;
+    }
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
 #pragma unroll
         for (int k = 0; k < kTapeArrays; ++k) {
@@ -388,7 +393,7 @@ __global__ void k_adj_sum_alpha(const float4* __restrict__ ub_id, uint32_t n, do
 }  // namespace
 
 void launch_tape_copy(const void* const* src, void* const* dst, const bool* wide, int count, uint32_t n,
-                      cudaStream_t st) {
+                      DevStatus* status, uint32_t n_removed, cudaStream_t st) {
     TapeCopy tc{};
     tc.count = count;
     for (int k = 0; k < count && k < kTapeArrays; ++k) {
@@ -396,7 +401,7 @@ void launch_tape_copy(const void* const* src, void* const* dst, const bool* wide
         tc.dst[k] = dst[k];
         tc.wide |= wide[k] ? (1u << k) : 0u;
     }
-    k_tape_copy<<<grid_for(n ? n : 1, 256), 256, 0, st>>>(tc, n);
+    k_tape_copy<<<grid_for(n ? n : 1, 256), 256, 0, st>>>(tc, n, status, n_removed);
 }
 
 void launch_adj_load(const AdjBuffers& a, uint32_t n, const float* xbar, const float* ubar, const float* dbar,

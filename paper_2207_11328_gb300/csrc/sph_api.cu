@@ -18,7 +18,8 @@ struct AdjTape {
     bool valid = false;
     uint64_t gen = 0;          // generation of the valid recording (0: none)
     uint64_t next_gen = 1;     // the next sph_record's generation
-    uint32_t T = 0, K = 0, n = 0;
+    uint32_t T = 0, K = 0, n = 0;               // n: active particles (the size of every array below)
+    uint32_t n_uploaded = 0, n_removed = 0;     // of the state that was recorded
     double dt = 0.0;
     Phys ph_rec{};
     std::vector<char*> ckpt;   // T/K checkpoints (pos4 vel4 phat cell pinfo pid)
@@ -1238,8 +1239,9 @@ void free_tape(sph_ctx* c) {
     t.gen = 0;
 }
 
-// copy the particle arrays of buffer `cur` to / from a flat device block (one launch)
-void tape_io(const std::vector<std::pair<void*, size_t>>& arrays, char* blk, bool save, cudaStream_t st, uint32_t n) {
+// copy the particle arrays of buffer `cur` to / from a flat device block (one launch); a restored state
+// brings its particle counts
+void tape_io(sph_ctx* c, const std::vector<std::pair<void*, size_t>>& arrays, char* blk, bool save, cudaStream_t st, uint32_t n) {
     const void* src[kTapeArrays];
     void* dst[kTapeArrays];
     bool wide[kTapeArrays];
@@ -1252,15 +1254,15 @@ void tape_io(const std::vector<std::pair<void*, size_t>>& arrays, char* blk, boo
         off += align_up(a.second * n, 256);
         ++k;
     }
-    launch_tape_copy(src, dst, wide, k, n, st);
+    launch_tape_copy(src, dst, wide, k, n, save ? nullptr : c->b.status, c->tape.n_removed, st);
 }
 
 // checkpoint: the sorted state of buffer cur (positions, velocities, P/rho^2, cell, scene, id)
 void state_io(sph_ctx* c, char* blk, bool save, cudaStream_t st, uint32_t n) {
     Buffers& b = c->b;
     const int k = c->cur;
-    tape_io({{b.pos[k], sizeof(float4)}, {b.vel[k], sizeof(float4)}, {b.phat[k], sizeof(float)},
-             {b.cell[k], sizeof(uint32_t)}, {b.pinfo[k], sizeof(uint32_t)}, {b.pid[k], sizeof(uint32_t)}},
+    tape_io(c, {{b.pos[k], sizeof(float4)}, {b.vel[k], sizeof(float4)}, {b.phat[k], sizeof(float)},
+                {b.cell[k], sizeof(uint32_t)}, {b.pinfo[k], sizeof(uint32_t)}, {b.pid[k], sizeof(uint32_t)}},
             blk, save, st, n);
 }
 
@@ -1451,6 +1453,8 @@ int sph_record(sph_ctx* c, uint32_t T, uint32_t K, void* stream, double* dt_out)
     t.T = T;
     t.K = K;
     t.n = n;
+    t.n_uploaded = c->n_uploaded;
+    t.n_removed = hs.n_removed;
     t.dt = dt;
     t.ph_rec = c->ph;
     t.ph_rec.dt_fixed = dt;
@@ -1510,6 +1514,8 @@ int sph_backward(sph_ctx* c, const float* xbar_T, const float* ubar_T, const flo
     if (!t.valid || !c->uploaded) return SPH_ERR_STATE;
     cudaStream_t st = S(stream);
     const uint32_t n = t.n;
+    c->n_uploaded = t.n_uploaded;  // the recorded particles from here on, whatever was uploaded since
+    default_variants(c, t.n_uploaded);
     launch_adj_load(t.a, n, xbar_T, ubar_T, dbar_T, st);
     for (int seg = (int)(t.T / t.K) - 1; seg >= 0; --seg) {
         // the segment's checkpoint, then its recompute and reverse (one captured graph:

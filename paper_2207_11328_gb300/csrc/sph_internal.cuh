@@ -342,10 +342,11 @@ void launch_adj_sum_alpha(const AdjBuffers& a, uint32_t n, double* out, cudaStre
 void launch_adj_load(const AdjBuffers& a, uint32_t n, const float* xbar, const float* ubar, const float* dbar,
                      cudaStream_t st);
 void launch_adj_store(const AdjBuffers& a, uint32_t n, float* xbar, float* ubar, float* dbar, cudaStream_t st);
-// copies of n elements of `count` arrays (16-byte elements where wide[k], else 4-byte), one launch
+// copies of n elements of `count` arrays (16-byte elements where wide[k], else 4-byte), one launch;
+// status (a restored state, else null): its particle counts are set to n and n_removed
 constexpr int kTapeArrays = 6;
 void launch_tape_copy(const void* const* src, void* const* dst, const bool* wide, int count, uint32_t n,
-                      cudaStream_t st);
+                      DevStatus* status, uint32_t n_removed, cudaStream_t st);
 
 // forces.cu
 enum ForceMode { kForcesOnly = 0, kPredict = 1, kCorrect = 2 };

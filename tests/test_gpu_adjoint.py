@@ -7,6 +7,7 @@ image), target = initial positions + seeded N(0, (0.1 dp)^2); dt frozen.
 Tolerance: |g.v - J(v)| <= 1e-3 max(|J(v)|, rms_v |J|) for seeded unit
 directions v in u0 space, and the same for d/dalpha.
 """
+import dataclasses
 import multiprocessing as mp
 
 import numpy as np
@@ -174,3 +175,50 @@ def _gpu_grad_sum(s, T, K):
                 torch.tensor(s.ptype), T=T, K=K)
     x.sum().backward()
     return None, u0.grad.cpu().numpy(), float(al.grad), sim
+
+
+@pytest.mark.parametrize("between", ["smaller", "larger", "removal"])
+def test_backward_after_another_state_was_uploaded(between):
+    # the recording outlives later uploads of fewer or more particles, and a particle leaving the
+    # domain in later steps: backward restores the recorded state with its particle count, so its
+    # gradient is that of the uninterrupted run, and the context is back at that state
+    import torch
+    big = scenes.dam_break(dp=0.05)
+    big.dt_fixed = 4e-4
+    s = scenes.subset(big, (big.ptype == 1) | (np.arange(big.n) % 3 > 0))
+    few = scenes.subset(big, np.arange(big.n) % 3 == 0)
+    rng = np.random.default_rng(3)
+    xb = torch.tensor(rng.normal(size=(s.n, 3)), dtype=torch.float32, device="cuda")
+
+    def recorded():
+        sim = sim_for(s, max_particles=big.n)
+        sim.record(6, 3)
+        return sim
+
+    def grads(sim):
+        gx, gu, gd, ga = sim.backward(xbar_T=xb, want_x=True, want_delta=True)
+        return [t.cpu().numpy() for t in (gx, gu, gd)] + [np.array(ga)]
+
+    ref = grads(recorded())
+    sim = recorded()
+    if between == "removal":
+        # one particle placed at the open top with a speed that takes it out
+        up = dataclasses.replace(s, pos=s.pos.copy(), vel=s.vel.copy())
+        k = int(np.flatnonzero(s.ptype == 0)[0])
+        up.pos[k] = [0.5 * s.size[0] + s.origin[0], 0.5 * s.size[1] + s.origin[1], s.origin[2] + s.size[2] - 0.01 * s.dp]
+        up.vel[k] = [0, 0, 200.0]
+        sim.upload(up)
+        sim.step(4)
+        assert sim.stats()["n_active"] == s.n - 1
+    else:
+        sim.upload(few if between == "smaller" else big)
+        sim.step(2)
+    for a, b in zip(grads(sim), ref):
+        assert np.array_equal(a, b)
+    st = sim.stats()
+    assert st["n_active"] == s.n and st["n_removed"] == 0
+    fresh = sim_for(s, max_particles=big.n)
+    for a, b in zip(sim.download(), fresh.download()):
+        assert a.shape == b.shape and np.array_equal(a, b)
+    for a, b in zip(grads(sim), ref):  # a second reversal of the recording
+        assert np.array_equal(a, b)
