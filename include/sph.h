@@ -173,7 +173,7 @@ int sph_create(const sph_params* p, sph_ctx** out);
 /* Replace the scene table by n_scenes independent scenes (batched stepping).
  * Must precede sph_upload; reallocates the cell tables (host call, syncs).
  * Each scene keeps its own grid, sound speed, dt and time; scenes never
- * interact. */
+ * interact.  Invalidates a recording (sph_record). */
 int sph_set_scenes(sph_ctx* ctx, uint32_t n_scenes, const sph_scene* scenes);
 
 /* Upload n particles from HOST arrays (copied):
@@ -323,7 +323,8 @@ int sph_backward(sph_ctx* ctx, const float* xbar_T, const float* ubar_T, const f
 
 /* Generation of the recording sph_backward would reverse: every successful
  * sph_record numbers its tape 1, 2, 3, ... per context; *gen = 0 when no
- * valid recording exists (none yet, a failed sph_record, sph_set_alpha).
+ * valid recording exists (none yet, a failed sph_record, sph_set_alpha,
+ * sph_set_scenes).
  * A caller that holds several recordings' results (e.g. an autograd graph
  * with two rollouts on one context) stores the generation after its
  * sph_record and checks it before sph_backward: a mismatch means the tape

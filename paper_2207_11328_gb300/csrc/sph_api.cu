@@ -472,6 +472,26 @@ void drop_graphs(sph_ctx* c) {
             }
 }
 
+void free_tape(sph_ctx* c) {
+    AdjTape& t = c->tape;
+    for (char* p : t.ckpt) cudaFree(p);
+    t.ckpt.clear();
+    cudaFree(t.steps);
+    cudaFree(t.lists);
+    cudaFree(t.adj_mem);
+    t.steps = nullptr;
+    t.lists = nullptr;
+    t.adj_mem = nullptr;
+    for (auto* gs : {t.seg_graph, t.rec_graph})
+        for (int k = 0; k < 2; ++k)
+            if (gs[k]) {
+                cudaGraphExecDestroy(gs[k]);
+                gs[k] = nullptr;
+            }
+    t.valid = false;
+    t.gen = 0;
+}
+
 inline bool skin_mode(const sph_ctx* c) { return c->p.rebuild_every > 1; }
 
 int alloc_cells(sph_ctx* c) {
@@ -512,6 +532,7 @@ int set_scene_table(sph_ctx* c, uint32_t n, const sph_scene* sc) {
         }
     if (centres.size() >= 0xFFFFFFFFull) return SPH_ERR_ARG;
     drop_graphs(c);
+    free_tape(c);  // its graphs hold the old cell tables, its states cells of the old grid
     free_cells(c);
     c->scenes_h = tab;
     c->centres_h = centres;
@@ -1218,26 +1239,6 @@ const char* sph_build_variant_name(int variant) { return build_variant_name(vari
 const char* sph_forces_variant_name(int variant) { return forces_variant_name(variant); }
 
 namespace {
-
-void free_tape(sph_ctx* c) {
-    AdjTape& t = c->tape;
-    for (char* p : t.ckpt) cudaFree(p);
-    t.ckpt.clear();
-    cudaFree(t.steps);
-    cudaFree(t.lists);
-    cudaFree(t.adj_mem);
-    t.steps = nullptr;
-    t.lists = nullptr;
-    t.adj_mem = nullptr;
-    for (auto* gs : {t.seg_graph, t.rec_graph})
-        for (int k = 0; k < 2; ++k)
-            if (gs[k]) {
-                cudaGraphExecDestroy(gs[k]);
-                gs[k] = nullptr;
-            }
-    t.valid = false;
-    t.gen = 0;
-}
 
 // copy the particle arrays of buffer `cur` to / from a flat device block (one launch); a restored state
 // brings its particle counts

@@ -222,3 +222,32 @@ def test_backward_after_another_state_was_uploaded(between):
         assert a.shape == b.shape and np.array_equal(a, b)
     for a, b in zip(grads(sim), ref):  # a second reversal of the recording
         assert np.array_equal(a, b)
+
+
+def test_a_new_scene_table_ends_the_recording():
+    # the recording's graphs hold the old grid's tables: backward refuses after sph_set_scenes, and a
+    # recording of the same shape made on the new table has the gradients of a context of its own
+    import ctypes
+    import torch
+    from paper_2207_11328_gb300 import SceneDesc, SphError, _lib
+    s, _ = _box(8)
+    xb = torch.tensor(np.random.default_rng(4).normal(size=(s.n, 3)), dtype=torch.float32, device="cuda")
+
+    def grad(sim):
+        sim.record(4, 2)
+        return sim.backward(xbar_T=xb)[1].cpu().numpy()
+
+    ref = grad(sim_for(s))
+    sim = sim_for(s)
+    assert np.array_equal(grad(sim), ref)
+    assert sim.tape_generation() > 0
+    d = SceneDesc()
+    d.origin[:], d.size[:] = list(s.origin), list(s.size)
+    d.periodic_mask, d.c0 = s.periodic, s.c0
+    assert _lib().sph_set_scenes(sim._h, 1, ctypes.byref(d)) == 0
+    assert sim.tape_generation() == 0
+    sim.upload(s)
+    with pytest.raises(SphError) as e:
+        sim.backward(xbar_T=xb)
+    assert e.value.code == -8
+    assert np.array_equal(grad(sim), ref)
