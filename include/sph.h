@@ -316,7 +316,8 @@ int sph_record(sph_ctx* ctx, uint32_t T, uint32_t K, void* stream, double* dt_ou
  * step by step; the vector-Jacobian products are gathers over the
  * symmetric neighbour lists (deterministic, no atomics).  n is the recorded
  * upload's, and so is the gradient, whatever was uploaded, stepped or removed
- * since.  Leaves the context at the recorded initial state (its n again for
+ * since.  A particle that had left the domain before the recording has no
+ * part in it: its adjoints come back as given.  Leaves the context at the recorded initial state (its n again for
  * the downloads).  Synchronises `stream`. */
 int sph_backward(sph_ctx* ctx, const float* xbar_T, const float* ubar_T, const float* dbar_T, float* xbar_0,
                  float* ubar_0, float* dbar_0, double* alphabar, void* stream);

@@ -1517,7 +1517,8 @@ int sph_backward(sph_ctx* c, const float* xbar_T, const float* ubar_T, const flo
     const uint32_t n = t.n;
     c->n_uploaded = t.n_uploaded;  // the recorded particles from here on, whatever was uploaded since
     default_variants(c, t.n_uploaded);
-    launch_adj_load(t.a, n, xbar_T, ubar_T, dbar_T, st);
+    // adjoints in upload order: ids go up to the uploaded count, also where particles were removed since
+    launch_adj_load(t.a, t.n_uploaded, xbar_T, ubar_T, dbar_T, st);
     for (int seg = (int)(t.T / t.K) - 1; seg >= 0; --seg) {
         // the segment's checkpoint, then its recompute and reverse (one captured graph:
         // the same work for every segment, on the same tape buffers)
@@ -1537,8 +1538,8 @@ int sph_backward(sph_ctx* c, const float* xbar_T, const float* ubar_T, const flo
         CK(cudaGraphLaunch(t.seg_graph[p0], st));
         c->cur = t.seg_end_cur[p0];
     }
-    launch_adj_store(t.a, n, xbar_0, ubar_0, dbar_0, st);
-    launch_adj_sum_alpha(t.a, n, t.a.alpha_sum, st);
+    launch_adj_store(t.a, t.n_uploaded, xbar_0, ubar_0, dbar_0, st);
+    launch_adj_sum_alpha(t.a, t.n_uploaded, t.a.alpha_sum, st);
     double ab = 0.0;
     CK(cudaMemcpyAsync(&ab, t.a.alpha_sum, sizeof(double), cudaMemcpyDeviceToHost, st));
     // leave the context at the recorded initial state, with its cell tables and list
