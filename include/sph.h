@@ -336,7 +336,8 @@ int sph_tape_generation(sph_ctx* ctx, uint64_t* gen);
 /* Autotuner (launch shapes only; results are unchanged): times each
  * neighbour-build variant (one thread per particle with 128 or 256 threads
  * per block, or nine warps per 32 particles, a warp per row of neighbour
- * cells, with 2, 3 or 4 blocks per SM) and each
+ * cells, with 2, 3 or 4 blocks per SM; those with lists of up to 256
+ * entries, max_neibs) and each
  * force-kernel shape (128 or 256 threads per block with at most 64
  * registers; and for small states 8 lanes per particle, or a thread per
  * particle that evaluates 8 or 16 list entries together) on the uploaded

@@ -606,7 +606,6 @@ __device__ __forceinline__ void build_tpp_body(
 // thread's build.
 constexpr int kRowWarps = 9;
 constexpr int kRowBlock = 32 * kRowWarps;
-constexpr uint32_t kStageNeibs = 256;
 // shared words: the tile's lists (an odd stride apart: lanes of a warp write different banks), the
 // hits of every row and particle
 __host__ __device__ constexpr uint32_t rows_list_words(uint32_t max_neibs) { return max_neibs | 1u; }

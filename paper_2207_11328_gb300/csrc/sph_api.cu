@@ -646,7 +646,10 @@ inline unsigned grid_for(uint32_t n, int block) {
 // Default launch shapes for n particles, until sph_set_variants, sph_set_forces_variants or
 // sph_autotune choose.  Nine warps per 32 particles build the list while a thread per particle would
 // leave most of the GPU idle: us per step on periodic boxes, thread against warps, 98 / 71 at 4,096
-// particles, 114 / 94 at 32,768, 124 / 117 at 64,000, 166 / 174 at 125,000 (the line between).  The
+// particles, 114 / 94 at 32,768, 124 / 117 at 64,000, 166 / 174 at 125,000 (the line between).  Lists too
+// long for its shared memory take a thread per particle at any size: the warps fall back to one in
+// nine (us per step with max_neibs 320, thread against warps: 73 / 82 at 4,096, 87 / 145 at 32,768,
+// 106 / 259 at 64,000).  The
 // every-step passes of states that do not fill the GPU keep more of a particle's pairs in flight; the
 // figures on both sides of each line stand at launch_forces_v (forces.cu).
 // Large states, us per step: the thread build in blocks of 128 / of 256 / fused with the predictor in
@@ -668,7 +671,8 @@ int default_forces(uint32_t n) {
 void default_variants(sph_ctx* c, uint32_t n) {
     Phys ph = c->ph;
     if (c->auto_fuse) ph.fuse_predict = c->auto_build && n > kApartMax && can_fuse(c) ? 128 : 0;
-    if (c->auto_build) ph.build_variant = n <= kRowBuildMax ? 4 : (n <= kTpp128Max ? 0 : 1);
+    if (c->auto_build)
+        ph.build_variant = n <= kRowBuildMax && ph.max_neibs <= kStageNeibs ? 4 : (n <= kTpp128Max ? 0 : 1);
     if (c->auto_forces)
         ph.forces_variant = ph.forces_variant_c = skin_mode(c) || c->ph.general ? 1 : default_forces(n);
     if (ph.build_variant == c->ph.build_variant && ph.forces_variant == c->ph.forces_variant &&
@@ -1111,7 +1115,7 @@ int sph_autotune(sph_ctx* c, void* stream, int* build_variant, int* forces_varia
     enqueue_build(c, st);
     // (the small states' shapes are not timed where they cannot win)
     const bool large = c->n_uploaded > kSmallTuneMax;
-    for (int v = 0; v < (large ? 2 : kBuildVariants); ++v) {
+    for (int v = 0; v < (large || c->ph.max_neibs > kStageNeibs ? 2 : kBuildVariants); ++v) {
         c->ph.build_variant = v;
         const float ms = time_ms([&] { launch_build(c->b, c->cur, c->g, c->ph, st); });
         if (ms < best) {

@@ -181,6 +181,7 @@ __device__ __forceinline__ bool cfl_counts(const Phys& ph, const uint32_t* __res
 }
 
 constexpr int kBuildVariants = 5;
+constexpr uint32_t kStageNeibs = 256;  // longest list that the build by rows of cells (variants 2..4) keeps in shared memory
 // Quads: four consecutive sorted particles' x, then their y, then their z (48 bytes), which the
 // list build loads as three 16-byte words from one address.
 __host__ __device__ constexpr size_t quad_word(uint32_t i) { return (size_t)(i >> 2) * 12u + (i & 3u); }  // x; y, z at + 4, + 8

@@ -150,3 +150,13 @@ def test_fused_build_and_predictor_by_size(n_axis):
         assert np.array_equal(x, y)
     sa, sf = a.stats(), f.stats()
     assert sa["list_entries"] == sf["list_entries"] and sa["dt"] == sf["dt"]
+
+
+@pytest.mark.parametrize("max_neibs,rows", [(256, True), (257, False)])
+def test_lists_too_long_for_shared_memory_take_the_thread_build(max_neibs, rows):
+    """The default of a small state, and what tuning may choose, by list length."""
+    s = scenes.periodic_box(n_per_axis=16)
+    sim = sim_for(s, max_neibs=max_neibs)
+    assert sim.variants()["build"].startswith("warp/row" if rows else "thread/particle")
+    sim.autotune()
+    assert rows or sim.variants()["build"].startswith("thread/particle")
