@@ -603,9 +603,13 @@ __device__ __forceinline__ void build_tpp_body(
 // instructions a particle against 224).  Before, a warp per particle with a lane per cell: 11, 36, 102 us
 // (1,019 instructions, every lane at an address of its own); nine lanes per particle: 11, 33, 91 us.
 // A tile beside a cell of over 64 candidate slots, and lists of over kStageNeibs entries, take the one
-// thread's build.
+// thread's build, after the block's other tiles: marked in ncount, one tile per warp.  (By the first warp, at
+// once: 556 us for 79,507 particles at h = 1.9 dp, every tile of them; now 222, a thread per particle 144.
+// The marks keep the main loop's registers: with the put-off tiles in registers the three-block shape spilled,
+// 2 to 3% of a step.)
 constexpr int kRowWarps = 9;
 constexpr int kRowBlock = 32 * kRowWarps;
+constexpr uint32_t kPutOff = ~0u;  // a list count that no list has
 // shared words: the tile's lists (an odd stride apart: lanes of a warp write different banks), the
 // hits of every row and particle
 __host__ __device__ constexpr uint32_t rows_list_words(uint32_t max_neibs) { return max_neibs | 1u; }
@@ -675,6 +679,8 @@ __device__ __forceinline__ void build_rows_body(
     const uint32_t r2lim = __float_as_uint(R2) - 1u;
     const f2 mR2 = f2_dup(-R2);
     uint32_t most = 0, sum = 0;  // of this lane's particles
+    __shared__ uint32_t put_off;
+    if (threadIdx.x == 0) put_off = 0u;
     for (uint32_t i0 = blockIdx.x * 32u; i0 < n; i0 += gridDim.x * 32u) {
         const uint32_t i = i0 + (uint32_t)lane;
         const bool have = i < n;
@@ -720,13 +726,9 @@ __device__ __forceinline__ void build_rows_body(
             }
         }
         const bool crowded = e[0] > (b[0] & ~3u) + 64u || e[1] > (b[1] & ~3u) + 64u || e[2] > (b[2] & ~3u) + 64u;
-        if (__syncthreads_or(crowded || !can_stage)) {
-            if (r == 0 && have) {
-                uint32_t nfound;
-                sum += build_particle_alone(i, pos, quads, cell, pinfo, start, cell_nfluid, scenes, nlist, ncount, R2,
-                                            max_neibs, stride, &nfound, st, n);
-                most = max(most, nfound);
-            }
+        if (__syncthreads_or(crowded || !can_stage)) {  // put off
+            if (r == 0 && have) ncount[i] = kPutOff;
+            if (threadIdx.x == 0) put_off = 1u;
             continue;
         }
         // hits of the row's three cells, up to 64 candidate slots each; fluid candidates first in a cell
@@ -806,14 +808,23 @@ __device__ __forceinline__ void build_rows_body(
         }
         __syncthreads();  // the shared lists are free again
     }
-    if (r == 0) {
-        most = __reduce_max_sync(0xffffffffu, most);
-        sum = __reduce_add_sync(0xffffffffu, sum);
-        if (lane == 0 && most) {
-            if (most > max_neibs) atomicOr(&st->error_bits, SPH_EBIT_NEIB_OVERFLOW);
-            atomicMax(&st->max_neibs_seen, most);
-            atomicAdd(&st->list_entries, (unsigned long long)sum);
+    __syncthreads();
+    if (put_off) {  // the block's tiles one by one over its warps
+        for (uint32_t i = (blockIdx.x + (uint32_t)r * gridDim.x) * 32u + (uint32_t)lane; i < n;
+             i += kRowWarps * gridDim.x * 32u) {
+            if (ncount[i] != kPutOff) continue;
+            uint32_t nfound;
+            sum += build_particle_alone(i, pos, quads, cell, pinfo, start, cell_nfluid, scenes, nlist, ncount, R2,
+                                        max_neibs, stride, &nfound, st, n);
+            most = max(most, nfound);
         }
+    }
+    most = __reduce_max_sync(0xffffffffu, most);
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    if (lane == 0 && most) {
+        if (most > max_neibs) atomicOr(&st->error_bits, SPH_EBIT_NEIB_OVERFLOW);
+        atomicMax(&st->max_neibs_seen, most);
+        atomicAdd(&st->list_entries, (unsigned long long)sum);
     }
 }
 
