@@ -799,7 +799,7 @@ void launch_conservation(const Buffers& b, int cur, double* scratch, cudaStream_
 
 void launch_forces(const Buffers& b, int cur, const Geometry& g, const Phys& ph, ForceMode mode, int acc_dt,
                    cudaStream_t st) {
-    if (b.pos_ref && mode != kCorrect)  // a skin list: first the step's exact list
+    if (b.pos_ref && mode != kCorrect && !ph.general)  // a skin list: first the step's exact list
         k_exact_list<<<g.cap ? (g.cap + 127) / 128 : 1, 128, 0, st>>>(
             b.pos[cur], b.pinfo[cur], b.nlist, b.ncount, b.scenes, b.status, ph.R2, ph.max_neibs, ph.stride,
             mode == kPredict, b.nlist_x, b.ncount_x);

@@ -1,6 +1,6 @@
 // Interaction kernels for the model options of Table 1 beyond the default
-// (Wendland C2, formulation 1, artificial or Morris/harmonic viscosity, no
-// density diffusion, which forces.cu runs with tuned launch shapes):
+// (Wendland C2, formulation 1, artificial or Morris/harmonic viscosity, which
+// forces.cu runs with tuned launch shapes, with density diffusion too):
 //
 //   kernels (kernel-templates listing, Section 4), F = aF f(q):
 //     Wendland (q-2)^3; cubic spline -3 + 9/4 q (q<1), -3/4 (2-q)^2/q (q<2);
@@ -20,9 +20,9 @@
 //
 // Same structure as the tuned kernels: one thread per particle, split
 // neighbour list read four entries (two chunks) ahead, aF applied once per particle, the
-// predictor/corrector epilogue of forces_common.cuh.  The kernel and the
-// viscous model are template parameters; formulation, averaging, diffusion
-// and the skin list are uniform run-time switches.
+// predictor/corrector epilogue of forces_common.cuh.  The kernel, the viscous
+// model and the kind of list are template parameters; formulation, averaging
+// and diffusion are uniform run-time switches.
 #include "forces_common.cuh"
 
 namespace sphg {
@@ -55,20 +55,29 @@ __device__ __forceinline__ float visc_weight(int op, float ri, float rj) {
     return __fdividef(2.0f, ri + rj);
 }
 
-// one neighbour of a fluid particle (BND: boundary neighbour, negated mass, u_j = 0)
-template <int KT, int VISC, bool BND>
-__device__ __forceinline__ void model_pair(uint32_t e, const Central& ci, const float4& vi, float phat_i, float ri,
-                                           const float4* __restrict__ pos, const float4* __restrict__ vel,
-                                           const float* __restrict__ phat, float pi_coef, float dd_coef,
-                                           const Phys& ph, Acc& acc) {
+// what a pair gathers of its neighbour
+struct Neib {
+    float4 p, v;
+    float h;
+};
+__device__ __forceinline__ Neib gather(uint32_t e, const float4* __restrict__ pos, const float4* __restrict__ vel,
+                                       const float* __restrict__ phat) {
     const uint32_t j = e >> kCodeBits;
-    const float4 pj = pos[j];
-    const float4 vj = vel[j];
-    const float phat_j = phat[j];
+    return Neib{pos[j], vel[j], phat[j]};
+}
+
+// one neighbour of a fluid particle (BND: boundary neighbour, negated mass, u_j = 0); FILTER: pairs beyond
+// the cutoff are left out.  Returns whether the pair is within it
+template <int KT, int VISC, bool BND, bool FILTER>
+__device__ __forceinline__ bool model_pair(uint32_t e, const Central& ci, const float4& vi, float phat_i, float ri,
+                                           const Neib& nb, float pi_coef, float dd_coef, const Phys& ph, Acc& acc) {
+    const float4 pj = nb.p, vj = nb.v;
+    const float phat_j = nb.h;
     const float rx = pick(e, ci.xm, ci.x0, ci.xp) - pj.x;
     const float ry = pick(e >> 2, ci.ym, ci.y0, ci.yp) - pj.y;
     const float rz = pick(e >> 4, ci.zm, ci.z0, ci.zp) - pj.z;
     const float r2 = fmaxf(fmaf(rx, rx, fmaf(ry, ry, rz * rz)), 1e-30f);
+    if (FILTER && !(r2 < ph.R2)) return false;
     const float rinv = rsqrtf(r2);
     const float mF = (BND ? -pj.w : pj.w) * kernel_shape<KT>(r2, rinv, ph);  // m_j F / aF
     const float rj = 1.0f + vj.w;
@@ -106,17 +115,31 @@ __device__ __forceinline__ void model_pair(uint32_t e, const Central& ci, const 
             acc.az = fmaf(lx, rz, acc.az);
         }
     }
+    return true;
 }
 
-template <int KT, int VISC, int MODE>
-__global__ void __launch_bounds__(kModelBlock, 4) k_forces_m(
+// The list of a pass: rebuilt every step; a skin list, whose pairs beyond the cutoff the pass leaves out
+// (the predictor keeps the others for the corrector and counts them); the list so kept, in chunks of
+// four entries.  A pass that tests its pairs costs less here than a list kernel before it: 1.65M dam break,
+// skin 0.3 h, cubic spline / second formulation: predictor 496 / 516 us against 622 / 606, accelerations
+// alone 442 / 456 against 578 / 600.
+// Bound by the gathers through L1, with as many warps as fit: two pairs' gathers at a time in 64
+// registers (8 blocks, spills of up to 32 bytes).  Accelerations alone over the skin list with four at a time
+// in 96 registers 548 / 574, with one at a time in 64 476 / 511; over a list of every step, by one kernel for
+// both kinds of list, 384 / 405, now 334 / 328.
+enum ModelList { kListEvery, kListSkin, kListExact };
+
+template <int KT, int VISC, int MODE, int LIST>
+__global__ void __launch_bounds__(kModelBlock, 8) k_forces_m(
     const float4* __restrict__ pos, const float4* __restrict__ vel, const float* __restrict__ phat,
     float4* io_pos, float4* io_vel, float* io_phat, float4* __restrict__ force_out,
     const uint32_t* __restrict__ pinfo, const uint32_t* __restrict__ nlist, const uint32_t* __restrict__ ncount,
     const SceneDev* __restrict__ scenes, SceneDyn* __restrict__ dyn, DevStatus* __restrict__ st, const Phys ph,
-    int acc_dt, int skin, const float4* __restrict__ pos_ref, const uint32_t* __restrict__ pid) {
-    // skin: nlist/ncount are the step's exact list, in chunks of four entries
+    int acc_dt, const float4* __restrict__ pos_ref, uint32_t* __restrict__ nlist_x, uint32_t* __restrict__ ncount_x,
+    const uint32_t* __restrict__ pid) {
+    constexpr bool FILTER = LIST == kListSkin, KEEP = FILTER && MODE == kPredict, EXACT = LIST == kListExact;
     const uint32_t n = st->n_active;
+    uint32_t kept = 0;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const uint32_t s = pinfo[i];
         const SceneDev& sc = scenes[s];
@@ -131,21 +154,27 @@ __global__ void __launch_bounds__(kModelBlock, 4) k_forces_m(
         const size_t S = ph.stride;
         Acc acc{0.f, 0.f, 0.f, 0.f};
         const uint32_t kxb = exact_bnd_chunk(ph.max_neibs);
+        ChunkWriter xf{make_uint4(0u, 0u, 0u, 0u), 0u, reinterpret_cast<uint4*>(nlist_x) + i, S};
+        ChunkWriter xb{make_uint4(0u, 0u, 0u, 0u), 0u, reinterpret_cast<uint4*>(nlist_x) + (size_t)kxb * S + i, S};
         auto fluid_entry = [&](uint32_t k) -> uint32_t {
-            return skin ? __ldg(nlist + ((size_t)(k >> 2) * S + i) * 4 + (k & 3u)) : __ldg(nlist + list_fluid_word(k, i, S));
+            return EXACT ? __ldg(nlist + ((size_t)(k >> 2) * S + i) * 4 + (k & 3u)) : __ldg(nlist + list_fluid_word(k, i, S));
         };
         auto bnd_entry = [&](uint32_t k) -> uint32_t {
-            return skin ? __ldg(nlist + ((size_t)(kxb + (k >> 2)) * S + i) * 4 + (k & 3u))
+            return EXACT ? __ldg(nlist + ((size_t)(kxb + (k >> 2)) * S + i) * 4 + (k & 3u))
                         : __ldg(nlist + list_bnd_word(k, i, S, ph.max_neibs));
         };
         if (fluid_i) {
             const float phat_i = phat[i];
             const float pic = sc.pi_coef, ddc = sc.dd_coef;
             uint32_t k = 0;
-#define SPH_PAIR(BND, e) model_pair<KT, VISC, BND>(e, ci, vi, phat_i, ri, pos, vel, phat, pic, ddc, ph, acc)
+#define SPH_PAIR(BND, e, nb)                                                                   \
+    do {                                                                                       \
+        if (model_pair<KT, VISC, BND, FILTER>(e, ci, vi, phat_i, ri, nb, pic, ddc, ph, acc) && KEEP) \
+            (BND ? xb : xf).put(true, e);                                                      \
+    } while (0)
             for (; k + 4 <= nf; k += 4) {
                 uint2 a, b;
-                if (skin) {
+                if (EXACT) {
                     const uint4 q = __ldg(reinterpret_cast<const uint4*>(nlist) + (size_t)(k >> 2) * S + i);
                     a = make_uint2(q.x, q.y);
                     b = make_uint2(q.z, q.w);
@@ -155,20 +184,26 @@ __global__ void __launch_bounds__(kModelBlock, 4) k_forces_m(
                     b = __ldg(lp + S);
                 }
                 SPH_GUARD((max(max(a.x, a.y), max(b.x, b.y)) >> kCodeBits) < n, st, break)
-                SPH_PAIR(false, a.x);
-                SPH_PAIR(false, a.y);
-                SPH_PAIR(false, b.x);
-                SPH_PAIR(false, b.y);
+                {
+                    const Neib n0 = gather(a.x, pos, vel, phat), n1 = gather(a.y, pos, vel, phat);
+                    SPH_PAIR(false, a.x, n0);
+                    SPH_PAIR(false, a.y, n1);
+                }
+                {
+                    const Neib n0 = gather(b.x, pos, vel, phat), n1 = gather(b.y, pos, vel, phat);
+                    SPH_PAIR(false, b.x, n0);
+                    SPH_PAIR(false, b.y, n1);
+                }
             }
             for (; k < nf; ++k) {
                 const uint32_t e = fluid_entry(k);
                 SPH_GUARD((e >> kCodeBits) < n, st, continue)
-                SPH_PAIR(false, e);
+                SPH_PAIR(false, e, gather(e, pos, vel, phat));
             }
             for (k = 0; k < nb; ++k) {
                 const uint32_t e = bnd_entry(k);
                 SPH_GUARD((e >> kCodeBits) < n, st, continue)
-                SPH_PAIR(true, e);
+                SPH_PAIR(true, e, gather(e, pos, vel, phat));
             }
 #undef SPH_PAIR
             acc.ax = fmaf(ph.aF, acc.ax, ph.g[0]);
@@ -189,6 +224,8 @@ __global__ void __launch_bounds__(kModelBlock, 4) k_forces_m(
                 const float ry = pick(e >> 2, ci.ym, ci.y0, ci.yp) - pj.y;
                 const float rz = pick(e >> 4, ci.zm, ci.z0, ci.zp) - pj.z;
                 const float r2 = fmaxf(fmaf(rx, rx, fmaf(ry, ry, rz * rz)), 1e-30f);
+                if (FILTER && !(r2 < ph.R2)) continue;
+                if (KEEP) xf.put(true, e);
                 float mF = pj.w * kernel_shape<KT>(r2, rsqrtf(r2), ph);
                 if (form2) mF *= __fdividef(ri, 1.0f + vj.w);
                 const float udx = -fmaf(vj.x, rx, fmaf(vj.y, ry, vj.z * rz));
@@ -196,8 +233,18 @@ __global__ void __launch_bounds__(kModelBlock, 4) k_forces_m(
             }
             acc.drho *= ph.aF;
         }
+        if (KEEP) {
+            xf.flush();
+            xb.flush();
+            ncount_x[i] = xf.n | (xb.n << 16);
+            kept += xf.n + xb.n;
+        }
         finish_particle<MODE>(i, s, sc, pi, vi, fluid_i, acc, io_pos, io_vel, io_phat, force_out, dyn, st, ph,
                               acc_dt, pos_ref, pid);
+    }
+    if (KEEP) {
+        const uint32_t w = __reduce_add_sync(0xffffffffu, kept);
+        if ((threadIdx.x & 31) == 0 && w) atomicAdd(&st->interactions, (unsigned long long)w);
     }
 }
 
@@ -205,25 +252,29 @@ template <int KT, int VISC>
 void launch_m(const Buffers& b, int cur, const Geometry& g, const Phys& ph, ForceMode mode, int acc_dt,
               cudaStream_t st) {
     const unsigned grid = g.cap ? (g.cap + kModelBlock - 1) / kModelBlock : 1;
-    const bool skin = b.pos_ref != nullptr;  // then the step's exact list
-    const uint32_t* const list = skin ? b.nlist_x : b.nlist;
-    const uint32_t* const count = skin ? b.ncount_x : b.ncount;
+    const bool skin = b.pos_ref != nullptr;
     switch (mode) {
-        case kForcesOnly:
-            k_forces_m<KT, VISC, kForcesOnly><<<grid, kModelBlock, 0, st>>>(
-                b.pos[cur], b.vel[cur], b.phat[cur], nullptr, nullptr, nullptr, b.force, b.pinfo[cur], list, count,
-                b.scenes, b.dyn, b.status, ph, acc_dt, skin, nullptr, b.pid[cur]);
+        case kForcesOnly: {
+            const auto k = skin ? k_forces_m<KT, VISC, kForcesOnly, kListSkin> : k_forces_m<KT, VISC, kForcesOnly, kListEvery>;
+            k<<<grid, kModelBlock, 0, st>>>(b.pos[cur], b.vel[cur], b.phat[cur], nullptr, nullptr, nullptr, b.force,
+                                            b.pinfo[cur], b.nlist, b.ncount, b.scenes, b.dyn, b.status, ph, acc_dt,
+                                            nullptr, nullptr, nullptr, b.pid[cur]);
             break;
-        case kPredict:
-            k_forces_m<KT, VISC, kPredict><<<grid, kModelBlock, 0, st>>>(
-                b.pos[cur], b.vel[cur], b.phat[cur], b.pos_s, b.vel_s, b.phat_s, nullptr, b.pinfo[cur], list, count,
-                b.scenes, b.dyn, b.status, ph, 0, skin, nullptr, b.pid[cur]);
+        }
+        case kPredict: {
+            const auto k = skin ? k_forces_m<KT, VISC, kPredict, kListSkin> : k_forces_m<KT, VISC, kPredict, kListEvery>;
+            k<<<grid, kModelBlock, 0, st>>>(b.pos[cur], b.vel[cur], b.phat[cur], b.pos_s, b.vel_s, b.phat_s, nullptr,
+                                            b.pinfo[cur], b.nlist, b.ncount, b.scenes, b.dyn, b.status, ph, 0, nullptr,
+                                            b.nlist_x, b.ncount_x, b.pid[cur]);
             break;
-        case kCorrect:
-            k_forces_m<KT, VISC, kCorrect><<<grid, kModelBlock, 0, st>>>(
-                b.pos_s, b.vel_s, b.phat_s, b.pos[cur], b.vel[cur], b.phat[cur], nullptr, b.pinfo[cur], list, count,
-                b.scenes, b.dyn, b.status, ph, 0, skin, b.pos_ref, b.pid[cur]);
+        }
+        case kCorrect: {
+            const auto k = skin ? k_forces_m<KT, VISC, kCorrect, kListExact> : k_forces_m<KT, VISC, kCorrect, kListEvery>;
+            k<<<grid, kModelBlock, 0, st>>>(b.pos_s, b.vel_s, b.phat_s, b.pos[cur], b.vel[cur], b.phat[cur], nullptr,
+                                            b.pinfo[cur], skin ? b.nlist_x : b.nlist, skin ? b.ncount_x : b.ncount,
+                                            b.scenes, b.dyn, b.status, ph, 0, b.pos_ref, nullptr, nullptr, b.pid[cur]);
             break;
+        }
     }
 }
 

@@ -354,7 +354,8 @@ enum ForceMode { kForcesOnly = 0, kPredict = 1, kCorrect = 2 };
 // With a skin list (pos_ref allocated) the forces-only and predictor passes first write the
 // step's exact list to nlist_x/ncount_x (the predictor counts its pairs,
 // DevStatus.interactions), and every pass reads that; the corrector checks the
-// displacement since the build.
+// displacement since the build.  (The general models' passes test the pairs of the skin list themselves,
+// and their predictor writes the exact list.)
 void launch_forces(const Buffers& b, int cur, const Geometry& g, const Phys& ph, ForceMode mode,
                    int acc_dt, cudaStream_t st);
 // forces_models.cu: the same passes for the other model options of Table 1

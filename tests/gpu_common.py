@@ -172,3 +172,16 @@ def compare_neighbor_sets_of(scene, sample, counts, ids, band=1e-6):
         assert np.all(ids[k, nf + nb:] == 0xFFFFFFFF)
         total += len(sure)
     return total
+
+
+def launches(call, stream):
+    """Kernels that call() launches on `stream` (a torch stream), counted by capturing it."""
+    import ctypes
+    cu = ctypes.CDLL("libcuda.so.1")
+    st, graph, n = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p(), ctypes.c_size_t()
+    assert cu.cuStreamBeginCapture_v2(st, 1) == 0  # thread local
+    call()
+    assert cu.cuStreamEndCapture(st, ctypes.byref(graph)) == 0
+    assert cu.cuGraphGetNodes(graph, None, ctypes.byref(n)) == 0
+    cu.cuGraphDestroy(graph)
+    return n.value

@@ -7,7 +7,7 @@ import pytest
 
 import oracle
 from paper_2207_11328_gb300 import SphError, scenes
-from tests.gpu_common import rel_check, require_gpu, sim_for
+from tests.gpu_common import launches, rel_check, require_gpu, sim_for
 
 pytestmark = pytest.mark.gpu
 
@@ -105,3 +105,44 @@ def test_record_rejects_skin_mode():
     sim = sim_for(s, rebuild_every=10, skin=0.3 * s.h, max_neibs=192)
     with pytest.raises(SphError):
         sim.record(4, 2)
+
+
+@pytest.mark.parametrize("visc,kernel,form", [(0, 1, 0), (0, 0, 1), (2, 2, 1), (3, 1, 1)])
+@pytest.mark.parametrize("walls", [False, True])
+def test_general_models_over_a_skin_list(visc, kernel, form, walls):
+    # pairs beyond the cutoff are left out, by the pass itself (no list kernel before it); the predictor
+    # keeps and counts the others, and the corrector's list is what it kept.  (Kernels whose F vanishes at
+    # the cutoff: a pair that crosses it within a step is then the same to the oracle, which searches at
+    # each stage; the cut Gaussian jumps there.)
+    import dataclasses
+    import torch
+    if walls:
+        s = scenes.dam_break(dp=0.05)
+        f = s.ptype == 0
+        s.vel[f] = scenes.seeded_normal((int(f.sum()), 3), 0.05, 5).astype(np.float32)
+    else:
+        s = _box(seed=11)
+    s = dataclasses.replace(s, visc=visc, nu=1e-3 if visc else 0.0, kernel_type=kernel, formulation=form)
+    sim = sim_for(s, rebuild_every=10, skin=0.3 * s.h, max_neibs=256)
+    sim.forces()
+    acc, drho = sim.download_forces()
+    a_ref, d_ref, mag = oracle.rhs(oracle.params(s), s.pos, s.vel, s.delta, s.mass, s.ptype, with_mag=True)
+    rel_check(acc, a_ref, 1e-5, "acceleration", mag[:, 0])
+    rel_check(drho, d_ref, 1e-5, "density rate", mag[:, 1])
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    assert launches(lambda: sim.forces(stream=stream), stream) == 1
+    sim.step(6)
+    pos, vel, delta = sim.download()
+    st = sim.stats()
+    assert st["error_bits"] == 0
+    off, idx = oracle.neighbors(oracle.params(s), s.pos)
+    i = np.repeat(np.arange(s.n), np.diff(off))
+    pairs = int(((s.ptype[i] == 0) | (s.ptype[idx] == 0)).sum())
+    assert st["interactions"] == pytest.approx(6 * pairs, rel=0.01)
+    x1, u1, d1, _, _ = oracle.step(oracle.params(s), s.pos, s.vel, s.delta, s.mass, s.ptype, 6)
+    per = np.array([(s.periodic >> a) & 1 for a in range(3)])
+    dx = pos - x1
+    dx -= per * np.array(s.size) * np.round(dx / np.array(s.size))
+    assert np.max(np.abs(dx)) < 1e-4 * s.dp
+    assert np.max(np.abs(vel - u1)) < 1e-4 * 0.05
