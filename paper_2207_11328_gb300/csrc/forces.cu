@@ -86,18 +86,17 @@ __host__ __device__ constexpr bool is_artificial(int v) { return (v & ~kDiffusio
 __host__ __device__ constexpr bool is_laminar(int v) { return (v & ~kDiffusion) == SPH_VISC_LAMINAR; }
 __host__ __device__ constexpr bool has_diffusion(int v) { return (v & kDiffusion) != 0; }
 
-template <int VISC, bool BND, class Out>
-__device__ __forceinline__ void fluid_pair(uint32_t e, const Central& ci, const float4& vi, float phat_i,
-                                           const float4* __restrict__ pos, const float4* __restrict__ vel,
-                                           float phat_coef, float pi_coef, float dd_coef, const Phys& ph, Out& out) {
-    const uint32_t j = e >> kCodeBits;
-    const float4 pj = pos[j];
-    const float4 vj = vel[j];  // both gathers issued together
+// FILTER: a pair beyond the cutoff is left out.
+template <int VISC, bool BND, bool FILTER, class Out>
+__device__ __forceinline__ void fluid_pair(uint32_t e, const float4& pj, const float4& vj, const Central& ci,
+                                           const float4& vi, float phat_i, float phat_coef, float pi_coef, float dd_coef,
+                                           const Phys& ph, Out& out) {
     const float phat_j = eos_phat(vj.w, ph, phat_coef);
     const float rx = pick(e, ci.xm, ci.x0, ci.xp) - pj.x;
     const float ry = pick(e >> 2, ci.ym, ci.y0, ci.yp) - pj.y;
     const float rz = pick(e >> 4, ci.zm, ci.z0, ci.zp) - pj.z;
     const float r2 = fmaxf(fmaf(rx, rx, fmaf(ry, ry, rz * rz)), 1e-30f);
+    if (FILTER && !(r2 < ph.R2)) return;
     const float r = r2 * rsqrt_fast(r2);
     const float t = fminf(fmaf(r, ph.inv_h, -2.0f), 0.0f);
     const float mj = BND ? -pj.w : pj.w;
@@ -120,7 +119,7 @@ __device__ __forceinline__ void fluid_pair(uint32_t e, const Central& ci, const 
 }
 
 // one fluid neighbour of a boundary particle: continuity, u_i = 0
-template <class Out>
+template <bool FILTER, class Out>
 __device__ __forceinline__ void boundary_pair(uint32_t e, const Central& ci, const float4* __restrict__ pos,
                                               const float4* __restrict__ vel, const Phys& ph, Out& out) {
     const uint32_t j = e >> kCodeBits;
@@ -130,6 +129,7 @@ __device__ __forceinline__ void boundary_pair(uint32_t e, const Central& ci, con
     const float ry = pick(e >> 2, ci.ym, ci.y0, ci.yp) - pj.y;
     const float rz = pick(e >> 4, ci.zm, ci.z0, ci.zp) - pj.z;
     const float r2 = fmaxf(fmaf(rx, rx, fmaf(ry, ry, rz * rz)), 1e-30f);
+    if (FILTER && !(r2 < ph.R2)) return;
     const float r = r2 * rsqrt_fast(r2);
     const float t = fminf(fmaf(r, ph.inv_h, -2.0f), 0.0f);
     add_rate(out, pj.w * (t * t * t), -fmaf(vj.x, rx, fmaf(vj.y, ry, vj.z * rz)));
@@ -183,8 +183,8 @@ __device__ __forceinline__ void lanes_sum(const uint2* __restrict__ lp, ptrdiff_
     }
 }
 
-// (the forces-only pass keeps the |a|^2 reduction for dt0 live beside the sums: it gets
-// a looser register cap than the step's passes, so that no shape spills)
+// (the forces-only pass over a list of every step keeps the |a|^2 reduction for dt0 live beside the sums: it
+// gets a looser register cap than the step's passes)
 // One particle of a force pass (one iteration of the pass's particle loop): its pair sums
 // over its list and the epilogue of the pass (store, predictor or corrector update).
 __device__ __forceinline__ uint32_t ld_count_fresh(const uint32_t* p) {
@@ -203,8 +203,9 @@ __device__ __forceinline__ uint2 ld_chunk(const uint2* p) {
     return v;
 }
 
-// SKIN: nlist/ncount are the step's exact list in its four-entry chunks; the corrector also checks
-// and reduces the displacement since the list's build.
+// SKIN: nlist/ncount are the step's exact list in its four-entry chunks, but in the forces-only pass, which
+// leaves out the skin list's pairs beyond the cutoff itself; the corrector also checks and reduces the
+// displacement since the list's build.
 // WIDE: list chunks of two entries evaluated together as long as the fluid part has so many left, their
 // gathers issued before the first is used.  A state that does not fill the GPU is bound by
 // that latency, and has the registers to spare (see launch_forces_v).
@@ -216,6 +217,7 @@ __device__ __forceinline__ void particle_pass(
     const SceneDev* __restrict__ scenes, SceneDyn* __restrict__ dyn, DevStatus* __restrict__ st, const Phys& ph,
     int acc_dt, const float4* __restrict__ pos_ref, const uint32_t* __restrict__ pid, uint32_t cnt_fresh = 0) {
     static_assert(LANES == 1 || !(FRESH || SKIN), "a group of lanes takes an every-step list");
+    constexpr bool FILTER = SKIN && MODE == kForcesOnly, EXACT = SKIN && !FILTER;
     const uint32_t s = pinfo[i];
     const SceneDev& sc = scenes[s];
     const float4 pi = pos[i];
@@ -227,7 +229,27 @@ __device__ __forceinline__ void particle_pass(
     const float cx = sc.cell_f[0], cy = sc.cell_f[1], cz = sc.cell_f[2];
     Acc acc{0.f, 0.f, 0.f, 0.f};
     const size_t S = ph.stride;
-#define SPH_PAIR(BND, e, out) fluid_pair<VISC, BND>(e, ci, vi, phat_i, pos, vel, sc.phat_coef, pic, sc.dd_coef, ph, out)
+#define SPH_PAIR_OF(BND, e, pj, vj, out) \
+    fluid_pair<VISC, BND, FILTER>(e, pj, vj, ci, vi, phat_i, sc.phat_coef, pic, sc.dd_coef, ph, out)
+// both gathers issued together
+#define SPH_PAIR(BND, e, out)                                                              \
+    do {                                                                                   \
+        const float4 pj_ = pos[(e) >> kCodeBits], vj_ = vel[(e) >> kCodeBits];             \
+        SPH_PAIR_OF(BND, e, pj_, vj_, out);                                                \
+    } while (0)
+// the filter's branch would keep the second pair's gathers behind the first pair
+#define SPH_PAIR2(BND, e0, e1, out)                                                        \
+    do {                                                                                   \
+        if (FILTER) {                                                                      \
+            const float4 pa_ = pos[(e0) >> kCodeBits], va_ = vel[(e0) >> kCodeBits];       \
+            const float4 pb_ = pos[(e1) >> kCodeBits], vb_ = vel[(e1) >> kCodeBits];       \
+            SPH_PAIR_OF(BND, e0, pa_, va_, out);                                           \
+            SPH_PAIR_OF(BND, e1, pb_, vb_, out);                                           \
+        } else {                                                                           \
+            SPH_PAIR(BND, e0, out);                                                        \
+            SPH_PAIR(BND, e1, out);                                                        \
+        }                                                                                  \
+    } while (0)
     if (LANES > 1) {
         const float phat_i = phat[i];
         const float pic = sc.pi_coef;
@@ -242,11 +264,11 @@ __device__ __forceinline__ void particle_pass(
             acc.az = fmaf(ph.aF, acc.az, ph.g[2]);
         } else {
             lanes_sum<VISC, LANES>(fl, (ptrdiff_t)S, nf, n, st, acc, [&](uint32_t e, Terms& tm) {
-                boundary_pair(e, ci, pos, vel, ph, tm); });
+                boundary_pair<false>(e, ci, pos, vel, ph, tm); });
         }
         acc.drho *= ph.aF;
         if (threadIdx.x % LANES != 0) return;  // the first lane finishes the particle
-    } else if (fluid_i && SKIN) {
+    } else if (fluid_i && EXACT) {
         const float phat_i = phat[i];
         const float pic = sc.pi_coef;
         const Central ci = central_of(pi, cx, cy, cz);
@@ -341,10 +363,8 @@ __device__ __forceinline__ void particle_pass(
                 bn = ld_chunk<FRESH>(lp + 3 * S);
             }
             SPH_GUARD((max(max(a.x, a.y), max(b.x, b.y)) >> kCodeBits) < n, st, break)
-            SPH_PAIR(false, a.x, acc);
-            SPH_PAIR(false, a.y, acc);
-            SPH_PAIR(false, b.x, acc);
-            SPH_PAIR(false, b.y, acc);
+            SPH_PAIR2(false, a.x, a.y, acc);
+            SPH_PAIR2(false, b.x, b.y, acc);
         }
         for (; k < nf; k += 2, lp += S) {
             const uint2 a = ld_chunk<FRESH>(lp);
@@ -369,13 +389,13 @@ __device__ __forceinline__ void particle_pass(
         // boundary particle: continuity over its fluid neighbours, u_i = 0
         const Central ci = central_of(pi, cx, cy, cz);
         const uint2* lp = reinterpret_cast<const uint2*>(nlist) + i;
-        const uint4* cp = reinterpret_cast<const uint4*>(nlist) + i;  // SKIN
+        const uint4* cp = reinterpret_cast<const uint4*>(nlist) + i;  // EXACT
         uint4 q = make_uint4(0u, 0u, 0u, 0u);
         uint2 q2 = make_uint2(0u, 0u);
 #pragma unroll 2
         for (uint32_t k = 0; k < nf; ++k) {
             uint32_t e;
-            if (SKIN) {
+            if (EXACT) {
                 if ((k & 3u) == 0u) {
                     q = __ldg(cp);
                     cp += S;
@@ -389,11 +409,13 @@ __device__ __forceinline__ void particle_pass(
                 e = (k & 1u) ? q2.y : q2.x;
             }
             SPH_GUARD((e >> kCodeBits) < n, st, continue)
-            boundary_pair(e, ci, pos, vel, ph, acc);
+            boundary_pair<FILTER>(e, ci, pos, vel, ph, acc);
         }
         acc.drho *= ph.aF;
     }
+#undef SPH_PAIR2
 #undef SPH_PAIR
+#undef SPH_PAIR_OF
 
     // epilogue written out here rather than through finish_particle() of
     // forces_common.cuh (same operations): measured 7 % faster in these kernels
@@ -477,7 +499,7 @@ __device__ __forceinline__ void forces_body(
 }
 
 template <int VISC, int MODE, int kBlock, int kMinBlocks, bool SKIN, int LANES, int WIDE>
-__global__ void __launch_bounds__(kBlock, MODE == kForcesOnly ? (kMinBlocks * 2 + 2) / 3 : kMinBlocks) k_forces(
+__global__ void __launch_bounds__(kBlock, MODE == kForcesOnly && !SKIN ? (kMinBlocks * 2 + 2) / 3 : kMinBlocks) k_forces(
     const float4* __restrict__ pos, const float4* __restrict__ vel, const float* __restrict__ phat,
     float4* io_pos, float4* io_vel, float* io_phat, float4* __restrict__ force_out,
     const uint32_t* __restrict__ pinfo, const uint32_t* __restrict__ nlist, const uint32_t* __restrict__ ncount,
@@ -489,18 +511,20 @@ __global__ void __launch_bounds__(kBlock, MODE == kForcesOnly ? (kMinBlocks * 2 
 
 // ---------------------------------------------------------------------
 // A list with a skin (rebuilt every k steps): the step's exact list, the listed pairs within the
-// influence radius at x^n, in list order, in chunks of four entries.  Both passes of the step (and
-// sph_forces) then run over it.  One gather and one test a listed pair; the
+// influence radius at x^n, in list order, in chunks of four entries.  Both passes of the step
+// then run over it.  One gather and one test a listed pair; the
 // predictor over the skin list itself evaluated a warp's pairs beyond the radius along with the others
 // (1.65M dam break, skin 0.3 h: 640 us, now 290 for the list and 283 for the pass; bound by the gathers
-// through L1).
-// count: add the pairs kept to DevStatus.interactions.
+// through L1).  The pairs kept are counted (DevStatus.interactions).
+// A forces-only pass would use the list once: it tests the skin list's pairs itself, two pairs' gathers at a
+// time, in 64 registers (the same state: 336 us; the list and a pass over it 495; one pair at a time 350; in
+// 85 registers 356; with 42,120 particles 38 / 45 / 40 / 38).
 // ---------------------------------------------------------------------
 __global__ void __launch_bounds__(128, 8) k_exact_list(const float4* __restrict__ pos, const uint32_t* __restrict__ pinfo,
                                                        const uint32_t* __restrict__ nlist,
                                                        const uint32_t* __restrict__ ncount,
                                                        const SceneDev* __restrict__ scenes, DevStatus* __restrict__ st,
-                                                       float R2, uint32_t max_neibs, uint32_t stride, int count,
+                                                       float R2, uint32_t max_neibs, uint32_t stride,
                                                        uint32_t* __restrict__ nlist_x, uint32_t* __restrict__ ncount_x) {
     const uint32_t n = st->n_active;
     uint32_t kept = 0;
@@ -557,10 +581,8 @@ __global__ void __launch_bounds__(128, 8) k_exact_list(const float4* __restrict_
         ncount_x[i] = wf.n | (wb.n << 16);
         kept += wf.n + wb.n;
     }
-    if (count) {
-        const uint32_t w = __reduce_add_sync(0xffffffffu, kept);
-        if ((threadIdx.x & 31) == 0 && w) atomicAdd(&st->interactions, (unsigned long long)w);
-    }
+    const uint32_t w = __reduce_add_sync(0xffffffffu, kept);
+    if ((threadIdx.x & 31) == 0 && w) atomicAdd(&st->interactions, (unsigned long long)w);
 }
 
 // Predictor update (reading C6) from forces already stored by a
@@ -685,8 +707,9 @@ template <int VISC, int B, int MB, bool SKIN, int LANES, int WIDE>
 void launch_forces_s(const Buffers& b, int cur, const Geometry& g, const Phys& ph, ForceMode mode, int acc_dt,
                      cudaStream_t st) {
     const unsigned grid = g.cap ? (unsigned)(((uint64_t)g.cap * LANES + B - 1) / B) : 1;
-    const uint32_t* const list = SKIN ? b.nlist_x : b.nlist;
-    const uint32_t* const count = SKIN ? b.ncount_x : b.ncount;
+    const bool exact = SKIN && mode != kForcesOnly;
+    const uint32_t* const list = exact ? b.nlist_x : b.nlist;
+    const uint32_t* const count = exact ? b.ncount_x : b.ncount;
     switch (mode) {
         case kForcesOnly:
             k_forces<VISC, kForcesOnly, B, MB, SKIN, LANES, WIDE><<<grid, B, 0, st>>>(
@@ -799,10 +822,10 @@ void launch_conservation(const Buffers& b, int cur, double* scratch, cudaStream_
 
 void launch_forces(const Buffers& b, int cur, const Geometry& g, const Phys& ph, ForceMode mode, int acc_dt,
                    cudaStream_t st) {
-    if (b.pos_ref && mode != kCorrect && !ph.general)  // a skin list: first the step's exact list
+    if (b.pos_ref && mode == kPredict && !ph.general)  // a skin list: first the step's exact list
         k_exact_list<<<g.cap ? (g.cap + 127) / 128 : 1, 128, 0, st>>>(
             b.pos[cur], b.pinfo[cur], b.nlist, b.ncount, b.scenes, b.status, ph.R2, ph.max_neibs, ph.stride,
-            mode == kPredict, b.nlist_x, b.ncount_x);
+            b.nlist_x, b.ncount_x);
     if (ph.general) {
         launch_forces_models(b, cur, g, ph, mode, acc_dt, st);
         return;

@@ -351,11 +351,10 @@ void launch_tape_copy(const void* const* src, void* const* dst, const bool* wide
 
 // forces.cu
 enum ForceMode { kForcesOnly = 0, kPredict = 1, kCorrect = 2 };
-// With a skin list (pos_ref allocated) the forces-only and predictor passes first write the
-// step's exact list to nlist_x/ncount_x (the predictor counts its pairs,
-// DevStatus.interactions), and every pass reads that; the corrector checks the
-// displacement since the build.  (The general models' passes test the pairs of the skin list themselves,
-// and their predictor writes the exact list.)
+// With a skin list (pos_ref allocated) the predictor pass first writes the step's exact list to
+// nlist_x/ncount_x and counts its pairs (DevStatus.interactions), and the step's passes read
+// that; the corrector checks the displacement since the build.  The forces-only pass tests the pairs
+// of the skin list itself.  (So does the general models' predictor, which writes the exact list as it goes.)
 void launch_forces(const Buffers& b, int cur, const Geometry& g, const Phys& ph, ForceMode mode,
                    int acc_dt, cudaStream_t st);
 // forces_models.cu: the same passes for the other model options of Table 1

@@ -146,3 +146,37 @@ def test_general_models_over_a_skin_list(visc, kernel, form, walls):
     dx -= per * np.array(s.size) * np.round(dx / np.array(s.size))
     assert np.max(np.abs(dx)) < 1e-4 * s.dp
     assert np.max(np.abs(vel - u1)) < 1e-4 * 0.05
+
+
+@pytest.mark.parametrize("visc,ddiff", [(0, 0), (1, 0), (0, 1), (1, 1)])
+@pytest.mark.parametrize("walls", [False, True])
+def test_forces_over_a_used_skin_list(visc, ddiff, walls):
+    # accelerations between steps, on a list some steps old: one launch, the oracle's values there, and
+    # no effect on the steps that follow
+    import dataclasses
+    import torch
+    if walls:
+        s = scenes.dam_break(dp=0.05)
+        f = s.ptype == 0
+        s.vel[f] = scenes.seeded_normal((int(f.sum()), 3), 0.05, 5).astype(np.float32)
+    else:
+        s = _box(seed=12)
+    s = dataclasses.replace(s, visc=visc, nu=1e-3 if visc else 0.0, ddiff=ddiff, ddiff_coef=0.1 * ddiff)
+    sim, other = (sim_for(s, rebuild_every=10, skin=0.3 * s.h, max_neibs=192) for _ in range(2))
+    for k in (sim, other):
+        k.step(4)
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    sim.forces()
+    acc, drho = sim.download_forces()
+    assert launches(lambda: sim.forces(stream=stream), stream) == 1
+    pos, vel, delta = sim.download()
+    # (the downloaded positions are the state's to half an FP32 ulp of the offset in the cell)
+    a_ref, d_ref, mag = oracle.rhs(oracle.params(s), pos, vel, delta, s.mass, s.ptype, with_mag=True)
+    rel_check(acc, a_ref, 1e-5, "acceleration", mag[:, 0])
+    rel_check(drho, d_ref, 1e-5, "density rate", mag[:, 1])
+    for k in (sim, other):
+        k.step(5)
+    for a, b in zip(sim.download(), other.download()):
+        assert np.array_equal(a, b)
+    assert sim.stats()["interactions"] == other.stats()["interactions"]
