@@ -261,7 +261,9 @@ int sph_next_dt(sph_ctx* ctx, double* dt, void* stream);
  * the list and the candidates it has just tested are in cache.  The same list
  * and the same results, to the bit.  Until this call, sph_autotune (which
  * fuses them when that is at least 2% faster) or a build variant set, each
- * upload of more than 2.5 million particles fuses them.  Only with the list rebuilt every step and the default model
+ * upload of more than 2.5 million particles fuses them.  Fused already, on
+ * keeps the block size that the upload or tuning chose; else it is 256
+ * threads.  Only with the list rebuilt every step and the default model
  * (SPH_ERR_ARG otherwise); the paper runs the two as separate commands
  * (Section 3 "Code structure").  Synchronises the device. */
 int sph_set_fused_predict(sph_ctx* ctx, int on);

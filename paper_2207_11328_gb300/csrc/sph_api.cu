@@ -1066,7 +1066,7 @@ int sph_set_fused_predict(sph_ctx* c, int on) {
     if (!c) return SPH_ERR_ARG;
     if (on && !can_fuse(c)) return SPH_ERR_ARG;
     CK(cudaDeviceSynchronize());
-    c->ph.fuse_predict = on ? 256 : 0;
+    c->ph.fuse_predict = fused_threads(c->ph.fuse_predict, on != 0);
     c->auto_fuse = false;
     drop_graphs(c);
     return SPH_OK;

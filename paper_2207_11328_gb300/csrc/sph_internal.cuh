@@ -187,6 +187,10 @@ constexpr uint32_t kStageNeibs = 256;  // longest list that the build by rows of
 __host__ __device__ constexpr size_t quad_word(uint32_t i) { return (size_t)(i >> 2) * 12u + (i & 3u); }  // x; y, z at + 4, + 8
 __host__ __device__ constexpr size_t quad_floats(uint32_t cap) { return ((size_t)cap / 4u + 1u) * 12u; }
 const char* build_variant_name(int v);
+// threads per block of the fused build and predictor when it is asked for: those that an upload or tuning
+// has chosen stay, else 256 (figures of both at default_variants, sph_api.cu: the better one on boxes and dam
+// breaks, 1.5 to 2.7% behind 128 on batches of tanks)
+constexpr int fused_threads(int now, bool on) { return !on ? 0 : (now ? now : 256); }
 constexpr int kForcesVariants = 5;
 const char* forces_variant_name(int v);
 

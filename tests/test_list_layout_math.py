@@ -5,6 +5,7 @@ the library accepts (8..1024) and every nf + nb <= max_neibs the two parts
 never share a chunk.  The formula is read from the header, not restated."""
 import os
 import re
+import subprocess
 
 HEADER = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
                       "paper_2207_11328_gb300", "csrc", "sph_internal.cuh")
@@ -48,3 +49,20 @@ def test_exact_list_parts_fit():
         k = kxb(mn)
         assert (mn + 3) // 4 <= k          # a fluid part of up to max_neibs entries
         assert k + (mn + 3) // 4 <= 2 * k  # a boundary part of up to max_neibs entries
+
+
+def test_fused_build_keeps_a_chosen_block_size(tmp_path):
+    # reading the option and setting it back changes nothing; asked for anew it takes 256 threads
+    src = open(HEADER).read()
+    line = re.search(r"constexpr int fused_threads\(int now, bool on\) .*}", src).group(0)
+    (tmp_path / "t.cpp").write_text(f"""#include <cstdio>
+{line}
+int main() {{
+    for (int now : {{0, 128, 256}}) std::printf("%d %d ", fused_threads(now, true), fused_threads(now, false));
+}}
+""")
+    subprocess.run(["g++", "-std=c++17", "-o", str(tmp_path / "t"), str(tmp_path / "t.cpp")], check=True)
+    out = subprocess.run([str(tmp_path / "t")], check=True, capture_output=True, text=True).stdout
+    assert out.split() == ["256", "0", "128", "0", "256", "0"]
+    api = open(os.path.join(os.path.dirname(HEADER), "sph_api.cu")).read()
+    assert "fuse_predict = fused_threads(c->ph.fuse_predict, on != 0);" in api
