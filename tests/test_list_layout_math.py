@@ -56,6 +56,7 @@ def test_fused_build_keeps_a_chosen_block_size(tmp_path):
     src = open(HEADER).read()
     line = re.search(r"constexpr int fused_threads\(int now, bool on\) .*}", src).group(0)
     (tmp_path / "t.cpp").write_text(f"""#include <cstdio>
+#include <initializer_list>
 {line}
 int main() {{
     for (int now : {{0, 128, 256}}) std::printf("%d %d ", fused_threads(now, true), fused_threads(now, false));
