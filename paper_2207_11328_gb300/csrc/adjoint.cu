@@ -429,9 +429,14 @@ void launch_adj_vjps(const AdjBuffers& a, const Buffers& b, int cur, const Geome
 template <int VISC>
 void launch_adj_vjps_v(const AdjBuffers& a, const Buffers& b, int cur, const Geometry& g, const Phys& ph, float dt,
                        cudaStream_t st) {
-    // lanes per particle: enough threads to fill the GPU (~150k resident) on small states (backward
-    // pass with 8 / 4 / 2 lanes, ms: 26,082 particles and 16 steps 2.13 / 2.24 / 2.46, 32,768 and 64
-    // steps 8.47 / 8.34 / 9.02)
+    // lanes per particle, by the context's capacity: enough threads to fill the GPU (~150k resident) on small
+    // states.  Backward pass of 16 steps with 8 / 4 / 2 lanes, ms:
+    //   periodic boxes  8,000  1.05 / 1.15 / 1.45    dam breaks  13,023  1.66 / 1.75 / 2.06
+    //                  13,824  1.16 / 1.20 / 1.49                26,082  1.82 / 1.89 / 2.18
+    //                  17,576  1.34 / 1.27 / 1.52                33,750  2.00 / 2.05 / 2.33
+    //                  27,000  1.66 / 1.67 / 1.80                52,229  2.31 / 2.41 / 2.52
+    //                  32,768  1.83 / 1.80 / 1.94
+    //                  64,000  3.05 / 3.02 / 3.04
     if (g.cap <= 28672u)
         launch_adj_vjps<VISC, 8>(a, b, cur, g, ph, dt, st);
     else if (g.cap <= (1u << 16))

@@ -178,3 +178,77 @@ def test_crowded_cells_in_the_row_build():
     for a, b in zip(*got):
         assert np.array_equal(a, b)
     assert ms[1] < 2.5 * ms[0]
+
+
+def _row_build_tiles(s):
+    """Tiles of 32 sorted particles by what the build by rows does with them (lists of up to 256 entries):
+    (kept in shared memory, of those beside a cell of over 32 candidate slots, put off)."""
+    nc = np.floor(np.array(s.size) / (s.kernel_radius * s.h)).astype(int)
+    c = np.minimum((s.pos / (np.array(s.size) / nc)).astype(int), nc - 1)
+    key = c[:, 0] + nc[0] * (c[:, 1] + nc[1] * c[:, 2])
+    order = np.lexsort((np.arange(s.n), s.ptype, key))
+    start = np.searchsorted(key[order], np.arange(nc.prod() + 1))
+    end = np.stack([start[1:], start[:-1] + np.bincount(key[s.ptype == 0], minlength=nc.prod())], 1)  # of a fluid, a wall particle
+    slots = end - (start[:-1] & ~3)[:, None]
+    slots[end - start[:-1, None] == 0] = 0
+    most = np.zeros(s.n, int)  # of the neighbour cells' slots, by sorted particle
+    for d in np.ndindex(3, 3, 3):
+        q = c[order] + np.array(d) - 1
+        ok = np.ones(s.n, bool)
+        for a in range(3):
+            if (s.periodic >> a) & 1:
+                q[:, a] %= nc[a]
+            else:
+                ok &= (q[:, a] >= 0) & (q[:, a] < nc[a])
+        q = np.where(ok[:, None], q, 0)
+        k = q[:, 0] + nc[0] * (q[:, 1] + nc[1] * q[:, 2])
+        most = np.maximum(most, np.where(ok, slots[k, s.ptype[order]], 0))
+    tile = np.array([most[i:i + 32].max() for i in range(0, s.n, 32)])
+    return int((tile <= 64).sum()), int(((tile <= 64) & (tile > 32)).sum()), int((tile > 64).sum())
+
+
+@pytest.mark.parametrize("n,cells,crowd,periodic,nb,max_neibs,put_off",
+                         [(700, 5, 33, True, 120, 256, False), (900, 5, 50, False, 250, 255, False),
+                          (1201, 6, 52, True, 400, 129, False), (1500, 6, 90, True, 300, 256, True),
+                          (1100, 6, 70, False, 300, 255, True)])
+def test_row_build_in_shared_memory(n, cells, crowd, periodic, nb, max_neibs, put_off):
+    """Lists put together in shared memory, beside cells of 33 to 64 slots (a second hit mask), alone and
+    with put-off tiles in the same launch: the oracle's sets, and every variant one list."""
+    s = _cloud(n, cells, crowd, periodic, nb, seed=n)
+    kept, two_masks, off = _row_build_tiles(s)
+    assert kept > 0 and (off > 0 if put_off else two_masks > 0 and off == 0), (kept, two_masks, off)
+    ref = None
+    for v in range(N_BUILD_VARIANTS):
+        sim = sim_for(s, max_neibs=max_neibs)
+        sim.set_variants(build=v)
+        sim.build_neighbors()
+        got = (*sim.download_neighbors(), sim.stats()["list_entries"], sim.stats()["max_neibs_seen"])
+        if ref is None:
+            ref = got
+            compare_neighbor_sets(s, *got[:2])
+        for a, b in zip(got, ref):
+            assert np.array_equal(a, b) if isinstance(a, np.ndarray) else a == b
+
+
+@pytest.mark.parametrize("max_neibs", [8, 17, 32, 33, 64, 65])
+def test_row_build_cuts_lists_in_shared_memory(max_neibs):
+    """The same lists cut at their last entry, in tiles that are kept in shared memory, fluid and wall parts."""
+    s = _cloud(900, 5, 50, True, 400, seed=8)
+    kept, two_masks, off = _row_build_tiles(s)
+    assert kept > 0 and two_masks > 0 and off == 0
+    full, _ = (lambda sim: (sim.build_neighbors(), sim.download_neighbors())[1])(sim_for(s, max_neibs=256))
+    ref = None
+    for v in range(N_BUILD_VARIANTS):
+        sim = sim_for(s, max_neibs=max_neibs)
+        sim.set_variants(build=v)
+        sim.build_neighbors()
+        st = sim.stats(check=False)
+        assert st["rc"] == -4
+        got = (*sim.download_neighbors(), np.array([st["max_neibs_seen"], st["list_entries"]]))
+        assert np.array_equal(got[0].sum(1), np.minimum(full.sum(1), max_neibs))
+        if ref is None:
+            ref = got
+            cut = full.sum(1) > max_neibs
+            assert (got[0][cut] > 0).all(1).any()  # both parts in a list that is cut
+        for a, b in zip(got, ref):
+            assert np.array_equal(a, b)
