@@ -177,7 +177,11 @@ template <int MB>
 void launch_build_rows(const Buffers& b, int cur, const Geometry& g, const Phys& ph, cudaStream_t st) {
     const size_t smem = ph.max_neibs <= kStageNeibs ? sizeof(uint32_t) * rows_smem_words(ph.max_neibs) : 0;
     // resident blocks at most: a block then takes several tiles in turn
-    const unsigned grid = std::min(grid_for(g.cap, 32), 152u * MB);
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
+        sms = 1;
+    const unsigned grid = std::min(grid_for(g.cap, 32), (unsigned)sms * MB);
     k_build_rows<MB><<<grid, kRowBlock, smem, st>>>(b.pos[cur], b.quads, b.cell[cur], b.pinfo[cur], b.start, b.cell_nfluid,
                                                    b.scenes, b.status, b.nlist, b.ncount, ph.R2_list, ph.max_neibs,
                                                    ph.stride, b.gate);

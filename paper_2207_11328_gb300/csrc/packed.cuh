@@ -1,5 +1,5 @@
 // Packed FP32 arithmetic: two FP32 values in one 64-bit register pair, each
-// operation one instruction on both (add/mul/fma.rn.f32x2, round to nearest,
+// operation one instruction on both (add/fma.rn.f32x2, round to nearest,
 // the same bits as two scalar operations).  On GB300 a packed FMA issues at the
 // rate of a scalar one (measured: 16 independent FMAs per warp and iteration
 // take 16.3 cycles of a scheduler either way), so it halves the issue slots and
@@ -32,20 +32,11 @@ __device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
 }
-__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
-    f2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
 __device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
     f2 r;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
 }
-// a - b (exact negation in the FMA, rounded once)
-__device__ __forceinline__ f2 f2_sub(f2 a, f2 b) { return f2_fma(b, f2_dup(-1.0f), a); }
-__device__ __forceinline__ f2 f2_min(f2 a, float b) { return f2_make(fminf(f2_lo(a), b), fminf(f2_hi(a), b)); }
-
 // approximate reciprocal and reciprocal square root of normal arguments (the
 // callers keep them away from zero and the subnormals, so flushing changes nothing)
 __device__ __forceinline__ float rcp_fast(float a) {
@@ -58,7 +49,5 @@ __device__ __forceinline__ float rsqrt_fast(float a) {
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
     return r;
 }
-__device__ __forceinline__ f2 f2_rcp(f2 a) { return f2_make(rcp_fast(f2_lo(a)), rcp_fast(f2_hi(a))); }
-__device__ __forceinline__ f2 f2_rsqrt(f2 a) { return f2_make(rsqrt_fast(f2_lo(a)), rsqrt_fast(f2_hi(a))); }
 
 }  // namespace sphg
