@@ -360,7 +360,9 @@ int sph_autotune(sph_ctx* ctx, void* stream, int* build_variant, int* forces_var
  * (0..4, for every pass) directly, as sph_autotune would (-1 keeps the
  * current one; a build variant set ends the fusion that an upload chose, see
  * sph_set_fused_predict); until then each upload picks them by the particle
- * count.
+ * count and max_neibs.  A skin list's passes know the shapes of 128 and of
+ * 256 threads (1 and 2): the others run as the one of 128.  The general model
+ * options have one shape, whatever is set; both still report the index set.
  * Every variant computes the same bits.  Synchronises the
  * device; SPH_ERR_ARG for an index out of range. */
 int sph_set_variants(sph_ctx* ctx, int build_variant, int forces_variant);

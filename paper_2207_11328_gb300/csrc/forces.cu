@@ -753,7 +753,7 @@ void launch_forces_b(const Buffers& b, int cur, const Geometry& g, const Phys& p
 template <int VISC>
 void launch_forces_v(const Buffers& b, int cur, const Geometry& g, const Phys& ph, ForceMode mode, int acc_dt,
                      cudaStream_t st) {
-    switch (mode == kCorrect ? ph.forces_variant_c : ph.forces_variant) {
+    switch (mode == kCorrect ? ph.forces_variant_c : mode == kPredict ? ph.forces_variant : ph.forces_variant_f) {
         case 0: launch_forces_b<VISC, 64, 10, 1, 4>(b, cur, g, ph, mode, acc_dt, st); break;
         case 2: launch_forces_b<VISC, 256, 4>(b, cur, g, ph, mode, acc_dt, st); break;
         case 3: launch_forces_b<VISC, 32, 9, 1, 8>(b, cur, g, ph, mode, acc_dt, st); break;

@@ -115,6 +115,7 @@ inline cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
 // the largest particle counts of the small states' launch shapes (see default_variants)
 constexpr uint32_t kRowBuildMax = 81920, kLanesMax = 8192, kWide16Max = 40960, kWide8Max = 81920;
+constexpr uint32_t kWide16MaxF = 36864, kWide8MaxF = 73728;  // of the forces-only pass
 constexpr uint32_t kTpp128Max = 524288, kApartMax = 2500000;  // and of large ones
 constexpr uint32_t kSmallTuneMax = 131072;  // sph_autotune times those shapes up to here
 
@@ -662,10 +663,10 @@ inline unsigned grid_for(uint32_t n, int block) {
 //          20,139,024 15.52 / 15.35 / 14.82 / 14.80 ms
 // so blocks of 256 above half a million, and the fused kernel above 2.5 million, in the shape that lost
 // nowhere.  A build variant or fusion that was set or tuned stays.
-int default_forces(uint32_t n) {
+int default_forces(uint32_t n, uint32_t wide16_max, uint32_t wide8_max) {
     if (n <= kLanesMax) return 4;
-    if (n <= kWide16Max) return 3;
-    return n <= kWide8Max ? 0 : 1;
+    if (n <= wide16_max) return 3;
+    return n <= wide8_max ? 0 : 1;
 }
 
 void default_variants(sph_ctx* c, uint32_t n) {
@@ -673,8 +674,17 @@ void default_variants(sph_ctx* c, uint32_t n) {
     if (c->auto_fuse) ph.fuse_predict = c->auto_build && n > kApartMax && can_fuse(c) ? 128 : 0;
     if (c->auto_build)
         ph.build_variant = n <= kRowBuildMax && ph.max_neibs <= kStageNeibs ? 4 : (n <= kTpp128Max ? 0 : 1);
-    if (c->auto_forces)
-        ph.forces_variant = ph.forces_variant_c = skin_mode(c) || c->ph.general ? 1 : default_forces(n);
+    if (c->auto_forces) {
+        const bool plain = skin_mode(c) || c->ph.general;
+        ph.forces_variant = ph.forces_variant_c = plain ? 1 : default_forces(n, kWide16Max, kWide8Max);
+        // The forces-only pass has registers to spare in the plain shape, and so gains less by the others: us by
+        // 128 threads / 8 / 16 entries a round on boxes of 35,937 particles 17.2 / 16.5 / 16.6, 39,304 18.8 /
+        // 18.5 / 21.1, 54,872 19.2 / 19.3 / 26.0, 68,921 23.1 / 23.2 / 27.3, 74,088 23.0 / 24.2 / 27.3, 79,507
+        // 27.3 / 29.7 / 33.5; on dam breaks of 42,120 31.3 / 27.2 / 28.9, 68,958 30.9 / 28.3 / 27.6, 75,800
+        // 31.0 / 28.8 / 29.5
+        ph.forces_variant_f = plain ? 1 : default_forces(n, kWide16MaxF, kWide8MaxF);
+    }
+    c->ph.forces_variant_f = ph.forces_variant_f;  // (in no captured launch)
     if (ph.build_variant == c->ph.build_variant && ph.forces_variant == c->ph.forces_variant &&
         ph.forces_variant_c == c->ph.forces_variant_c && ph.fuse_predict == c->ph.fuse_predict)
         return;
@@ -816,6 +826,7 @@ int sph_create(const sph_params* p, sph_ctx** out) {
     ph.gamma_i = (int)gm;
     ph.build_variant = 0;
     ph.forces_variant = 1;
+    ph.forces_variant_f = 1;
     ph.forces_variant_c = 1;
     const uint32_t cap = p->max_particles;
     ph.stride = (uint32_t)align_up(cap, 32);
@@ -1139,7 +1150,7 @@ int sph_autotune(sph_ctx* c, void* stream, int* build_variant, int* forces_varia
             best_f = v;
         }
     }
-    c->ph.forces_variant = best_f;
+    c->ph.forces_variant = c->ph.forces_variant_f = best_f;
     // the corrector pass, on its own (its best shape differs from the predictor's): it runs
     // on the predicted state the tuned predictor leaves, and reads state n from and writes
     // n+1 to a copy in the sort's second buffer (free between builds); the per-scene |a|^2
@@ -1215,7 +1226,7 @@ int sph_set_forces_variants(sph_ctx* c, int forces_predict, int forces_correct) 
         forces_correct >= kForcesVariants)
         return SPH_ERR_ARG;
     if (forces_predict >= 0 || forces_correct >= 0) c->auto_forces = false;
-    if (forces_predict >= 0) c->ph.forces_variant = forces_predict;
+    if (forces_predict >= 0) c->ph.forces_variant = c->ph.forces_variant_f = forces_predict;
     if (forces_correct >= 0) c->ph.forces_variant_c = forces_correct;
     CK(cudaDeviceSynchronize());
     drop_graphs(c);  // captured launches carry the old shapes
@@ -1232,7 +1243,7 @@ int sph_set_variants(sph_ctx* c, int build_variant, int forces_variant) {
         if (c->auto_fuse) c->ph.fuse_predict = 0;  // the variant asked for
     }
     if (forces_variant >= 0) c->auto_forces = false;
-    if (forces_variant >= 0) c->ph.forces_variant = c->ph.forces_variant_c = forces_variant;
+    if (forces_variant >= 0) c->ph.forces_variant = c->ph.forces_variant_f = c->ph.forces_variant_c = forces_variant;
     CK(cudaDeviceSynchronize());
     drop_graphs(c);  // captured launches carry the old shapes
     return SPH_OK;

@@ -158,8 +158,8 @@ struct Phys {
     uint32_t n_scenes;
     int gamma_i;             // EOS exponent (integer)
     int build_variant;       // neighbour-build kernel variant (autotuned), see build_variant_name
-    int forces_variant;      // launch shape of the forces-only and predictor passes (autotuned), see
-                             //   forces_variant_name
+    int forces_variant;      // launch shape of the predictor pass (autotuned), see forces_variant_name
+    int forces_variant_f;    // of the forces-only pass: the predictor's, or a default of its own
     int forces_variant_c;    // launch shape of the corrector pass (autotuned on its own)
     int fuse_predict;        // the list build and the predictor pass as one kernel: its threads per block, or 0
     // model options (Table 1); general != 0 selects the kernels of forces_models.cu (density

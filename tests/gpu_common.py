@@ -175,7 +175,8 @@ def compare_neighbor_sets_of(scene, sample, counts, ids, band=1e-6):
 
 
 def launches(call, stream):
-    """Kernels that call() launches on `stream` (a torch stream), counted by capturing it."""
+    """Threads per block of the kernels that call() launches on `stream` (a torch stream), in order, by
+    capturing it."""
     import ctypes
     cu = ctypes.CDLL("libcuda.so.1")
     st, graph, n = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p(), ctypes.c_size_t()
@@ -183,5 +184,13 @@ def launches(call, stream):
     call()
     assert cu.cuStreamEndCapture(st, ctypes.byref(graph)) == 0
     assert cu.cuGraphGetNodes(graph, None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n)) == 0
+    out, kind, params = [], ctypes.c_int(), (ctypes.c_uint32 * 64)()
+    for k in nodes:
+        assert cu.cuGraphNodeGetType(ctypes.c_void_p(k), ctypes.byref(kind)) == 0
+        if kind.value == 0:  # a kernel: function pointer, three grid sizes, the block's x
+            assert cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(k), params) == 0
+            out.append(params[5])
     cu.cuGraphDestroy(graph)
-    return n.value
+    return out

@@ -9,7 +9,7 @@ import pytest
 
 import oracle
 from paper_2207_11328_gb300 import N_BUILD_VARIANTS, N_FORCES_VARIANTS, scenes
-from tests.gpu_common import compare_neighbor_sets, rel_check, require_gpu, sim_for
+from tests.gpu_common import compare_neighbor_sets, launches, rel_check, require_gpu, sim_for
 
 pytestmark = pytest.mark.gpu
 
@@ -252,3 +252,20 @@ def test_row_build_cuts_lists_in_shared_memory(max_neibs):
             assert (got[0][cut] > 0).all(1).any()  # both parts in a list that is cut
         for a, b in zip(got, ref):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n_axis,threads", [(20, 128), (33, 32), (34, 64), (41, 64), (42, 128)])
+def test_shape_of_accelerations_alone(n_axis, threads):
+    """sph_forces by particle count: 8 lanes, 16 and 8 entries a round, plain, on lines of its own; a shape that is
+    set holds for it too."""
+    import torch
+    s = scenes.periodic_box(n_per_axis=n_axis)
+    sim = sim_for(s)
+    stream = torch.cuda.Stream()
+    sim.forces()
+    torch.cuda.synchronize()
+    assert launches(lambda: sim.forces(stream=stream), stream) == [threads]
+    sim.set_variants(forces=2)
+    sim.forces()
+    torch.cuda.synchronize()
+    assert launches(lambda: sim.forces(stream=stream), stream) == [256]

@@ -131,7 +131,7 @@ def test_general_models_over_a_skin_list(visc, kernel, form, walls):
     rel_check(drho, d_ref, 1e-5, "density rate", mag[:, 1])
     stream = torch.cuda.Stream()
     torch.cuda.synchronize()
-    assert launches(lambda: sim.forces(stream=stream), stream) == 1
+    assert launches(lambda: sim.forces(stream=stream), stream) == [128]
     sim.step(6)
     pos, vel, delta = sim.download()
     st = sim.stats()
@@ -169,7 +169,7 @@ def test_forces_over_a_used_skin_list(visc, ddiff, walls):
     torch.cuda.synchronize()
     sim.forces()
     acc, drho = sim.download_forces()
-    assert launches(lambda: sim.forces(stream=stream), stream) == 1
+    assert launches(lambda: sim.forces(stream=stream), stream) == [128]
     pos, vel, delta = sim.download()
     # (the downloaded positions are the state's to half an FP32 ulp of the offset in the cell)
     a_ref, d_ref, mag = oracle.rhs(oracle.params(s), pos, vel, delta, s.mass, s.ptype, with_mag=True)
