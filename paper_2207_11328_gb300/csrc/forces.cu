@@ -630,9 +630,11 @@ __global__ void k_dt(const DtArgs a) { dt_body(a); }
 // just loaded are in cache; no separate pass re-reads the list.  The same
 // list and, pair for pair in the same order, the same sums and update as the
 // two kernels.  List rebuilt every step (no skin), default model.
-// The build waits on instruction issue and the pass on its gathers; mixed on an SM they overlap: 1.0M box
-// 942 -> 907 us a step, 20.1M dam break 15.35 -> 14.80 ms; not where many warps hold wall particles
-// (figures by size and block at default_variants, sph_api.cu).
+// What it saves is the list's second reading: 1.65M dam break, 239 MB of DRAM reads against the two kernels' 238 +
+// 422, the same 562M warp instructions (363M + 197M) at 67% issue (66 and 66%), 708 us against 451 + 265;
+// 20.1M, 13.0 GB of traffic against 11.6 + 7.4, 9.77 ms against 6.60 + 3.53.  Per step 1.0M box 942 -> 907 us,
+// 20.1M dam break 15.35 -> 14.80 ms, tanks of 2.0M 1301 -> 1320 (figures by size and block at
+// default_variants, sph_api.cu).
 // ---------------------------------------------------------------------
 template <int VISC, int kBlockT>
 __global__ void __launch_bounds__(kBlockT, 1024 / kBlockT) k_build_predict(const Buffers b, int cur, const Phys ph) {

@@ -646,22 +646,23 @@ inline unsigned grid_for(uint32_t n, int block) {
 
 // Default launch shapes for n particles, until sph_set_variants, sph_set_forces_variants or
 // sph_autotune choose.  Nine warps per 32 particles build the list while a thread per particle would
-// leave most of the GPU idle: us per step on periodic boxes, thread against warps, 98 / 71 at 4,096
-// particles, 114 / 94 at 32,768, 124 / 117 at 64,000, 166 / 174 at 125,000 (the line between).  Lists too
-// long for its shared memory take a thread per particle at any size: the warps fall back to one in
-// nine (us per step with max_neibs 320, thread against warps: 73 / 82 at 4,096, 87 / 145 at 32,768,
-// 106 / 259 at 64,000).  The
-// every-step passes of states that do not fill the GPU keep more of a particle's pairs in flight; the
+// leave most of the GPU idle: us per step, thread against warps, on periodic boxes of 4,096 particles
+// 65.2 / 36.0, 32,768 84.4 / 63.0, 64,000 103.7 / 93.8, 85,184 123.7 / 120.7, 97,336 130.0 / 132.2, 125,000
+// 148.8 / 154.2; on dam breaks of 42,120 115.8 / 89.0, 84,996 136.5 / 122.6, 119,736 139.6 / 134.6.  Lists
+// too long for its shared memory take a thread per particle at any size, which the warps fall back to (us per
+// step with max_neibs 320, thread against warps: 72 / 81 at 4,096, 88 / 100 at 32,768, 106 / 124 at 64,000).
+// The every-step passes of states that do not fill the GPU keep more of a particle's pairs in flight; the
 // figures on both sides of each line stand at launch_forces_v (forces.cu).
 // Large states, us per step: the thread build in blocks of 128 / of 256 / fused with the predictor in
-// blocks of 128 (the build waits on issue, the pass on its gathers: mixed on an SM they overlap, where
-// the particles are mostly fluid) / of 256:
+// blocks of 128 (its counters at k_build_predict, forces.cu) / of 256:
 //   dam break 572,120  397 /  395 /  407 /  406    box 1,030,301   954 /  942 /  920 /  907
 //           1,647,828 1082 / 1066 / 1068 / 1068        2,097,152  1963 / 1912 / 1854 / 1808
 //           2,817,201 1950 / 1900 / 1873 / 1856    tanks 2,030,211 1320 / 1301 / 1320 / 1339
 //           4,250,593 3010 / 2920 / 2865 / 2827          6,573,863 4083 / 4098 / 4073 / 4185
 //          20,139,024 15.52 / 15.35 / 14.82 / 14.80 ms
-// so blocks of 256 above half a million, and the fused kernel above 2.5 million, in the shape that lost
+// so blocks of 256 above half a million (below a million the two are within 2% either way: boxes of 262,144 287 /
+// 293, 512,000 522 / 530, 681,472 656 / 666, 884,736 822 / 833; dam breaks of 446,310 316 / 313, 534,210 367 /
+// 363, 702,842 466 / 464), and the fused kernel above 2.5 million, in the shape that lost
 // nowhere.  A build variant or fusion that was set or tuned stays.
 int default_forces(uint32_t n, uint32_t wide16_max, uint32_t wide8_max) {
     if (n <= kLanesMax) return 4;
